@@ -86,7 +86,7 @@ constexpr int kStageHalves = 2;       // half-slabs per ring stage (one barrier 
 
 struct Params {
   const int32_t* fill;     // [G] rows per expert group (final once the router completed)
-  int G, region, per_pair; // G = K + 1 groups of `region` rows; tile run capacity
+  int G, region, per_pair; // G = K + 1 groups of `region` rows; run table capacity
   const int32_t* row_tok;  // [G][region] pass-relative token of each row
   const float* row_w;      // [G][region] the row's pathway weight
   const uint64_t* shr;     // [T] shared block set of each token of the pass
@@ -105,7 +105,27 @@ struct Params {
 // pair tiles).
 __host__ __device__ constexpr uint32_t smem_bytes(int num_kb, int slots, int G, int per_pair) {
   return 1024u + (uint32_t)num_kb * kXBlock + 2u * kXBlock + (uint32_t)slots * kHalf + kStaging +
-         kBarBytes + (uint32_t)((2 * G + 1 + 3 * per_pair) * 4 + 15) / 16u * 16u;
+         kBarBytes + (uint32_t)((2 * G + 2 + 3 * per_pair) * 4 + 15) / 16u * 16u;
+}
+
+// How many parts the chunks of every tile are split into, so that the pairs
+// get equal runs of parts: a part's D is a partial sum over its chunks and
+// goes into the accumulator like a whole tile's. Whole tiles leave pairs
+// idle where their number is not close below a multiple of the pairs (one
+// 197-token image: 9 tiles on 76 pairs), but each run of parts costs its own
+// x gather and drain. In units of a quarter chunk: a chunk takes 1.77 us
+// (4) and each run of one tile's chunks ~4.8 us more (11) on d = 384, both
+// measured; S parts give a pair at most L = ceil(nt S / n_pairs) parts,
+// L nch / S chunks in at most (L + S - 2) / S + 1 runs. Called by one warp.
+__device__ __forceinline__ int pick_split(int nt, int nch, int n_pairs, int lane) {
+  const int S = lane + 1;
+  unsigned cost = 0xffffffffu;
+  if (S <= nch) {
+    const int L = (nt * S + n_pairs - 1) / n_pairs;
+    cost = 4u * (unsigned)((L * nch + S - 1) / S) + 11u * (unsigned)((L + S - 2) / S + 1);
+  }
+  const unsigned best = __reduce_min_sync(0xffffffffu, cost);
+  return __ffs(__ballot_sync(0xffffffffu, cost == best));  // the fewest parts of that cost
 }
 
 // cp.async.wait_group with a run-time count of groups allowed in flight.
@@ -211,11 +231,14 @@ ffn_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 49);
   static_assert(8 * 49 + 8 <= kBarBytes, "barrier region");
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  // tile table: first pair tile and size of every group, then (group,
-  // first row, real rows) of each pair tile of this pair's run
+  // tile table: first pair tile and size of every group, the length of this
+  // pair's run, then for each entry of the run (a range of one pair tile's
+  // chunks) its group and real rows (group << 16 | rows), its first row and
+  // its chunks (first << 16 | count)
   int32_t* first_s = reinterpret_cast<int32_t*>(reinterpret_cast<uint8_t*>(bars) + kBarBytes);
   int32_t* gcnt_s = first_s + p.G + 1;
-  int32_t* run_s = gcnt_s + p.G;
+  int32_t* n_run_s = gcnt_s + p.G;
+  int32_t* run_s = n_run_s + 1;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_rank();  // 0: the CTA that issues the MMAs
   const bool leader = rank == 0;
@@ -259,8 +282,12 @@ ffn_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     pair_tile_table<kPairRows>(p.fill, p.G, p.region, lane, first_s, gcnt_s);
     __syncwarp();
     const int nt = first_s[p.G];
-    const int tb = (int)(((long long)pair * nt) / n_pairs);
-    const int te = (int)(((long long)(pair + 1) * nt) / n_pairs);
+    // this pair's parts [ub, ue) of the nt S parts, tile by tile
+    const int S = pick_split(nt, nch, n_pairs, lane);
+    const int ub = (int)(((long long)pair * nt * S) / n_pairs);
+    const int ue = (int)(((long long)(pair + 1) * nt * S) / n_pairs);
+    const int tb = ub / S, te = ue > ub ? (ue - 1) / S + 1 : tb;
+    if (lane == 0) *n_run_s = te - tb;
     for (int k = tb + lane; k < te; k += 32) {
       int lo = 0, hi = p.G - 1;  // the last group whose first tile is <= k
       while (lo < hi) {
@@ -268,9 +295,10 @@ ffn_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
         if (first_s[mid] <= k) lo = mid; else hi = mid - 1;
       }
       const int i = k - first_s[lo];
-      run_s[k - tb] = lo;
+      const int c0 = nch * max(ub - k * S, 0) / S, c1 = nch * min(ue - k * S, S) / S;
+      run_s[k - tb] = (lo << 16) | min(kPairRows, gcnt_s[lo] - kPairRows * i);
       run_s[p.per_pair + k - tb] = lo * p.region + kPairRows * i;
-      run_s[2 * p.per_pair + k - tb] = min(kPairRows, gcnt_s[lo] - kPairRows * i);
+      run_s[2 * p.per_pair + k - tb] = (c0 << 16) | (c1 - c0);
     }
   }
   __syncwarp();
@@ -281,21 +309,30 @@ ffn_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   grid_dep_wait();
-  grid_dep_launch();
-  const int nt = first_s[p.G];
-  const int t_begin = (int)(((long long)pair * nt) / n_pairs);
-  const int n_run = (int)(((long long)(pair + 1) * nt) / n_pairs) - t_begin;
+  const int n_run = *n_run_s;
   const uint64_t full = p.B >= 64 ? ~0ull : ((1ull << p.B) - 1ull);
-  // Each pair walks the chunks of a tile from its own starting chunk, so
-  // that the pairs working on one expert at the same time read different
+  // Each pair walks the chunks of a run entry from its own starting chunk,
+  // so that the pairs working on one expert at the same time read different
   // weight slabs; D's sum over the chunks is the same in any order up to
   // the order of the fp32 additions.
-  const int rot = pair % nch;
-  auto chunk_of = [&](int c) { return c + rot < nch ? c + rot : c + rot - nch; };
-  // this CTA's rows of pair tile i: [r0 + 128 rank, + rows_mine)
+  struct Chunks {
+    int c0, n, rot;  // chunks [c0, c0 + n), starting at c0 + rot
+    __device__ __forceinline__ int of(int c) const {
+      return c0 + (c + rot < n ? c + rot : c + rot - n);
+    }
+  };
+  auto chunks = [&](int i) {
+    const int v = run_s[2 * p.per_pair + i];
+    Chunks k;
+    k.c0 = v >> 16;
+    k.n = v & 0xffff;
+    k.rot = pair % k.n;
+    return k;
+  };
+  // this CTA's rows of run entry i: [r0 + 128 rank, + rows_mine)
   auto my_rows = [&](int i, int& r0, int& rows) {
     r0 = run_s[p.per_pair + i] + kBM * (int)rank;
-    rows = min(kBM, max(0, run_s[2 * p.per_pair + i] - kBM * (int)rank));
+    rows = min(kBM, max(0, (run_s[i] & 0xffff) - kBM * (int)rank));
   };
   // y[tok] += w D over columns [c_begin, c_end) of tile i's D, for the 32
   // rows of TMEM lane quarter warp % 4 (thread = row). 16 columns per
@@ -421,7 +458,7 @@ ffn_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     // (hh, np = 2 P + rank); the 128-column remainder piece holds this
     // CTA's 64-row halves of slabs (0, npc - 1) and (1, npc - 1).
     auto load_down = [&](int e, int c) {
-      const long long v0 = (long long)(e * nch + chunk_of(c)) * 2 * npc;
+      const long long v0 = (long long)(e * nch + c) * 2 * npc;
 #pragma unroll
       for (int st = 0; st < kDownStages; ++st) {
         int hh, P;
@@ -435,15 +472,16 @@ ffn_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
       }
     };
     for (int i = 0; i < n_run && ok; ++i) {
-      const int e = run_s[i];
-      for (int c = 0; c < nch; ++c) {
-        const long long u0 = (long long)(e * nch + chunk_of(c)) * num_kb;
+      const int e = run_s[i] >> 16;
+      const Chunks ch = chunks(i);
+      for (int c = 0; c < ch.n; ++c) {
+        const long long u0 = (long long)(e * nch + ch.of(c)) * num_kb;
         for (int kb = 0; kb < num_kb; kb += kStageHalves)
           stage(&tmK, (u0 + kb) * 128 + 64 * (long long)rank,
                 (u0 + kb + 1) * 128 + 64 * (long long)rank);
-        if (c > 0) load_down(e, c - 1);
+        if (c > 0) load_down(e, ch.of(c - 1));
       }
-      load_down(e, nch - 1);
+      load_down(e, ch.of(ch.n - 1));
     }
     // the loads still in flight land before the pair exits (their bytes
     // complete on the leader's barriers)
@@ -465,7 +503,7 @@ ffn_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
       auto next = [&]() {
         if (++s == n_stages) { s = 0; ph ^= 1u; }
       };
-      auto up = [&](int i, int c) {
+      auto up = [&](int i, int c, int nc) {
         if (!wait_warp_cluster(uempty, (uc & 1u) ^ 1u, abort_flag, p.status, p.wait_limit))
           return false;
         tc_fence_after();
@@ -489,7 +527,7 @@ ffn_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                 umma_bf16_pair(tU, a + 2 * k, b + 2 * k, idesc, (kb | k) != 0 ? 1u : 0u);
             }
             umma_commit_pair(wempty(s), both);
-            if (c == nch - 1 && kb0 + kStageHalves == num_kb) umma_commit_pair(xempty, both);
+            if (c == nc - 1 && kb0 + kStageHalves == num_kb) umma_commit_pair(xempty, both);
           }
           __syncwarp();
           any = true;
@@ -501,7 +539,7 @@ ffn_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
         return true;
       };
       // down stages in the order of down_stage (the loader's order)
-      auto down = [&](int i, int c) {
+      auto down = [&](int i, int c, int nc) {
         if (c == 0) {
           if (!wait_warp_cluster(dempty, ((uint32_t)i & 1u) ^ 1u, abort_flag, p.status,
                                  p.wait_limit))
@@ -550,18 +588,19 @@ ffn_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
           next();
         }
         ++dc;
-        if (c == nch - 1) {
+        if (c == nc - 1) {
           if (elect_one()) umma_commit_pair(dfull, both);
           __syncwarp();
         }
         return true;
       };
       for (int i = 0; i < n_run && ok; ++i) {
-        for (int c = 0; c < nch && ok; ++c) {
-          ok = up(i, c);
-          if (ok && c > 0) ok = down(i, c - 1);
+        const int nc = chunks(i).n;
+        for (int c = 0; c < nc && ok; ++c) {
+          ok = up(i, c, nc);
+          if (ok && c > 0) ok = down(i, c - 1, nc);
         }
-        if (ok) ok = down(i, nch - 1);
+        if (ok) ok = down(i, nc - 1, nc);
       }
       // every MMA issued has completed before the pair releases TMEM
       if (any) {
@@ -592,7 +631,8 @@ ffn_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     uint32_t n = 0;  // chunks done by this CTA
     bool ok = true;
     for (int i = 0; i < n_run && ok; ++i) {
-      const int e = run_s[i];
+      const int e = run_s[i] >> 16;
+      const Chunks ch = chunks(i);
       int r0, rows;
       my_rows(i, r0, rows);
       // the blocks this row runs (none for a padding row)
@@ -601,10 +641,10 @@ ffn_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
         const uint64_t sh = p.shr[p.row_tok[r0 + r]];
         bm = e == 0 ? sh : (~sh & full);
       }
-      for (int c = 0; c < nch; ++c, ++n) {
+      for (int c = 0; c < ch.n; ++c, ++n) {
         if (!wait_warp(ufull, n & 1u, abort_flag, p.status, p.wait_limit)) { ok = false; break; }
         tc_fence_after();
-        const int blk = (chunk_of(c) * kChunk + hh * kBK) / p.M;
+        const int blk = (ch.of(c) * kChunk + hh * kBK) / p.M;
         // rows that do not run this block keep h = 0: GeLU is computed for
         // every row and masked (a per-row select compiles to a branch per
         // element, which serialises the GeLU chains: 4x slower)
@@ -735,7 +775,9 @@ int gemm_fused_setup(unif_moe_layer* L) {
     return UNIF_MOE_ERR_CUDA;
   }
   // one pair per two SMs, as many pairs as fit at once
-  int per_pair_guess = (int)((max_tiles + L->n_sm / 2 - 1) / (L->n_sm / 2));
+  // (run entries per pair: ceil(tiles / pairs) whole tiles, or up to two
+  // more ranges of chunks where pick_split splits the tiles)
+  int per_pair_guess = (int)((max_tiles + L->n_sm / 2 - 1) / (L->n_sm / 2)) + 2;
   uint32_t fixed = smem_bytes(num_kb, 0, G, per_pair_guess);
   int slots = fixed < kMaxSmem ? (int)((kMaxSmem - fixed) / kHalf) : 0;
   if (slots > kMaxSlots) slots = kMaxSlots;
@@ -772,7 +814,7 @@ int gemm_fused_setup(unif_moe_layer* L) {
   }
   if (clusters > L->n_sm / 2) clusters = L->n_sm / 2;
   L->ffn_pairs = clusters;
-  L->ffn_per_cta = (int)((max_tiles + clusters - 1) / clusters);  // pair tiles per pair
+  L->ffn_per_cta = (int)((max_tiles + clusters - 1) / clusters) + 2;  // run entries per pair
   if (L->ffn_per_cta > per_pair_guess) {  // fewer pairs than SMs / 2: a longer run table
     L->ffn_smem = smem_bytes(num_kb, slots, G, L->ffn_per_cta);
     while (L->ffn_smem > kMaxSmem && slots > 2 * kStageHalves) {
@@ -781,7 +823,7 @@ int gemm_fused_setup(unif_moe_layer* L) {
       L->ffn_smem = smem_bytes(num_kb, slots, G, L->ffn_per_cta);
     }
     if (L->ffn_smem > kMaxSmem) {
-      set_error("expert-tile FFN: a run of %d pair tiles per pair does not fit in shared memory",
+      set_error("expert-tile FFN: a run of %d entries per pair does not fit in shared memory",
                 L->ffn_per_cta);
       return UNIF_MOE_ERR_SHAPE;
     }
