@@ -34,3 +34,14 @@ def test_expert_tiles_split_over_chunks(T):
 def _run(wl):
     g = run_gpu(wl)
     return g, compare(wl, g)
+
+
+@pytest.mark.parametrize("shape", [
+    dict(d_model=72, d_ff=60, n_blocks=4),     # M = 15: unaligned weight columns; d % 32 = 8
+    dict(d_model=64, d_ff=280, n_blocks=4),    # M = 70: one whole 64-column item and 6 columns
+    dict(d_model=200, d_ff=512, n_blocks=2),   # several reduction steps, d % 64 = 8
+])
+@pytest.mark.parametrize("T", [1, 33, 500])
+def test_f32_items(shape, T):
+    wl = workloads.make_workload(small("f32", tokens=T, n_experts=3, **shape))
+    assert_parity(wl, *_run(wl))
