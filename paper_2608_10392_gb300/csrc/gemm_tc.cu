@@ -128,6 +128,11 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  // The tile list and the rows (up), h (down). The next kernel is not let in
+  // before this one ends: its CTAs on the SMs that finish first cost more
+  // than the prologue they hide (65,536 tokens, d = 1024: 3.81 ms with
+  // griddepcontrol.launch_dependents here, 3.71 without).
+  grid_dep_wait();
   const int n_items = p.n_tiles[0] * p.n_sub;
   // Bytes the TMA brings per stage (the up kernel gathers A with cp.async).
   const uint32_t stage_bytes = (MODE == 0 ? 0u : kStageA) + (uint32_t)p.bn * kBK * 2;
@@ -374,10 +379,12 @@ __global__ void timeout_probe_kernel(int* status, long long limit) {
 // TMEM lanes: a thread reads its token's Cp logits, takes the decisions of
 // Eqs. 18-27 and the warp counts its chunk's (expert, block) pairs.
 constexpr int kRtThreads = 192;   // warp 0 TMA, warp 1 TMEM + MMA, warps 2-5 decisions
-constexpr int kRtStages = 6;
+constexpr int kRtStages = 6;      // ring depth; kRtStages2 where two CTAs share an SM
+constexpr int kRtStages2 = 3;
 constexpr uint32_t kRtStageB = 160u * kBK * 2;  // up to 160 router columns
-constexpr size_t kRtSmem = 1024 + kRtStages * (kStageA + kRtStageB) + 256;
-constexpr int kRtRingBytes = kRtStages * (kStageA + kRtStageB);
+constexpr int router_ring_bytes(int stages) { return stages * (int)(kStageA + kRtStageB); }
+constexpr size_t router_smem_bytes(int stages) { return 1024 + router_ring_bytes(stages) + 256; }
+static_assert(2 * (router_smem_bytes(kRtStages2) + 1024) <= 228 * 1024, "two router CTAs per SM");
 
 // Bytes of the operand ring that the decision warps reuse once the MMAs are
 // done: logits [128][Cp + 1] and decision scratch [128][2K + 1] (fp32), lane
@@ -395,12 +402,13 @@ struct RouterTcParams {
   int d, Cp;
   int rows;      // tokens per CTA: 32, 64, 96 or 128 (the MMA always spans 128
                  // rows; the rows past the tile are never read back)
+  int stages;    // ring depth
   uint32_t tmem_cols;
   int* status;
   long long wait_limit;
 };
 
-__global__ void __launch_bounds__(kRtThreads, 1)
+__global__ void __launch_bounds__(kRtThreads, 2)
 router_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w,
                  RouterTcParams p) {
   extern __shared__ uint8_t smem_raw[];
@@ -408,23 +416,21 @@ router_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant
   // compiler keeps every access through it in the shared state space
   uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   const uint32_t sA = smem_u32(smem);
-  const uint32_t sB = sA + kRtStages * kStageA;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kRtStages * (kStageA + kRtStageB));
+  const int n_st = p.stages;
+  const uint32_t sB = sA + n_st * kStageA;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + n_st * (kStageA + kRtStageB));
   const uint32_t bar0 = smem_u32(bars);
   auto full_bar = [&](int s) { return bar0 + 8u * s; };
-  auto empty_bar = [&](int s) { return bar0 + 8u * (kRtStages + s); };
-  const uint32_t accf = bar0 + 8u * (2 * kRtStages);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kRtStages + 1);
+  auto empty_bar = [&](int s) { return bar0 + 8u * (n_st + s); };
+  const uint32_t accf = bar0 + 8u * (2 * n_st);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * n_st + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int R = p.rows;
   const int t0 = blockIdx.x * R;
   const int Cp = p.Cp, K = p.dec.K;
-  // the up projection may start its prologue on SMs this grid leaves free
-  grid_dep_launch();
-
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kRtStages; ++s) {
+    for (int s = 0; s < n_st; ++s) {
       mbar_init(full_bar(s), 1);
       mbar_init(empty_bar(s), 1);
     }
@@ -442,6 +448,9 @@ router_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   const int num_kb = p.d / kBK;
+  // x, and the records, counters and rows of the pass before, are this
+  // grid's from here
+  grid_dep_wait();
   if (warp == 0) {
     if (lane == 0) {
       int stage = 0;
@@ -452,7 +461,7 @@ router_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant
         mbar_expect_tx(full_bar(stage), bytes);
         tma_load_2d(sA + stage * kStageA, &tm_x, full_bar(stage), kb * kBK, t0);
         tma_load_2d(sB + stage * kRtStageB, &tm_w, full_bar(stage), kb * kBK, 0);
-        if (++stage == kRtStages) { stage = 0; phase ^= 1u; }
+        if (++stage == n_st) { stage = 0; phase ^= 1u; }
       }
     }
     __syncwarp();
@@ -474,7 +483,7 @@ router_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant
           umma_bf16(tmem_base, sw128_desc(a_base + k * 32), sw128_desc(b_base + k * 32), idesc,
                     (kb | k) != 0 ? 1u : 0u);
         umma_commit(empty_bar(stage));
-        if (++stage == kRtStages) { stage = 0; phase ^= 1u; }
+        if (++stage == n_st) { stage = 0; phase ^= 1u; }
       }
       if (ok) umma_commit(accf);
     }
@@ -671,18 +680,16 @@ cudaError_t launch_gemms_tc(unif_moe_layer* L, const void* x, int T, cudaEvent_t
   if (L->up_ws) {
     e = launch_up_ws(L, x, s);
   } else {
-    tc::grouped_gemm_kernel<0><<<L->n_sm, tc::kThreads, tc::Cfg<0>::kSmem, s>>>(L->tm_h,
-                                                                               L->tm_wup, p);
-    e = cudaGetLastError();
+    e = launch_dependent(tc::grouped_gemm_kernel<0>, dim3(L->n_sm), dim3(tc::kThreads),
+                         tc::Cfg<0>::kSmem, s, L->tm_h, L->tm_wup, p);
   }
   if (e != cudaSuccess) return e;
   if (mid) cudaEventRecord(mid, s);
   // down: N = d, reduction over the block's M channels
   if (L->down_ws) return launch_down_ws(L, s);
   p.n_sub = L->down_nsub; p.bn = L->down_bn; p.num_kb = L->M / tc::kBK;
-  tc::grouped_gemm_kernel<1><<<L->n_sm, tc::kThreads, tc::Cfg<1>::kSmem, s>>>(L->tm_h, L->tm_wdown,
-                                                                             p);
-  return cudaGetLastError();
+  return launch_dependent(tc::grouped_gemm_kernel<1>, dim3(L->n_sm), dim3(tc::kThreads),
+                          tc::Cfg<1>::kSmem, s, L->tm_h, L->tm_wdown, p);
 }
 
 // The streaming down-projection kernel on other operands: out[tok] +=
@@ -703,12 +710,12 @@ cudaError_t launch_down_streaming(unif_moe_layer* L, const CUtensorMap& tmA,
   p.status = L->ws.status;
   p.wait_limit = tc::g_wait_limit;
   p.n_sub = L->down_nsub; p.bn = L->down_bn; p.num_kb = L->M / tc::kBK;
-  tc::grouped_gemm_kernel<1><<<L->n_sm, tc::kThreads, tc::Cfg<1>::kSmem, s>>>(tmA, tmB, p);
-  return cudaGetLastError();
+  return launch_dependent(tc::grouped_gemm_kernel<1>, dim3(L->n_sm), dim3(tc::kThreads),
+                          tc::Cfg<1>::kSmem, s, tmA, tmB, p);
 }
 
 bool router_can_group(int Cp, int K, int G) {
-  return tc::router_overlay_bytes(Cp, K, G, true) <= tc::kRtRingBytes;
+  return tc::router_overlay_bytes(Cp, K, G, true) <= tc::router_ring_bytes(tc::kRtStages);
 }
 
 int router_tc_setup(unif_moe_layer* L) {
@@ -722,7 +729,7 @@ int router_tc_setup(unif_moe_layer* L) {
     return UNIF_MOE_ERR_CUDA;
   }
   if (cudaFuncSetAttribute(tc::router_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)tc::kRtSmem) != cudaSuccess) {
+                           (int)tc::router_smem_bytes(tc::kRtStages)) != cudaSuccess) {
     set_error("cudaFuncSetAttribute failed for the router kernel");
     return UNIF_MOE_ERR_CUDA;
   }
@@ -754,12 +761,20 @@ cudaError_t launch_router_tc(unif_moe_layer* L, const void* x, const uint8_t* ma
   p.d = L->d;
   p.Cp = L->router_cols_pad;
   p.rows = R;
+  // More CTAs than SMs: two share an SM, each with half the ring, so that one
+  // CTA's decisions run under the other's loads, where the decisions' scratch
+  // fits in the shorter ring (two passes of 32,768 tokens, d = 1024, K = 32:
+  // 62 us less per forward).
+  p.stages = (T + R - 1) / R > L->n_sm &&
+                     tc::router_overlay_bytes(p.Cp, L->K, p.fused == 2 ? L->K + 1 : L->G,
+                                              L->fused_group) <=
+                         tc::router_ring_bytes(tc::kRtStages2)
+                 ? tc::kRtStages2 : tc::kRtStages;
   p.tmem_cols = p.Cp <= 32 ? 32u : (p.Cp <= 64 ? 64u : (p.Cp <= 128 ? 128u : 256u));
   p.status = L->ws.status;
   p.wait_limit = tc::g_wait_limit;
-  tc::router_tc_kernel<<<(T + R - 1) / R, tc::kRtThreads, tc::kRtSmem, s>>>(
-      tm_x, L->tm_wr, p);
-  return cudaGetLastError();
+  return launch_dependent(tc::router_tc_kernel, dim3((T + R - 1) / R), dim3(tc::kRtThreads),
+                          tc::router_smem_bytes(p.stages), s, tm_x, L->tm_wr, p);
 }
 
 cudaError_t launch_timeout_probe(unif_moe_layer* L, int timeout_us, cudaStream_t s) {

@@ -20,13 +20,19 @@ constexpr int kChunkTokens = 256;
 constexpr int kStatusTimeout = 1;
 constexpr int kStatusBadIndex = 2;
 
-// Programmatic dependent launch. The kernels of a forward after the router
-// are launched with launch_dependent: each may start (prologue: barriers,
-// tensor memory, loads that need no result of the kernel before it) while
-// the kernel before it still runs, and waits in grid_dep_wait, which
-// returns once that kernel has completed and its writes are visible. A
-// kernel lets its dependent start with grid_dep_launch. In a kernel launched
-// without the attribute grid_dep_wait returns at once.
+// Programmatic dependent launch. The kernels of a forward are launched with
+// launch_dependent: each is set up while the kernel before it drains, and
+// waits in grid_dep_wait, which returns once that kernel has completed and
+// its writes are visible. In a kernel launched without the attribute
+// grid_dep_wait returns at once. A kernel may let its dependent's CTAs in
+// earlier with grid_dep_launch (those run their prologue, barriers and tensor
+// memory, beside it). Only the weight-stationary projections and the small
+// kernels of fp32 layers do: elsewhere the early CTAs took more from the
+// running kernel than their prologue saves (passes back to back; the router
+// letting the FFN in: 115.5 us per ViT-S forward against 114.0 without; the
+// combine letting the next router in: 692 us per ViT-B forward against 673;
+// the streaming projections: 3.81 ms per forward of 65,536 tokens of d = 1024
+// against 3.71).
 __device__ __forceinline__ void grid_dep_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }

@@ -119,6 +119,8 @@ router_kernel(const Tin* __restrict__ x, RouterArgs a) {
   uint32_t* cscr = reinterpret_cast<uint32_t*>(ss + kRouterTokens * (2 * K + 1));  // [2][128]
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int t0 = blockIdx.x * kRouterTokens;
+  grid_dep_launch();
+  grid_dep_wait();  // x, and the last pass's use of the records and counts
 
   // ---- z = x W for 64 tokens x Cp columns (Eqs. 17, 21) ----
   const int ty = tid >> 4, tx = tid & 15;  // tokens 4ty..4ty+3, columns tx + 16 j
@@ -208,6 +210,8 @@ chunk_scan_kernel(int G, int n_chunks, int32_t* __restrict__ chunk_cnt,
                   int32_t* __restrict__ grp_cnt) {
   const int lane = threadIdx.x & 31;
   const int g = blockIdx.x * 8 + (threadIdx.x >> 5);
+  grid_dep_launch();
+  grid_dep_wait();  // the router's counts
   if (g >= G) return;
   int32_t* col = chunk_cnt + (size_t)g * n_chunks;
   int carry = 0;
@@ -241,6 +245,8 @@ group_scatter_kernel(const uint64_t* __restrict__ shr_o, const uint64_t* __restr
   __shared__ int wsum[4];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int G = (K + 1) * B;
+  grid_dep_launch();
+  grid_dep_wait();  // the scanned counts (and the router's decisions)
   const int per = (G + 127) / 128;
   const int ga = min(G, tid * per), gb = min(G, ga + per);
   int mine = 0;
@@ -490,11 +496,15 @@ __global__ void tile_list_kernel(const int32_t* __restrict__ fill, int G, int re
                                  int32_t* __restrict__ n_tiles, int32_t* __restrict__ tile_group,
                                  int32_t* __restrict__ tile_row0, int32_t* __restrict__ tile_rows) {
   extern __shared__ int32_t tl_s[];  // [G + 1] first tiles, [G] sizes
-  if (threadIdx.x < 32) tile_table(fill, G, region, threadIdx.x, tl_s, tl_s + G + 1);
+  grid_dep_wait();  // the group sizes are final
+  for (int g = threadIdx.x; g < G; g += blockDim.x)
+    tl_s[G + 1 + g] = min(__ldcg(fill + g), region);
+  __syncthreads();
+  if (threadIdx.x < 32) tile_scan(G, threadIdx.x, tl_s, tl_s + G + 1);
   __syncthreads();
   const int nt = tl_s[G];
-  if (threadIdx.x == 0) n_tiles[0] = nt;
-  for (int k = threadIdx.x; k < nt; k += blockDim.x) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) n_tiles[0] = nt;
+  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < nt; k += gridDim.x * blockDim.x) {
     int g, r0, rows;
     tile_lookup(k, tl_s, tl_s + G + 1, G, region, g, r0, rows);
     tile_group[k] = g;
@@ -622,6 +632,8 @@ layernorm_rows(const T* __restrict__ x, T* __restrict__ out, const uint8_t* __re
                int d) {
   const int lane = threadIdx.x & 31;
   const int warps = gridDim.x * (blockDim.x >> 5);
+  grid_dep_launch();
+  grid_dep_wait();  // x, and the last pass's reads of out
   for (int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); r < n_rows; r += warps) {
     const size_t base = (size_t)r * d;
     const bool pad = mask != nullptr && mask[r] == 0;
@@ -695,6 +707,7 @@ combine_residual(float* __restrict__ y, const T* __restrict__ x, T* __restrict__
 }
 
 __global__ void copy_out_f32(float4* __restrict__ y, float4* __restrict__ out, size_t n4) {
+  grid_dep_wait();  // the down projection's sums are complete
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n4;
        i += (size_t)gridDim.x * blockDim.x) {
     out[i] = y[i];
@@ -782,9 +795,17 @@ cudaError_t launch_router(unif_moe_layer* L, const void* x, const uint8_t* mask,
   a.wr = L->wr;
   const void* xp = x;
   void* args[] = {const_cast<void**>(&xp), &a};
-  const int grid = (T + kRouterTokens - 1) / kRouterTokens;
-  return cudaLaunchKernel(router_entry(L), dim3(grid), dim3(kRouterThreads), args, router_smem(L),
-                          s);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((T + kRouterTokens - 1) / kRouterTokens);
+  cfg.blockDim = dim3(kRouterThreads);
+  cfg.dynamicSmemBytes = router_smem(L);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelExC(&cfg, router_entry(L), args);
 }
 
 static size_t scatter_smem(const unif_moe_layer* L) {
@@ -803,12 +824,14 @@ cudaError_t launch_permute(unif_moe_layer* L, int T, cudaStream_t s) {
   const int n_chunks = forward_chunks(T);
   Workspace& w = L->ws;
   const size_t r0 = (size_t)L->rec0;  // the records of this pass's first token
-  chunk_scan_kernel<<<(L->G + 7) / 8, 256, 0, s>>>(L->G, n_chunks, w.chunk_cnt, w.grp_cnt);
-  group_scatter_kernel<<<(n_chunks + 3) / 4, 128, scatter_smem(L), s>>>(
-      w.shr_mask + r0, w.exp_mask + r0, w.alpha + r0, w.s + r0 * L->K, T, L->K, L->B, n_chunks,
-      w.chunk_cnt, w.grp_cnt,
-      w.grp_off, w.n_tiles, w.tile_group, w.tile_row0, w.tile_rows, w.row_tok, w.row_w);
-  return cudaGetLastError();
+  cudaError_t e = launch_dependent(chunk_scan_kernel, dim3((L->G + 7) / 8), dim3(256), 0, s, L->G,
+                                   n_chunks, w.chunk_cnt, w.grp_cnt);
+  if (e != cudaSuccess) return e;
+  return launch_dependent(group_scatter_kernel, dim3((n_chunks + 3) / 4), dim3(128),
+                          scatter_smem(L), s, w.shr_mask + r0, w.exp_mask + r0, w.alpha + r0,
+                          w.s + r0 * L->K, T, L->K, L->B, n_chunks, w.chunk_cnt, w.grp_cnt,
+                          w.grp_off, w.n_tiles, w.tile_group, w.tile_row0, w.tile_rows, w.row_tok,
+                          w.row_w);
 }
 
 cudaError_t launch_sort_affinities(unif_moe_layer* L, int T, int32_t* q, float* p,
@@ -823,9 +846,12 @@ cudaError_t launch_tile_list(unif_moe_layer* L, cudaStream_t s) {
 
 cudaError_t launch_tile_list_from(unif_moe_layer* L, const int32_t* sizes, cudaStream_t s) {
   Workspace& w = L->ws;
-  tile_list_kernel<<<1, 256, sizeof(int32_t) * (2 * (size_t)L->G + 1), s>>>(
-      sizes, L->G, L->region_rows, w.n_tiles, w.tile_group, w.tile_row0, w.tile_rows);
-  return cudaGetLastError();
+  // every CTA scans the group sizes for itself and writes its share of the
+  // tiles; a thread per tile where 32 CTAs allow it
+  const int grid = (int)std::min<int64_t>(32, (L->max_tiles + 255) / 256);
+  return launch_dependent(tile_list_kernel, dim3(grid), dim3(256),
+                          sizeof(int32_t) * (2 * (size_t)L->G + 1), s, sizes, L->G,
+                          L->region_rows, w.n_tiles, w.tile_group, w.tile_row0, w.tile_rows);
 }
 
 cudaError_t launch_layernorm(unif_moe_layer* L, const void* x, void* out, const uint8_t* mask,
@@ -833,15 +859,15 @@ cudaError_t launch_layernorm(unif_moe_layer* L, const void* x, void* out, const 
                              cudaStream_t s) {
   const int grid = std::min((T + 7) / 8, L->n_sm * 8);
   if (L->dtype == UNIF_MOE_BF16)
-    layernorm_rows<__nv_bfloat16><<<grid, 256, 0, s>>>(
+    return launch_dependent(
+        layernorm_rows<__nv_bfloat16>, dim3(grid), dim3(256), 0, s,
         static_cast<const __nv_bfloat16*>(x), static_cast<__nv_bfloat16*>(out), mask,
         static_cast<const __nv_bfloat16*>(gamma), static_cast<const __nv_bfloat16*>(beta), eps, T,
         L->d);
-  else
-    layernorm_rows<float><<<grid, 256, 0, s>>>(
-        static_cast<const float*>(x), static_cast<float*>(out), mask,
-        static_cast<const float*>(gamma), static_cast<const float*>(beta), eps, T, L->d);
-  return cudaGetLastError();
+  return launch_dependent(layernorm_rows<float>, dim3(grid), dim3(256), 0, s,
+                          static_cast<const float*>(x), static_cast<float*>(out), mask,
+                          static_cast<const float*>(gamma), static_cast<const float*>(beta), eps,
+                          T, L->d);
 }
 
 cudaError_t launch_combine_residual(unif_moe_layer* L, const void* x, void* out,
@@ -868,16 +894,16 @@ cudaError_t launch_combine_residual(unif_moe_layer* L, const void* x, void* out,
 
 cudaError_t launch_combine(unif_moe_layer* L, void* out, int T, cudaStream_t s) {
   const size_t n4 = (size_t)T * L->d / 4;
-  const int grid = L->n_sm * 8;
+  const size_t grid = (size_t)L->n_sm * 8;
   if (L->dtype == UNIF_MOE_BF16)
-    return launch_dependent(cast_out_bf16, dim3(grid), dim3(256), 0, s,
+    return launch_dependent(cast_out_bf16, dim3(std::min(grid, (n4 + 255) / 256)), dim3(256), 0, s,
                             reinterpret_cast<float4*>(acc_cur(L)), static_cast<uint2*>(out),
                             n4, L->ws.grp_fill, L->ws.grp_cnt, L->fused_group ? L->G : 0,
                             L->region_rows, L->ffn_fused ? 0 : 1);
   else
-    copy_out_f32<<<grid, 256, 0, s>>>(reinterpret_cast<float4*>(L->ws.y32),
-                                      static_cast<float4*>(out), n4);
-  return cudaGetLastError();
+    return launch_dependent(copy_out_f32, dim3(std::min<size_t>(grid, (n4 + 255) / 256)),
+                            dim3(256), 0, s, reinterpret_cast<float4*>(L->ws.y32),
+                            static_cast<float4*>(out), n4);
 }
 
 }  // namespace unif

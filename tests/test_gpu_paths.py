@@ -36,6 +36,43 @@ def _run(wl):
     return g, compare(wl, g)
 
 
+@pytest.mark.parametrize("K,B", [(5, 4), (8, 12), (3, 16), (9, 8), (16, 12), (17, 16), (32, 8),
+                                 (33, 4), (6, 32)])
+@pytest.mark.parametrize("topk", [0, 2])
+def test_decision_instances(K, B, topk):
+    """Every instance of the decision step (K up to 8, 16 and 32, B up to 16,
+    the general one beyond) with counts that leave entries unused."""
+    wl = workloads.make_workload(small(n_experts=K, n_blocks=B, d_ff=64 * B if B != 12 else 768,
+                                       topk_fixed=topk))
+    assert_parity(wl, *_run(wl))
+
+
+@pytest.mark.parametrize("K", [8, 16, 32])
+def test_decisions_of_tokens_that_are_not_finite(K):
+    """A token holding NaN or infinity takes all K residual experts (no prefix
+    of its affinities reaches beta) and leaves every other token as it is."""
+    s = small(n_experts=K)
+    wl = workloads.make_workload(s)
+    clean = run_gpu(wl)
+    x = wl.x.clone()
+    x[7, 3] = float("nan")
+    x[100, 0] = float("inf")
+    bad = run_gpu(wl, layer=clean.layer, x=x)
+    keep = np.ones(s.tokens, bool)
+    keep[[7, 100]] = False
+    assert (bad.k[~keep] == K).all()
+    assert (bad.b[keep] == clean.b[keep]).all() and (bad.k[keep] == clean.k[keep]).all()
+    assert (bad.shr[keep] == clean.shr[keep]).all() and (bad.em[keep] == clean.em[keep]).all()
+
+
+@pytest.mark.parametrize("T", [152 * 128, 152 * 128 + 1, 40001])
+def test_router_two_ctas_per_sm(T):
+    """One wave of 128-token router CTAs, one token more, and a ragged count
+    of two waves: decisions, rows and outputs of every token."""
+    wl = workloads.make_workload(small(tokens=T, n_experts=2, d_ff=256))
+    assert_parity(wl, *_run(wl))
+
+
 @pytest.mark.parametrize("shape", [
     dict(d_model=72, d_ff=60, n_blocks=4),     # M = 15: unaligned weight columns; d % 32 = 8
     dict(d_model=64, d_ff=280, n_blocks=4),    # M = 70: one whole 64-column item and 6 columns
