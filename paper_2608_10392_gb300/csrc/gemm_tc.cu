@@ -651,8 +651,9 @@ int gemm_tc_setup(unif_moe_layer* L) {
     set_error("cudaFuncSetAttribute: %s", cudaGetErrorString(e));
     return UNIF_MOE_ERR_CUDA;
   }
-  const int rc = gemm_ws_setup(L);
-  L->tile_list = L->fused_group && !L->ffn_fused && !(L->up_ws && L->down_ws);
+  int rc = gemm_ws_setup(L);
+  if (rc == UNIF_MOE_OK) rc = gemm_pair_setup(L);
+  L->tile_list = L->fused_group && !L->ffn_fused && !((L->up_ws || L->up_pair) && L->down_ws);
   return rc;
 }
 
@@ -679,6 +680,8 @@ cudaError_t launch_gemms_tc(unif_moe_layer* L, const void* x, int T, cudaEvent_t
   cudaError_t e;
   if (L->up_ws) {
     e = launch_up_ws(L, x, s);
+  } else if (L->up_pair) {
+    e = launch_up_pair(L, x, s);
   } else {
     e = launch_dependent(tc::grouped_gemm_kernel<0>, dim3(L->n_sm), dim3(tc::kThreads),
                          tc::Cfg<0>::kSmem, s, L->tm_h, L->tm_wup, p);

@@ -170,6 +170,12 @@ struct unif_moe_layer {
   // number of output column slices run as separate work items
   int ws_down_bn = 0, ws_down_nsub = 0, down_slices = 1;
   CUtensorMap tm_wdown_ws;  // w_down slabs of ws_down_bn rows
+  // Up projection on CTA pairs (where the slice does not fit): boxes of half
+  // a sub-tile's key rows, ring depth, shared memory, pairs launched.
+  bool up_pair = false;
+  CUtensorMap tm_wup_half;
+  int pair_stages = 0, pairs = 0;
+  uint32_t pair_smem = 0;
   // Expert-tile FFN (both projections in one kernel, rows grouped by
   // expert): its weight maps (128 x 64 slabs), shared memory and ring depth.
   bool ffn_fused = false;
@@ -235,6 +241,8 @@ cudaError_t launch_timeout_probe(unif_moe_layer* L, int timeout_us, cudaStream_t
 int gemm_ws_setup(unif_moe_layer* L);  // picks the weight-stationary kernels where they fit
 cudaError_t launch_up_ws(unif_moe_layer* L, const void* x, cudaStream_t s);
 cudaError_t launch_down_ws(unif_moe_layer* L, cudaStream_t s);
+int gemm_pair_setup(unif_moe_layer* L);  // picks the pair up projection where the slice streams
+cudaError_t launch_up_pair(unif_moe_layer* L, const void* x, cudaStream_t s);
 bool ffn_fused_fits(int d, int H, int M);
 int gemm_fused_setup(unif_moe_layer* L);  // the expert-tile FFN's maps and shared memory
 cudaError_t launch_ffn_fused(unif_moe_layer* L, const void* x, cudaStream_t s);

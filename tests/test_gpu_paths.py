@@ -82,3 +82,17 @@ def test_router_two_ctas_per_sm(T):
 def test_f32_items(shape, T):
     wl = workloads.make_workload(small("f32", tokens=T, n_experts=3, **shape))
     assert_parity(wl, *_run(wl))
+
+
+@pytest.mark.parametrize("shape", [
+    dict(d_model=768, d_ff=1536, n_blocks=4),   # two 192-channel sub-tiles
+    dict(d_model=832, d_ff=768, n_blocks=4),    # 13 reduction steps, no multiple of the ring
+    dict(d_model=1024, d_ff=1024, n_blocks=2),  # 256-channel sub-tiles
+    dict(d_model=2048, d_ff=320, n_blocks=5),   # 64-channel blocks
+])
+@pytest.mark.parametrize("T", [1, 130, 257, 1000])
+def test_pair_up_projection(shape, T):
+    """Wide layers' up projection on CTA pairs: groups of less than one half
+    of a pair tile, of one row into the second half, of several tiles."""
+    wl = workloads.make_workload(small(tokens=T, n_experts=2, **shape))
+    assert_parity(wl, *_run(wl))
