@@ -63,6 +63,9 @@ struct Params {
   __nv_bfloat16* h;        // [128-row tiles of all groups][M]
   int n_sub, bn, num_kb;   // N sub-tiles of bn columns, 64-deep steps
   int B, M, H, d, stages;
+  // SCATTER: the place in h of every row (bundles.cu)
+  const uint64_t* shr;     // [T] shared block sets
+  const int32_t* dst;      // [T][K+1][B / kBundle]
   int* status;
   long long wait_limit;
 };
@@ -81,6 +84,9 @@ __device__ __forceinline__ void wait_settle(uint32_t bar, uint32_t parity, long 
     if (clock64() - t0 > limit) return;
 }
 
+// SCATTER: h rows go where dst names (the bundled down projection's units);
+// otherwise each group's rows fill its 128-row tiles in list order.
+template <bool SCATTER>
 __global__ void __launch_bounds__(kThreads, 1)
 pair_up_kernel(const __grid_constant__ CUtensorMap tmB, Params p) {
   extern __shared__ uint8_t smem_raw[];
@@ -299,12 +305,35 @@ pair_up_kernel(const __grid_constant__ CUtensorMap tmB, Params p) {
     uint8_t* stg = staging + (size_t)(warp - kFirstEpi) * 32 * kHStageRow;
     int acc = 0;
     uint32_t acc_ph = 0;
+    // SCATTER: this lane's row of the next item, its token one item ahead
+    // and its shared set and place loaded while the current one is stored
+    Item it = item_of(min(pair, max(n_items - 1, 0)));
+    auto token_of = [&](const Item& m) {
+      const int r = 32 * q + lane;
+      return r < m.rows ? p.row_tok[(size_t)m.g * p.region + m.pos + r] : 0;
+    };
+    int tok = 0;
+    if (SCATTER && pair < n_items) tok = token_of(it);
     for (int item = pair; item < n_items; item += n_pairs) {
-      const Item it = item_of(item);
-      // the group's rows fill its 128-row tiles of h in list order
-      __nv_bfloat16* hrow0 =
-          p.h + ((size_t)first128_s[it.g] * kBM + it.pos + q * 32) * p.M + it.ns * p.bn + c_begin;
       const int rows = it.rows - q * 32;  // real rows of this quarter
+      __nv_bfloat16* hrow0;
+      int drow = 0;  // SCATTER: this lane's h row
+      Item nx = it;
+      if (item + n_pairs < n_items) nx = item_of(item + n_pairs);
+      if (SCATTER) {
+        const int e = it.g / p.B, blk = it.g - e * p.B, bit = blk % kBundle;
+        const uint64_t sh = p.shr[tok];
+        const int d0 = p.dst[((size_t)tok * (p.G / p.B) + e) * (p.B / kBundle) + blk / kBundle];
+        // the blocks of the bundle before this one that the row runs
+        const uint32_t run = (uint32_t)((e == 0 ? sh : ~sh) >> (blk - bit));
+        drow = d0 + kBM * __popc(run & ((1u << bit) - 1u));
+        tok = token_of(nx);
+        hrow0 = p.h + it.ns * p.bn + c_begin;
+      } else {
+        hrow0 =
+            p.h + ((size_t)first128_s[it.g] * kBM + it.pos + q * 32) * p.M + it.ns * p.bn + c_begin;
+      }
+      it = nx;
       if (!wait_warp(accf_bar(acc), acc_ph, abort_flag, p.status, p.wait_limit)) break;
       tc_fence_after();
       const uint32_t t_row =
@@ -326,8 +355,9 @@ pair_up_kernel(const __grid_constant__ CUtensorMap tmB, Params p) {
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
             const int r = 8 * i + (lane >> 2), seg = lane & 3;
+            const int hr = SCATTER ? __shfl_sync(0xffffffffu, drow, r) : r;
             if (r < rows)
-              *reinterpret_cast<uint4*>(hrow0 + (size_t)r * p.M + c + seg * 8) =
+              *reinterpret_cast<uint4*>(hrow0 + (size_t)hr * p.M + c + seg * 8) =
                   *reinterpret_cast<const uint4*>(stg + r * kHStageRow + 16 * seg);
           }
           __syncwarp();
@@ -370,7 +400,9 @@ int gemm_pair_setup(unif_moe_layer* L) {
   L->pair_smem = smem_bytes(L->up_bn, stages, L->G);
   if (!encode_bf16_map(&L->tm_wup_half, L->w_up, L->d, (uint64_t)(L->K + 1) * L->H, tc::kBK,
                        (uint32_t)L->up_bn / 2, 128) ||
-      cudaFuncSetAttribute(pair_up_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+      cudaFuncSetAttribute(pair_up_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)L->pair_smem) != cudaSuccess ||
+      cudaFuncSetAttribute(pair_up_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)L->pair_smem) != cudaSuccess) {
     set_error("setting up the pair up-projection kernel failed");
     return UNIF_MOE_ERR_CUDA;
@@ -387,7 +419,7 @@ int gemm_pair_setup(unif_moe_layer* L) {
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   int clusters = 0;
-  if (cudaOccupancyMaxActiveClusters(&clusters, pair_up_kernel, &cfg) != cudaSuccess) {
+  if (cudaOccupancyMaxActiveClusters(&clusters, pair_up_kernel<true>, &cfg) != cudaSuccess) {
     set_error("cudaOccupancyMaxActiveClusters failed for the pair up-projection kernel");
     return UNIF_MOE_ERR_CUDA;
   }
@@ -397,7 +429,7 @@ int gemm_pair_setup(unif_moe_layer* L) {
   return UNIF_MOE_OK;
 }
 
-cudaError_t launch_up_pair(unif_moe_layer* L, const void* x, cudaStream_t s) {
+cudaError_t launch_up_pair(unif_moe_layer* L, const void* x, bool scatter, cudaStream_t s) {
   tc::pair::Params p;
   p.fill = L->ws.grp_fill;
   p.G = L->G;
@@ -408,6 +440,8 @@ cudaError_t launch_up_pair(unif_moe_layer* L, const void* x, cudaStream_t s) {
   p.n_sub = L->up_nsub; p.bn = L->up_bn; p.num_kb = L->d / tc::kBK;
   p.B = L->B; p.M = L->M; p.H = L->H; p.d = L->d;
   p.stages = L->pair_stages;
+  p.shr = L->ws.shr_mask + L->rec0;
+  p.dst = L->ws.bd_dst;
   p.status = L->ws.status;
   p.wait_limit = gemm_wait_limit();
   cudaLaunchConfig_t cfg = {};
@@ -424,7 +458,8 @@ cudaError_t launch_up_pair(unif_moe_layer* L, const void* x, cudaStream_t s) {
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, tc::pair::pair_up_kernel, L->tm_wup_half, p);
+  return scatter ? cudaLaunchKernelEx(&cfg, tc::pair::pair_up_kernel<true>, L->tm_wup_half, p)
+                 : cudaLaunchKernelEx(&cfg, tc::pair::pair_up_kernel<false>, L->tm_wup_half, p);
 }
 
 }  // namespace unif

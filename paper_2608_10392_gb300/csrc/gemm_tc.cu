@@ -78,11 +78,31 @@ struct Params {
   const __nv_bfloat16* x;  // up: tokens [T][d] (rows gathered with cp.async)
   __nv_bfloat16* h;  // up: [rows][M]
   float* y32;        // down: [T][d]
+  // bundled down projection: the tiles' first units of h, and the group
+  // counters to zero for the next pass
+  const int32_t* tile_unit;
+  int32_t* bd_fill;
+  int bd_groups;
   int* status;
   long long wait_limit;  // clock cycles before a wait gives up
 };
 
-// MODE 0 = up-projection (+GeLU), MODE 1 = down-projection (+weighted add).
+// The blocks of a bundle group's tile (bundles.cu): group = (e, bundle c,
+// pattern s), reduction over the |s| blocks of s in order.
+struct BundleTile {
+  int e, c, s;
+  __device__ __forceinline__ explicit BundleTile(int g, int B) {
+    constexpr int kP = (1 << kBundle) - 1;
+    s = g % kP + 1;
+    const int ec = g / kP, Q = B / kBundle;
+    e = ec / Q;
+    c = ec - e * Q;
+  }
+};
+
+// MODE 0 = up-projection (+GeLU), MODE 1 = down-projection (+weighted add),
+// MODE 2 = down-projection of rows bundled over several blocks (num_kb steps
+// per block).
 template <int MODE>
 __global__ void __launch_bounds__(kThreads, 1)
 grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
@@ -133,6 +153,8 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
   // than the prologue they hide (65,536 tokens, d = 1024: 3.81 ms with
   // griddepcontrol.launch_dependents here, 3.71 without).
   grid_dep_wait();
+  if (MODE == 2 && blockIdx.x == 0)  // the group sizes have been read
+    for (int g = threadIdx.x; g < p.bd_groups; g += kThreads) p.bd_fill[g] = 0;
   const int n_items = p.n_tiles[0] * p.n_sub;
   // Bytes the TMA brings per stage (the up kernel gathers A with cp.async).
   const uint32_t stage_bytes = (MODE == 0 ? 0u : kStageA) + (uint32_t)p.bn * kBK * 2;
@@ -193,6 +215,40 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
       }
       seq += p.num_kb;
     }
+  } else if (MODE == 2 && warp == 0) {
+    // ------------------- producer (bundled down): the blocks of the pattern --
+    int stage = 0;
+    uint32_t phase = 0;
+    bool ok = true;
+    int g_nxt = 0, u_nxt = 0;
+    if (blockIdx.x < n_items) {
+      g_nxt = p.tile_group[blockIdx.x / p.n_sub];
+      u_nxt = p.tile_unit[blockIdx.x / p.n_sub];
+    }
+    for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
+      const int ns = item % p.n_sub;
+      const BundleTile bt(g_nxt, p.B);
+      int row0 = u_nxt * kBM;
+      if (item + (int)gridDim.x < n_items) {
+        g_nxt = p.tile_group[(item + gridDim.x) / p.n_sub];
+        u_nxt = p.tile_unit[(item + gridDim.x) / p.n_sub];
+      }
+      const int brow = bt.e * p.d + ns * p.bn;  // w_down viewed [(K+1)d][H]
+      for (int bits = bt.s; bits != 0 && ok; bits &= bits - 1, row0 += kBM) {
+        const int col = (bt.c * kBundle + __ffs(bits) - 1) * p.M;
+        for (int kb = 0; kb < p.num_kb; ++kb) {
+          ok = wait_warp(empty_bar(stage), phase ^ 1u, abort_flag, p.status, p.wait_limit);
+          if (!ok) break;
+          if (lane == 0) {
+            mbar_expect_tx(full_bar(stage), stage_bytes);
+            tma_load_2d(sA + stage * kStageA, &tmA, full_bar(stage), kb * kBK, row0);
+            tma_load_2d(sB + stage * kStageB, &tmB, full_bar(stage), col + kb * kBK, brow);
+          }
+          __syncwarp();
+          if (++stage == kStages) { stage = 0; phase ^= 1u; }
+        }
+      }
+    }
   } else if (MODE == 1 && warp == 0) {
     // ------------------- producer (down): h tile and weight tile ------------
     int stage = 0;
@@ -226,11 +282,17 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
       int acc = 0;
       uint32_t acc_phase = 0;
       bool ok = true;
+      int g_nxt = MODE == 2 && blockIdx.x < n_items ? p.tile_group[blockIdx.x / p.n_sub] : 0;
       for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
+        int num_kb = p.num_kb;
+        if (MODE == 2) {
+          num_kb *= __popc(BundleTile(g_nxt, p.B).s);
+          if (item + (int)gridDim.x < n_items) g_nxt = p.tile_group[(item + gridDim.x) / p.n_sub];
+        }
         if (!wait_bounded(acce_bar(acc), acc_phase ^ 1u, abort_flag, p.status, p.wait_limit)) break;
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + (uint32_t)acc * kAccStride;
-        for (int kb = 0; kb < p.num_kb; ++kb) {
+        for (int kb = 0; kb < num_kb; ++kb) {
           if (!wait_bounded(full_bar(stage), phase, abort_flag, p.status, p.wait_limit)) {
             ok = false;
             break;
@@ -261,7 +323,7 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     int t_nxt = -1;
     float w_nxt = 0.f;
     // (row_w == nullptr: every row's weight is 1)
-    if (MODE == 1 && blockIdx.x < n_items &&
+    if (MODE >= 1 && blockIdx.x < n_items &&
         q * 32 + lane < p.tile_rows[blockIdx.x / p.n_sub]) {
       const int r = p.tile_row0[blockIdx.x / p.n_sub] + q * 32 + lane;
       t_nxt = p.row_tok[r];
@@ -272,7 +334,7 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
       const int row0 = tile * kBM;
       const int t_cur = t_nxt;
       const float w_cur = w_nxt;
-      if (MODE == 1 && item + (int)gridDim.x < n_items) {
+      if (MODE >= 1 && item + (int)gridDim.x < n_items) {
         const int nt = (item + gridDim.x) / p.n_sub;
         const int r = p.tile_row0[nt] + q * 32 + lane;
         const bool real = q * 32 + lane < p.tile_rows[nt];
@@ -637,7 +699,7 @@ int gemm_tc_setup(unif_moe_layer* L) {
   const uint64_t E = (uint64_t)L->K + 1;
   if (!tc::encode_2d(&L->tm_wup, L->w_up, L->d, E * L->H, tc::kBK, L->up_bn) ||
       !tc::encode_2d(&L->tm_wdown, L->w_down, L->H, E * L->d, tc::kBK, L->down_bn) ||
-      !tc::encode_2d(&L->tm_h, L->ws.hbuf, L->M, (uint64_t)L->max_rows, tc::kBK, tc::kBM)) {
+      !tc::encode_2d(&L->tm_h, L->ws.hbuf, L->M, (uint64_t)L->h_rows, tc::kBK, tc::kBM)) {
     set_error("cuTensorMapEncodeTiled failed for the weight or activation maps");
     return UNIF_MOE_ERR_CUDA;
   }
@@ -647,19 +709,29 @@ int gemm_tc_setup(unif_moe_layer* L) {
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(tc::grouped_gemm_kernel<1>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::Cfg<1>::kSmem);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(tc::grouped_gemm_kernel<2>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::Cfg<2>::kSmem);
   if (e != cudaSuccess) {
     set_error("cudaFuncSetAttribute: %s", cudaGetErrorString(e));
     return UNIF_MOE_ERR_CUDA;
   }
   int rc = gemm_ws_setup(L);
   if (rc == UNIF_MOE_OK) rc = gemm_pair_setup(L);
+  if (rc == UNIF_MOE_OK && L->bundles) {
+    if (!L->up_pair) {
+      L->bundles = false;  // (only the pair kernel places its rows)
+    } else if (bundles_setup(L) != cudaSuccess) {
+      set_error("setting up the bundle kernels failed");
+      rc = UNIF_MOE_ERR_CUDA;
+    }
+  }
   L->tile_list = L->fused_group && !L->ffn_fused && !((L->up_ws || L->up_pair) && L->down_ws);
   return rc;
 }
 
 cudaError_t launch_gemms_tc(unif_moe_layer* L, const void* x, int T, cudaEvent_t mid,
                             cudaStream_t s) {
-  (void)T;
   if (L->ffn_fused) {  // both projections in one kernel (the down stage takes no time)
     cudaError_t e = launch_ffn_fused(L, x, s);
     if (e == cudaSuccess && mid) e = cudaEventRecord(mid, s);
@@ -668,6 +740,7 @@ cudaError_t launch_gemms_tc(unif_moe_layer* L, const void* x, int T, cudaEvent_t
   tc::Params p;
   p.n_tiles = L->ws.n_tiles; p.tile_group = L->ws.tile_group; p.tile_row0 = L->ws.tile_row0;
   p.tile_rows = L->ws.tile_rows;
+  p.tile_unit = nullptr; p.bd_fill = nullptr; p.bd_groups = 0;
   p.row_tok = L->ws.row_tok; p.row_w = L->ws.row_w;
   p.B = L->B; p.M = L->M; p.H = L->H; p.d = L->d;
   p.x = static_cast<const __nv_bfloat16*>(x);
@@ -681,14 +754,25 @@ cudaError_t launch_gemms_tc(unif_moe_layer* L, const void* x, int T, cudaEvent_t
   if (L->up_ws) {
     e = launch_up_ws(L, x, s);
   } else if (L->up_pair) {
-    e = launch_up_pair(L, x, s);
+    e = launch_up_pair(L, x, bundles_apply(L, T), s);
   } else {
     e = launch_dependent(tc::grouped_gemm_kernel<0>, dim3(L->n_sm), dim3(tc::kThreads),
                          tc::Cfg<0>::kSmem, s, L->tm_h, L->tm_wup, p);
   }
   if (e != cudaSuccess) return e;
   if (mid) cudaEventRecord(mid, s);
-  // down: N = d, reduction over the block's M channels
+  // down: N = d, reduction over the block's M channels (bundled: over the
+  // blocks of each row's pattern)
+  if (bundles_apply(L, T)) {
+    const Workspace& w = L->ws;
+    p.n_tiles = w.bd_n_tiles; p.tile_group = w.bd_tile_group; p.tile_row0 = w.bd_tile_row0;
+    p.tile_rows = w.bd_tile_rows; p.tile_unit = w.bd_tile_unit;
+    p.row_tok = w.bd_row_tok; p.row_w = w.bd_row_w;
+    p.bd_fill = w.bd_fill; p.bd_groups = bundle_groups(L);
+    p.n_sub = L->down_nsub; p.bn = L->down_bn; p.num_kb = L->M / tc::kBK;
+    return launch_dependent(tc::grouped_gemm_kernel<2>, dim3(L->n_sm), dim3(tc::kThreads),
+                            tc::Cfg<2>::kSmem, s, L->tm_h, L->tm_wdown, p);
+  }
   if (L->down_ws) return launch_down_ws(L, s);
   p.n_sub = L->down_nsub; p.bn = L->down_bn; p.num_kb = L->M / tc::kBK;
   return launch_dependent(tc::grouped_gemm_kernel<1>, dim3(L->n_sm), dim3(tc::kThreads),
@@ -705,6 +789,7 @@ cudaError_t launch_down_streaming(unif_moe_layer* L, const CUtensorMap& tmA,
   tc::Params p;
   p.n_tiles = L->ws.n_tiles; p.tile_group = L->ws.tile_group; p.tile_row0 = L->ws.tile_row0;
   p.tile_rows = L->ws.tile_rows;
+  p.tile_unit = nullptr; p.bd_fill = nullptr; p.bd_groups = 0;
   p.row_tok = L->ws.row_tok; p.row_w = row_w;
   p.B = L->B; p.M = L->M; p.H = L->H; p.d = L->d;
   p.x = nullptr;

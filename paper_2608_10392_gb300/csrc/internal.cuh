@@ -16,6 +16,8 @@ constexpr int kTileRows = 128;
 // Tokens per block in the router and in the permute kernels.
 constexpr int kRouterTokens = 64;
 constexpr int kChunkTokens = 256;
+// Blocks per bundle of the bundled down projection.
+constexpr int kBundle = 4;
 // Status-word bits written by kernels.
 constexpr int kStatusTimeout = 1;
 constexpr int kStatusBadIndex = 2;
@@ -86,6 +88,16 @@ struct Workspace {
   // Expert weights repacked into the expert-tile FFN's 16 KB operand slabs.
   void* wk_slabs = nullptr;      // K_e: [K+1][H/128][d/64] slabs
   void* wv_slabs = nullptr;      // V_e: [K+1][H/128][2][d/128] slabs
+  // Down-projection rows bundled over four blocks (bundles.cu), G2 groups.
+  int32_t* bd_fill = nullptr;       // [G2] rows per group, 0 between passes
+  int32_t* bd_row_tok = nullptr;    // [G2][region]
+  float* bd_row_w = nullptr;        // same layout
+  int32_t* bd_dst = nullptr;        // [pass_tokens][K+1][B/4] h row of the bundle's first block
+  int32_t* bd_n_tiles = nullptr;    // [1]
+  int32_t* bd_tile_group = nullptr; // per 128-row tile: group, first list row, real rows,
+  int32_t* bd_tile_row0 = nullptr;  // first 128-row unit of h
+  int32_t* bd_tile_rows = nullptr;
+  int32_t* bd_tile_unit = nullptr;
   // Host-buffer forward staging.
   void* xn = nullptr;             // [max_tokens][d] LN(x) of a norm-first sublayer
   // Staging buffers of the host-buffer forwards, two slots (the pipelined
@@ -175,6 +187,8 @@ struct unif_moe_layer {
   bool up_pair = false;
   CUtensorMap tm_wup_half;
   int pair_stages = 0, pairs = 0;
+  bool bundles = false;  // the bundled down projection's workspace is allocated
+  int64_t h_rows = 0;    // rows of hbuf
   uint32_t pair_smem = 0;
   // Expert-tile FFN (both projections in one kernel, rows grouped by
   // expert): its weight maps (128 x 64 slabs), shared memory and ring depth.
@@ -242,7 +256,15 @@ int gemm_ws_setup(unif_moe_layer* L);  // picks the weight-stationary kernels wh
 cudaError_t launch_up_ws(unif_moe_layer* L, const void* x, cudaStream_t s);
 cudaError_t launch_down_ws(unif_moe_layer* L, cudaStream_t s);
 int gemm_pair_setup(unif_moe_layer* L);  // picks the pair up projection where the slice streams
-cudaError_t launch_up_pair(unif_moe_layer* L, const void* x, cudaStream_t s);
+cudaError_t launch_up_pair(unif_moe_layer* L, const void* x, bool scatter, cudaStream_t s);
+// Bundled down projection (bundles.cu).
+bool bundles_fit(const unif_moe_layer* L);
+int bundle_groups(const unif_moe_layer* L);
+int64_t bundle_h_rows(const unif_moe_layer* L);
+int64_t bundle_max_tiles(const unif_moe_layer* L);
+bool bundles_apply(const unif_moe_layer* L, int T);  // a pass of T tokens uses them
+cudaError_t bundles_setup(const unif_moe_layer* L);
+cudaError_t launch_bundles(unif_moe_layer* L, int T, cudaStream_t s);
 bool ffn_fused_fits(int d, int H, int M);
 int gemm_fused_setup(unif_moe_layer* L);  // the expert-tile FFN's maps and shared memory
 cudaError_t launch_ffn_fused(unif_moe_layer* L, const void* x, cudaStream_t s);

@@ -76,7 +76,10 @@ void free_all(unif_moe_layer* L) {
                   L->ws.tile_rows, L->ws.w_upT, L->ws.w_downT, L->ws.da, L->ws.hw,
                   L->ws.dwt, L->ws.dz, L->ws.wrT, L->ws.gram, L->ws.diag_sets,
                   L->ws.diag_counts, L->ws.diag_pair, L->ws.diag_wts, L->ws.diag_q,
-                  L->ws.diag_E, L->ws.diag_ES, L->ws.wk_slabs, L->ws.wv_slabs, L->ws.y32_b};
+                  L->ws.diag_E, L->ws.diag_ES, L->ws.wk_slabs, L->ws.wv_slabs, L->ws.y32_b,
+                  L->ws.bd_fill, L->ws.bd_row_tok, L->ws.bd_row_w, L->ws.bd_dst,
+                  L->ws.bd_n_tiles, L->ws.bd_tile_group, L->ws.bd_tile_row0,
+                  L->ws.bd_tile_rows, L->ws.bd_tile_unit};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   for (int i = 0; i < 2; ++i) {
@@ -248,8 +251,23 @@ int unif_moe_create_ex(unif_moe_t* out, int d_model, int d_ff, int n_experts, in
   const size_t row_cap = L->fused_group ? (size_t)L->G * L->region_rows : (size_t)L->max_rows;
   ALLOC(w.row_tok, row_cap); ALLOC(w.row_w, row_cap);
   if (L->fused_group) ALLOC(w.grp_fill, (size_t)L->G);
+  // wide layers' passes of many tokens: the down projection's rows bundled
+  // over four blocks, h in their layout
+  L->bundles = true;
+  L->bundles = dtype == UNIF_MOE_BF16 && unif::bundles_fit(L) &&
+               unif::bundles_apply(L, L->pass_tokens);
+  L->h_rows = L->max_rows;
+  if (L->bundles) {
+    const size_t G2 = (size_t)unif::bundle_groups(L), nt = (size_t)unif::bundle_max_tiles(L);
+    L->h_rows = std::max(L->h_rows, unif::bundle_h_rows(L));
+    ALLOC(w.bd_fill, G2);
+    ALLOC(w.bd_row_tok, G2 * L->region_rows); ALLOC(w.bd_row_w, G2 * L->region_rows);
+    ALLOC(w.bd_dst, (size_t)L->pass_tokens * E * (n_blocks / unif::kBundle));
+    ALLOC(w.bd_n_tiles, 1); ALLOC(w.bd_tile_group, nt); ALLOC(w.bd_tile_row0, nt);
+    ALLOC(w.bd_tile_rows, nt); ALLOC(w.bd_tile_unit, nt);
+  }
   void* hb = nullptr;
-  if (rc == UNIF_MOE_OK) rc = dalloc(reinterpret_cast<char**>(&hb), es * (size_t)L->max_rows * M);
+  if (rc == UNIF_MOE_OK) rc = dalloc(reinterpret_cast<char**>(&hb), es * (size_t)L->h_rows * M);
   w.hbuf = hb;
   ALLOC(w.y32, (size_t)L->pass_tokens * d_model);
   if (L->ffn_fused) ALLOC(w.y32_b, (size_t)L->pass_tokens * d_model);
@@ -307,6 +325,13 @@ int unif_moe_create_ex(unif_moe_t* out, int d_model, int d_ff, int n_experts, in
                                 cudaSuccess ||
                             (w.y32_b && cudaMemset(w.y32_b, 0, sizeof(float) * L->pass_tokens *
                                                                    d_model) != cudaSuccess) ||
+                            // (a row whose place was never written goes to h row 0)
+                            (L->bundles &&
+                             (cudaMemset(w.bd_fill, 0, sizeof(int32_t) * unif::bundle_groups(L)) !=
+                                  cudaSuccess ||
+                              cudaMemset(w.bd_dst, 0, sizeof(int32_t) * L->pass_tokens * E *
+                                                          (n_blocks / unif::kBundle)) !=
+                                  cudaSuccess)) ||
                             (L->fused_group &&
                              (cudaMemset(w.grp_fill, 0, sizeof(int32_t) * L->G) != cudaSuccess ||
                               // rows hold token indices from the start, also any row a
@@ -410,6 +435,8 @@ static int forward_pass(unif_moe_t L, const void* x, void* out, int T, int t0,
     if (L->ws.y32_b)
       CK(cudaMemsetAsync(L->ws.y32_b, 0, sizeof(float) * (size_t)L->pass_tokens * L->d, s));
     if (L->fused_group) CK(cudaMemsetAsync(L->ws.grp_fill, 0, sizeof(int32_t) * L->G, s));
+    if (L->bundles)
+      CK(cudaMemsetAsync(L->ws.bd_fill, 0, sizeof(int32_t) * unif::bundle_groups(L), s));
   }
   L->y_dirty = true;
   L->rec0 = t0;
@@ -421,6 +448,7 @@ static int forward_pass(unif_moe_t L, const void* x, void* out, int T, int t0,
   }
   if (ev[1]) CK(cudaEventRecord(ev[1], s));
   if (!L->fused_group) CK(unif::launch_permute(L, T, s));
+  else if (unif::bundles_apply(L, T)) CK(unif::launch_bundles(L, T, s));
   else if (L->tile_list) CK(unif::launch_tile_list(L, s));
   if (ev[2]) CK(cudaEventRecord(ev[2], s));
   if (L->dtype == UNIF_MOE_BF16) {
@@ -878,6 +906,8 @@ int unif_moe_pass_tokens(unif_moe_t L) { return L ? L->pass_tokens : -1; }
 int unif_moe_kernels_per_forward(unif_moe_t L) {
   if (!L) return -1;
   if (L->ffn_fused) return 3;  // router, expert-tile FFN, combine
+  // router, bundle rows, bundle tiles, up, down, combine
+  if (unif::bundles_apply(L, L->pass_tokens)) return 6;
   return L->fused_group ? (L->tile_list ? 5 : 4) : 6;
 }
 

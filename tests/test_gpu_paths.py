@@ -96,3 +96,27 @@ def test_pair_up_projection(shape, T):
     of a pair tile, of one row into the second half, of several tiles."""
     wl = workloads.make_workload(small(tokens=T, n_experts=2, **shape))
     assert_parity(wl, *_run(wl))
+
+
+@pytest.mark.parametrize("shape", [
+    dict(d_model=832, d_ff=768, n_blocks=4, n_experts=2),    # one bundle
+    dict(d_model=1024, d_ff=1024, n_blocks=8, n_experts=1),  # two
+    dict(d_model=768, d_ff=3072, n_blocks=16, n_experts=2),  # four
+])
+@pytest.mark.parametrize("kw", [dict(), dict(topk_fixed=1), dict(prefix_blocks=1),
+                                dict(alpha_fixed=0.0), dict(seq_len=100, min_len=1)])
+def test_bundled_down_projection(shape, kw):
+    """Passes of enough tokens for the down projection's rows to be bundled
+    over four blocks: every pattern, only full ones (alpha = 0: no shared
+    block, all blocks of every residual expert), prefixes, padding."""
+    wl = workloads.make_workload(small(tokens=5111, **shape, **kw))
+    g, rep = _run(wl)
+    assert g.layer.kernels_per_forward() == 6
+    assert_parity(wl, g, rep)
+    # a smaller forward on the same handle takes the unbundled kernels, and
+    # the next large one the bundled ones again
+    few = run_gpu(wl, layer=g.layer, x=wl.x[:200].clone(),
+                  mask=None if wl.mask is None else wl.mask[:200])
+    assert (few.b == g.b[:200]).all() and (few.k == g.k[:200]).all()
+    again = run_gpu(wl, layer=g.layer)
+    assert np.abs(again.y - g.y).max() <= 2e-2 * np.abs(g.y).max()
