@@ -19,12 +19,14 @@
 // diversity-loss) adds lambda_div dL_div/dW*.
 //
 // Kernels (in stream order): tile list from the forward's group sizes,
-// bwd_hidden_kernel (two tcgen05 accumulators: x K and dy V^T over the same
-// gathered rows), the down kernel for dL/dx, bwd_wgrad_kernel (tcgen05 with
+// bwd_hidden_kernel (CTA pairs, two tcgen05 accumulators: x K and dy V^T over
+// the same gathered rows), the down kernel for dL/dx, bwd_wgrad_kernel (tcgen05 with
 // MN-major operands: the token rows are the reduction dimension), the
 // router-gradient kernels and the Gram kernel. Every wait on an mbarrier is
 // bounded; a wait that runs out records kStatusTimeout and the CTA unwinds.
 #include <stdio.h>
+
+#include <algorithm>
 
 #include "decide.cuh"
 #include "internal.cuh"
@@ -34,12 +36,26 @@ namespace unif {
 namespace tc {
 namespace bwd {
 
-// GeLU (exact erf form, Sec. II-A) and its derivative Phi(a) + a phi(a),
-// from one evaluation of Phi.
+// GeLU (exact erf form, Sec. II-A) and its derivative Phi(a) + a phi(a). Phi
+// from the erf approximation 7.1.26 of Abramowitz and Stegun (Handbook of
+// Mathematical Functions, 1964): erfc(z) = (b1 t + ... + b5 t^5) exp(-z^2),
+// t = 1 / (1 + p z), z >= 0, error at most 1.5e-7; with z = |a| / sqrt 2 its
+// exponential is the one that phi needs, so one value takes about 17
+// instructions in place of the 45 that erff and the exponential took. (The
+// same in packed fp32x2 arithmetic ran 8 us slower per ViT-S backward.)
 __device__ __forceinline__ void gelu_and_grad(float a, float& g, float& dg) {
-  const float cdf = 0.5f * (1.0f + erff(a * 0.70710678118654752f));
+  float e, t;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(a * a * -0.72134752044448170f));  // exp(-a^2/2)
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t) : "f"(fmaf(fabsf(a), 0.23164188819f, 1.0f)));
+  // -erfc / 2: the coefficients halved and negated
+  float q = fmaf(-0.5307027145f, t, 0.7265760135f);
+  q = fmaf(q, t, -0.7107068705f);
+  q = fmaf(q, t, 0.142248368f);
+  q = fmaf(q, t, -0.127414796f);
+  // Phi = 1/2 + sign(a) (1/2 - erfc / 2)
+  const float cdf = 0.5f + copysignf(fmaf(q * t, e, 0.5f), a);
   g = a * cdf;
-  dg = cdf + a * 0.39894228040143268f * __expf(-0.5f * a * a);
+  dg = fmaf(a * 0.39894228040143268f, e, cdf);
 }
 
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
@@ -70,226 +86,340 @@ constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kAcc2 = 256;   // TMEM column of the second accumulator
 
 // ---------------------------------------------------------------------------
-// bwd_hidden_kernel: per (tile, N sub-tile) item, over the forward's tile
-// list, acc_a = X[rows] K_e[cols]^T and acc_g = DY[rows] V_e^T[cols]^T (both
-// reductions over d), then the epilogue of the header comment.
-// Roles: warps 0-3 fill a 4-deep ring of single-operand stages (even
-// stages: 128 gathered x rows and the key tile; odd stages: dy rows and the
-// value tile, so that each 64-deep k-block takes one stage of each; warp s
-// owns stage s and its lane 0 brings the stage's weight tile by TMA); warp 4
-// allocates TMEM and issues the MMAs; warps 5-12 run the epilogue (warp w
-// reads TMEM lane quarter w % 4, one half of the columns).
+// bwd_hidden_kernel: per 256-row tile of a group and N sub-tile, on a pair of
+// CTAs (tcgen05 cta_group::2, M = 256, 128 rows each), acc_a = X[rows]
+// K_e[cols]^T and acc_g = DY[rows] V_e^T[cols]^T (both reductions over d),
+// then the epilogue of the header comment.
+// Roles (each CTA, 18 warps): warps 0-7 gather this CTA's 128 rows of a
+// step, a warp per ring stage (even steps x rows, odd steps dy rows: each
+// 64-deep k-block takes one of each); warp 8 brings this CTA's half of the
+// step's weight tile (keys, values) by TMA; warp 9 allocates TMEM and, in
+// the even CTA, issues the MMAs; warps 10-17 run the epilogue (warp w: TMEM
+// lane quarter w % 4, one half of the columns), which leaves 32 x 32 pieces
+// of both outputs in shared memory for TMA stores (64-byte swizzle). The two
+// accumulators take 2 bn <= 512 TMEM columns, so a tile's MMAs wait for the
+// epilogue of the one before; the ring holds the next tile's first steps by
+// then. (16 epilogue warps of half the columns ran no faster.)
+// Measured (ViT-S, 12,608 tokens; one CTA per tile, four gather warps, erff,
+// a 32-byte row piece per thread's store before): 138 -> HID_S us; BERT-base
+// (2,300 tokens) 102 -> HID_B.
 // ---------------------------------------------------------------------------
 struct HiddenParams {
-  const int32_t* n_tiles;
-  const int32_t* tile_group;
-  const int32_t* tile_row0;
-  const int32_t* tile_rows;
-  const int32_t* row_tok;
+  const int32_t* counts;   // [G] group sizes (the forward's)
+  int G, region;
+  const int32_t* row_tok;  // [G][region]
   const float* row_w;
   const __nv_bfloat16* x;
   const __nv_bfloat16* dy;
-  __nv_bfloat16* da;   // [rows][M]
-  __nv_bfloat16* hw;   // [rows][M]
   float* dwt;          // [T][K+1]
-  int n_sub, bn, num_kb, B, M, H, d, K1;
+  int n_sub, bn, num_kb, B, M, H, d, K1, stages;
   int* status;
   long long wait_limit;
 };
 
-constexpr int kHStages = 4;
+constexpr int kHGather = 8;     // at most one warp per ring stage
+constexpr int kHLoader = 8, kHMma = 9, kHFirstEpi = 10, kHEpiWarps = 8;
+constexpr int kHThreads = 32 * (kHFirstEpi + kHEpiWarps);  // 576
+constexpr int kHMinStages = 4;
+constexpr int kHPairRows = 256;
+constexpr uint32_t kHPiece = 32u * 64u;  // 32 rows x 32 bf16
+constexpr uint32_t kHStaging = kHEpiWarps * 2u * kHPiece;
+constexpr uint32_t kHBarBytes = 256;
 
 __host__ __device__ constexpr uint32_t hidden_stage_bytes(int bn) {
-  return kStageA + (uint32_t)bn * kBK * 2u;
+  return kStageA + (uint32_t)bn * 64u;
+}
+__host__ __device__ constexpr uint32_t hidden_smem_bytes(int bn, int stages, int G) {
+  return 1024u + (uint32_t)stages * hidden_stage_bytes(bn) + kHStaging + kHBarBytes +
+         (uint32_t)((3 * G + 2) * 4 + 15) / 16u * 16u;
 }
 
-__global__ void __launch_bounds__(kThreads, 1)
+// A bounded wait that ignores the abort flag (copies and MMAs in flight land
+// before the pair releases its TMEM).
+__device__ __forceinline__ void wait_settle(uint32_t bar, uint32_t parity, long long limit) {
+  const long long t0 = clock64();
+  while (!mbar_try_wait(bar, parity))
+    if (clock64() - t0 > limit) return;
+}
+
+__global__ void __launch_bounds__(kHThreads, 1)
 bwd_hidden_kernel(const __grid_constant__ CUtensorMap tm_wk, const __grid_constant__ CUtensorMap tm_wv,
+                  const __grid_constant__ CUtensorMap tm_da, const __grid_constant__ CUtensorMap tm_hw,
                   HiddenParams p) {
   extern __shared__ uint8_t smem_raw[];
+  // 1024-byte aligned base, the same offset in both CTAs of the pair
   uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+  const int n_st = p.stages;
   const uint32_t stage_bytes = hidden_stage_bytes(p.bn);
-  const uint32_t wtile = (uint32_t)p.bn * kBK * 2u;
   const uint32_t s0 = smem_u32(smem);
-  // stage s: [128 rows x 64 (16 KB)][weight tile bn x 64]
-  auto sa = [&](int s) { return s0 + s * stage_bytes; };
-  auto sw = [&](int s) { return s0 + s * stage_bytes + kStageA; };
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kHStages * stage_bytes);
+  // stage s: [128 rows x 64][bn / 2 weight rows x 64]
+  auto sa = [&](int s) { return s0 + (uint32_t)s * stage_bytes; };
+  auto sw = [&](int s) { return s0 + (uint32_t)s * stage_bytes + kStageA; };
+  uint8_t* staging = smem + (size_t)n_st * stage_bytes;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(staging + kHStaging);
   const uint32_t bar0 = smem_u32(bars);
   auto full_bar = [&](int s) { return bar0 + 8u * s; };
-  auto empty_bar = [&](int s) { return bar0 + 8u * (kHStages + s); };
-  const uint32_t accf = bar0 + 8u * (2 * kHStages);
-  const uint32_t acce = bar0 + 8u * (2 * kHStages + 1);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kHStages + 2);
+  auto empty_bar = [&](int s) { return bar0 + 8u * (kHGather + s); };
+  const uint32_t accf = bar0 + 8u * (2 * kHGather);
+  const uint32_t acce = bar0 + 8u * (2 * kHGather + 1);
+  const uint32_t mma_done = bar0 + 8u * (2 * kHGather + 2);
+  const uint32_t fin = bar0 + 8u * (2 * kHGather + 3);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kHGather + 4);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  static_assert(8 * (2 * kHGather + 5) <= kHBarBytes, "barrier region");
+  // first 256-row pair tile and first 128-row tile of every group, its size
+  int32_t* first_s = reinterpret_cast<int32_t*>(reinterpret_cast<uint8_t*>(bars) + kHBarBytes);
+  int32_t* first128_s = first_s + p.G + 1;
+  int32_t* cnt_s = first128_s + p.G + 1;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t rank = cluster_rank();
+  const bool leader = rank == 0;
+  auto arrive_leader = [&](uint32_t bar) {
+    if (leader) mbar_arrive(bar);
+    else mbar_arrive_cluster(mapa_shared(bar, 0));
+  };
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kHStages; ++s) {
-      mbar_init(full_bar(s), 1);
+    for (int s = 0; s < kHGather; ++s) {
+      mbar_init(full_bar(s), 3);  // an owner warp of each CTA, the leader's loader
       mbar_init(empty_bar(s), 1);
     }
     mbar_init(accf, 1);
-    mbar_init(acce, kEpiWarps);
+    mbar_init(acce, 2 * kHEpiWarps);
+    mbar_init(mma_done, 1);
+    mbar_init(fin, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == kMmaWarp) {
-    tmem_alloc(smem_u32(tmem_slot), kTmemCols);
-    tmem_relinquish();
+  if (warp == kHMma) {
+    tmem_alloc_pair(smem_u32(tmem_slot), kTmemCols);
+    tmem_relinquish_pair();
+  }
+  for (int g = threadIdx.x; g < p.G; g += kHThreads) cnt_s[g] = min(p.counts[g], p.region);
+  __syncthreads();
+  if (warp == 0) {
+    tile_scan<kBM>(p.G, lane, first128_s, cnt_s);
+  } else if (warp == 1) {
+    tile_scan<kHPairRows>(p.G, lane, first_s, cnt_s);
   }
   __syncwarp();
   tc_fence_before();
   __syncthreads();
+  // both CTAs' barriers are initialised before either CTA signals the other
+  cluster_sync_all();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  const int n_items = p.n_tiles[0] * p.n_sub;
+  const int pair = (int)(blockIdx.x >> 1), n_pairs = (int)(gridDim.x >> 1);
+  const int n_items = first_s[p.G] * p.n_sub;
+  // group, sub-tile, this CTA's first row in the group and its real rows
+  struct Item { int g, ns, pos, rows; };
+  auto item_of = [&](int item) {
+    Item it;
+    const int tile = item / p.n_sub;
+    it.ns = item - tile * p.n_sub;
+    int lo = 0, hi = p.G - 1;  // the last group whose first pair tile is <= tile
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (first_s[mid] <= tile) lo = mid; else hi = mid - 1;
+    }
+    it.g = lo;
+    it.pos = kHPairRows * (tile - first_s[lo]) + kBM * (int)rank;
+    it.rows = max(0, min(kBM, cnt_s[lo] - it.pos));
+    return it;
+  };
+  const int n_steps = 2 * p.num_kb;  // step 2 kb: x and keys, 2 kb + 1: dy and values
 
-  if (warp < kHStages) {
-    // ---- producers: warp s owns stage s (s even: x rows and key tiles, s
-    // odd: dy rows and value tiles) ----
-    const int my_stage = warp, kind = warp & 1;
-    const __nv_bfloat16* src = kind == 0 ? p.x : p.dy;
-    const CUtensorMap* tmw = kind == 0 ? &tm_wk : &tm_wv;
+  if (warp < kHGather) {
+    // ---- this CTA's rows of the steps of stage `warp` ----
     const int j = lane & 7, rsub = lane >> 3;
+    const uint32_t dst = sa(warp);
     bool ok = true;
-    int seq = 0;
-    for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
-      const int tile = item / p.n_sub, ns = item % p.n_sub;
-      const int g = p.tile_group[tile];
-      const int e = g / p.B, blk = g % p.B;
-      const int brow = e * p.H + blk * p.M + ns * p.bn;
-      const int r0 = p.tile_row0[tile], nrow = p.tile_rows[tile];
-      int tk[4];
+    uint32_t ph = 0;
+    int ks = warp;  // this warp's next step, counted from the item's first
+    for (int item = pair; item < n_items && ok && warp < n_st; item += n_pairs) {
+      if (ks < n_steps) {
+        const Item it = item_of(item);
+        int tk[4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        // padding rows gather token 0; their results are never kept
-        const int t = 32 * i + lane < nrow ? p.row_tok[r0 + 32 * i + lane] : 0;
-        tk[i] = t < 0 ? 0 : t;
+        for (int i = 0; i < 4; ++i)
+          tk[i] = 32 * i + lane < it.rows
+                      ? p.row_tok[(size_t)it.g * p.region + it.pos + 32 * i + lane] : -1;
+        for (; ks < n_steps; ks += n_st) {
+          ok = wait_warp(empty_bar(warp), ph ^ 1u, abort_flag, p.status, p.wait_limit);
+          if (!ok) break;
+          ph ^= 1u;
+          const __nv_bfloat16* sj = ((ks & 1) ? p.dy : p.x) + j * 8 + (ks >> 1) * kBK;
+#pragma unroll
+          for (int i = 0; i < 32; ++i) {
+            const int r = 4 * i + rsub;
+            const int t = __shfl_sync(0xffffffffu, tk[i >> 3], r & 31);
+            // (padding rows keep what the stage holds: their results are dropped)
+            if (t >= 0)
+              cp_async16(dst + r * 128u + ((j ^ (r & 7)) << 4), sj + (size_t)t * p.d);
+          }
+          cp_async_commit();
+          cp_async_wait<0>();
+          fence_proxy_async();
+          __syncwarp();
+          if (lane == 0) arrive_leader(full_bar(warp));
+        }
       }
-      // stage sequence: seq = 2 kb + kind over the item's k-blocks
-      for (int ks = 0; ks < 2 * p.num_kb; ++ks, ++seq) {
-        const int stage = seq % kHStages;
-        if (stage != my_stage) continue;
-        const int kb = ks >> 1;
-        const uint32_t phase = (uint32_t)(seq / kHStages) & 1u;
-        ok = wait_warp(empty_bar(stage), phase ^ 1u, abort_flag, p.status, p.wait_limit);
+      ks -= n_steps;
+    }
+  } else if (warp == kHLoader) {
+    // ---- this CTA's half of every step's weight tile ----
+    bool ok = true;
+    int s = 0;
+    uint32_t ph = 0;
+    long long issued = 0;
+    for (int item = pair; item < n_items && ok; item += n_pairs) {
+      const Item it = item_of(item);
+      const int e = it.g / p.B, blk = it.g - e * p.B;
+      const int row = e * p.H + blk * p.M + it.ns * p.bn + (int)rank * (p.bn / 2);
+      for (int ks = 0; ks < n_steps; ++ks) {
+        ok = wait_warp(empty_bar(s), ph ^ 1u, abort_flag, p.status, p.wait_limit);
         if (!ok) break;
         if (lane == 0) {
-          mbar_expect_tx_only(full_bar(stage), wtile);
-          tma_load_2d(sw(stage), tmw, full_bar(stage), kb * kBK, brow);
+          if (leader) mbar_expect_tx(full_bar(s), (uint32_t)p.bn * 128u);
+          tma_load_2d_pair(sw(s), (ks & 1) ? &tm_wv : &tm_wk, mapa_shared(full_bar(s), 0),
+                           (ks >> 1) * kBK, row);
         }
-        const uint32_t dst = sa(stage);
-        const __nv_bfloat16* sj = src + j * 8 + kb * kBK;
-#pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          const int r = 4 * i + rsub;
-          const int t = __shfl_sync(0xffffffffu, tk[i >> 3], r & 31);
-          cp_async16(dst + r * 128u + ((j ^ (r & 7)) << 4), sj + (size_t)t * p.d);
-        }
-        cp_async_commit();
-        cp_async_wait<0>();
-        fence_proxy_async();
         __syncwarp();
-        if (lane == 0) mbar_arrive(full_bar(stage));
+        ++issued;
+        if (++s == n_st) { s = 0; ph ^= 1u; }
       }
     }
-  } else if (warp == kMmaWarp) {
-    // ---- MMA issuer ----
-    const uint32_t idesc = idesc_bf16(kBM, p.bn);
-    int seq = 0;
-    uint32_t acc_phase = 0;
-    bool ok = true;
-    for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
-      ok = wait_warp(acce, acc_phase ^ 1u, abort_flag, p.status, p.wait_limit);
-      if (!ok) break;
-      tc_fence_after();
-      for (int ks = 0; ks < 2 * p.num_kb; ++ks, ++seq) {
-        const int stage = seq % kHStages;
-        const uint32_t phase = (uint32_t)(seq / kHStages) & 1u;
-        ok = wait_warp(full_bar(stage), phase, abort_flag, p.status, p.wait_limit);
+    // loads still in flight land before the pair exits
+    if (leader && lane == 0)
+      for (long long q = issued > n_st ? issued - n_st : 0; q < issued; ++q)
+        wait_settle(full_bar((int)(q % n_st)), (uint32_t)((q / n_st) & 1), p.wait_limit / 16);
+    __syncwarp();
+  } else if (warp == kHMma) {
+    // ---- MMA issuer (the leader CTA) ----
+    if (leader) {
+      const uint32_t idesc = idesc_bf16(2 * kBM, p.bn);
+      const uint16_t both = 3;
+      int s = 0;
+      uint32_t ph = 0, acc_ph = 0;
+      bool ok = true, any = false;
+      for (int item = pair; item < n_items && ok; item += n_pairs) {
+        ok = wait_warp_cluster(acce, acc_ph ^ 1u, abort_flag, p.status, p.wait_limit);
         if (!ok) break;
         tc_fence_after();
-        // even stages feed x K (acc_a), odd ones dy V^T (acc_g)
-        const uint32_t d_tmem = tmem_base + ((ks & 1) ? kAcc2 : 0u);
-        if (elect_one()) {
+        for (int ks = 0; ks < n_steps; ++ks) {
+          ok = wait_warp_cluster(full_bar(s), ph, abort_flag, p.status, p.wait_limit);
+          if (!ok) break;
+          tc_fence_after();
+          // even steps feed x K (acc_a), odd ones dy V^T (acc_g)
+          const uint32_t d_tmem = tmem_base + ((ks & 1) ? kAcc2 : 0u);
+          if (elect_one()) {
+            const uint64_t a = sw128_desc(sa(s)), b = sw128_desc(sw(s));
 #pragma unroll
-          for (int k = 0; k < kBK / 16; ++k)
-            umma_bf16(d_tmem, sw128_desc(sa(stage) + k * 32), sw128_desc(sw(stage) + k * 32),
-                      idesc, ((ks >> 1) | k) != 0 ? 1u : 0u);
-          umma_commit(empty_bar(stage));
+            for (int k = 0; k < kBK / 16; ++k)
+              umma_bf16_pair(d_tmem, a + 2 * k, b + 2 * k, idesc, ((ks >> 1) | k) != 0 ? 1u : 0u);
+            umma_commit_pair(empty_bar(s), both);
+            if (ks == n_steps - 1) umma_commit_pair(accf, both);
+          }
+          __syncwarp();
+          any = true;
+          if (++s == n_st) { s = 0; ph ^= 1u; }
         }
-        __syncwarp();
+        acc_ph ^= 1u;
       }
-      if (!ok) break;
-      if (elect_one()) umma_commit(accf);
-      __syncwarp();
-      acc_phase ^= 1u;
+      // every MMA issued has completed before the pair releases TMEM
+      if (any) {
+        if (elect_one()) umma_commit_pair(mma_done, 1);
+        __syncwarp();
+        wait_settle(mma_done, 0u, p.wait_limit);
+      }
     }
-  } else if (warp >= kFirstEpiWarp) {
+    __syncwarp();
+  } else {
     // ---- epilogue ----
     const int q = warp & 3;
-    const int half = (warp - kFirstEpiWarp) >> 2;
-    const int cols = p.bn / 2;
-    const int c_begin = half * cols;
-    uint32_t acc_phase = 0;
-    for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
-      const int tile = item / p.n_sub, ns = item % p.n_sub;
-      const int g = p.tile_group[tile];
-      const int e = g / p.B;
+    const int cols = p.bn / 2, c_begin = ((warp - kHFirstEpi) >> 2) * cols;
+    uint8_t* stg = staging + (size_t)(warp - kHFirstEpi) * 2 * kHPiece;
+    uint8_t* srow = stg + lane * 64;
+    const uint32_t sx = (uint32_t)(lane >> 1) & 3u;  // 64-byte swizzle of this row's chunks
+    uint32_t acc_ph = 0;
+    for (int item = pair; item < n_items; item += n_pairs) {
+      const Item it = item_of(item);
+      const int e = it.g / p.B;
       const int r = q * 32 + lane;
-      const bool real = r < p.tile_rows[tile];
-      const int tok = real ? p.row_tok[p.tile_row0[tile] + r] : -1;
-      const float w = real ? p.row_w[p.tile_row0[tile] + r] : 0.f;
-      if (!wait_warp(accf, acc_phase, abort_flag, p.status, p.wait_limit)) break;
+      const bool real = r < it.rows;
+      const size_t lr = (size_t)it.g * p.region + it.pos + r;
+      const int tok = real ? p.row_tok[lr] : -1;
+      // (padding rows have weight 0: their outputs are zeros, which the
+      // weight-gradient kernel sums over; see the finite selects below)
+      const float w = real ? p.row_w[lr] : 0.f;
+      if (!wait_warp(accf, acc_ph, abort_flag, p.status, p.wait_limit)) break;
       tc_fence_after();
-      const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16);
-      const size_t orow = ((size_t)tile * kBM + r) * p.M + ns * p.bn + c_begin;
-      float dot = 0.f;
-      for (int c = 0; c < cols; c += 16) {
-        float a[16], gv[16];
-        tmem_ld16(t_row + c_begin + c, a);
-        tmem_ld16(t_row + kAcc2 + c_begin + c, gv);
-        uint32_t od[8], oh[8];
+      if (it.rows > 0) {  // (a half past the group's end has no tile of its own)
+        const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16) + c_begin;
+        // rows and columns of the outputs' tile (maps of 32 x 32 boxes)
+        const int row0 = first128_s[it.g] * kBM + it.pos + q * 32;
+        const int col0 = it.ns * p.bn + c_begin;
+        float dot0 = 0.f, dot1 = 0.f;
+        for (int c = 0; c < cols; c += 32) {
+          uint32_t od[16], oh[16];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          float d0 = 0.f, d1 = 0.f, h0 = 0.f, h1 = 0.f;
-          if (tok >= 0) {
-            float g0, g1, dg0, dg1;
-            gelu_and_grad(a[2 * i], g0, dg0);
-            gelu_and_grad(a[2 * i + 1], g1, dg1);
-            dot = fmaf(g0, gv[2 * i], dot);
-            dot = fmaf(g1, gv[2 * i + 1], dot);
-            d0 = w * gv[2 * i] * dg0;
-            d1 = w * gv[2 * i + 1] * dg1;
-            h0 = w * g0;
-            h1 = w * g1;
+          for (int hh = 0; hh < 2; ++hh) {
+            float a[16], gv[16];
+            tmem_ld16(t_row + c + 16 * hh, a);
+            tmem_ld16(t_row + kAcc2 + c + 16 * hh, gv);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              // a padding row's accumulators may hold anything
+              const float a0 = real ? a[2 * i] : 0.f, a1 = real ? a[2 * i + 1] : 0.f;
+              const float v0 = real ? gv[2 * i] : 0.f, v1 = real ? gv[2 * i + 1] : 0.f;
+              float g0, g1, dg0, dg1;
+              gelu_and_grad(a0, g0, dg0);
+              gelu_and_grad(a1, g1, dg1);
+              dot0 = fmaf(g0, v0, dot0);
+              dot1 = fmaf(g1, v1, dot1);
+              od[8 * hh + i] = pack_bf16(w * v0 * dg0, w * v1 * dg1);
+              oh[8 * hh + i] = pack_bf16(w * g0, w * g1);
+            }
           }
-          od[i] = pack_bf16(d0, d1);
-          oh[i] = pack_bf16(h0, h1);
+          if (lane == 0) bulk_wait_read();  // the last pieces have left the staging
+          __syncwarp();
+#pragma unroll
+          for (int jj = 0; jj < 4; ++jj) {
+            const uint32_t ch = ((uint32_t)jj ^ sx) << 4;
+            *reinterpret_cast<uint4*>(srow + ch) =
+                make_uint4(od[4 * jj], od[4 * jj + 1], od[4 * jj + 2], od[4 * jj + 3]);
+            *reinterpret_cast<uint4*>(srow + kHPiece + ch) =
+                make_uint4(oh[4 * jj], oh[4 * jj + 1], oh[4 * jj + 2], oh[4 * jj + 3]);
+          }
+          fence_proxy_async();
+          __syncwarp();
+          if (lane == 0) {
+            tma_store_2d(&tm_da, smem_u32(stg), col0 + c, row0);
+            tma_store_2d(&tm_hw, smem_u32(stg) + kHPiece, col0 + c, row0);
+            bulk_commit();
+          }
         }
-        // padding rows are written as zeros: the weight-gradient kernel sums
-        // over whole tiles
-        uint4* pd = reinterpret_cast<uint4*>(p.da + orow + c);
-        uint4* ph = reinterpret_cast<uint4*>(p.hw + orow + c);
-        pd[0] = make_uint4(od[0], od[1], od[2], od[3]);
-        pd[1] = make_uint4(od[4], od[5], od[6], od[7]);
-        ph[0] = make_uint4(oh[0], oh[1], oh[2], oh[3]);
-        ph[1] = make_uint4(oh[4], oh[5], oh[6], oh[7]);
+        if (tok >= 0) atomicAdd(p.dwt + (size_t)tok * p.K1 + e, dot0 + dot1);
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(acce);
-      if (tok >= 0) atomicAdd(p.dwt + (size_t)tok * p.K1 + e, dot);
-      acc_phase ^= 1u;
+      if (lane == 0) arrive_leader(acce);
+      acc_ph ^= 1u;
     }
+    if (lane == 0) bulk_wait_all();
+    __syncwarp();
   }
+  // every warp converged before the CTA barrier; then each CTA tells its peer
+  // that it is done with the pair's TMEM (the leader after its MMAs
+  // completed), and the owner warp waits for the peer's word
   __syncwarp();
   tc_fence_before();
   __syncthreads();
-  if (warp == kMmaWarp) {
+  if (threadIdx.x == 0) mbar_arrive_cluster(mapa_shared(fin, rank ^ 1u));
+  if (warp == kHMma) {
+    wait_settle(fin, 0u, p.wait_limit);
     tc_fence_after();
-    tmem_dealloc(tmem_base, kTmemCols);
+    tmem_dealloc_pair(tmem_base, kTmemCols);
   }
 }
 
@@ -812,15 +942,22 @@ int backward_setup(unif_moe_layer* L) {
   using namespace tc::bwd;
   const uint64_t E = (uint64_t)L->K + 1;
   Workspace& w = L->ws;
-  if (!encode_bf16_map(&L->tm_wdownT, w.w_downT, L->d, E * L->H, tc::kBK, L->up_bn, 128) ||
+  if (!encode_bf16_map(&L->tm_wdownT, w.w_downT, L->d, E * L->H, tc::kBK, L->up_bn / 2, 128) ||
+      !encode_bf16_map(&L->tm_wup_half, L->w_up, L->d, E * L->H, tc::kBK, L->up_bn / 2, 128) ||
       !encode_bf16_map(&L->tm_wupT, w.w_upT, L->H, E * L->d, tc::kBK, L->down_bn, 128) ||
       !encode_bf16_map(&L->tm_da, w.da, L->M, (uint64_t)L->max_rows, tc::kBK, tc::kBM, 128) ||
+      !encode_bf16_map(&L->tm_da_st, w.da, L->M, (uint64_t)L->max_rows, 32, 32, 64) ||
+      !encode_bf16_map(&L->tm_hw_st, w.hw, L->M, (uint64_t)L->max_rows, 32, 32, 64) ||
       !encode_bf16_map(&L->tm_da_q, w.da, L->M, (uint64_t)L->max_rows, tc::kBK, kRows, 128) ||
       !encode_bf16_map(&L->tm_hw_q, w.hw, L->M, (uint64_t)L->max_rows, tc::kBK, kRows, 128)) {
     set_error("cuTensorMapEncodeTiled failed for the backward maps");
     return UNIF_MOE_ERR_CUDA;
   }
-  L->bwd_hidden_smem = 1024 + kHStages * hidden_stage_bytes(L->up_bn) + 256;
+  L->bwd_hidden_stages = kHGather;
+  while (L->bwd_hidden_stages > kHMinStages &&
+         hidden_smem_bytes(L->up_bn, L->bwd_hidden_stages, L->G) > 232448)
+    --L->bwd_hidden_stages;
+  L->bwd_hidden_smem = hidden_smem_bytes(L->up_bn, L->bwd_hidden_stages, L->G);
   L->bwd_wgrad_smem =
       1024 + kWStages * wgrad_stage_bytes(L->up_bn) + 96 + 4 * (3 * (uint32_t)L->G + 2) + 16;
   if (L->bwd_hidden_smem > 232448 || L->bwd_wgrad_smem > 232448) {
@@ -835,6 +972,24 @@ int backward_setup(unif_moe_layer* L) {
     set_error("cudaFuncSetAttribute failed for the backward kernels");
     return UNIF_MOE_ERR_CUDA;
   }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(L->n_sm);
+  cfg.blockDim = dim3(kHThreads);
+  cfg.dynamicSmemBytes = L->bwd_hidden_smem;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 2;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int clusters = 0;
+  if (cudaOccupancyMaxActiveClusters(&clusters, bwd_hidden_kernel, &cfg) != cudaSuccess ||
+      clusters < 1) {
+    set_error("backward: no CTA pair fits on this device");
+    return UNIF_MOE_ERR_CUDA;
+  }
+  L->bwd_pairs = std::min(clusters, L->n_sm / 2);
   return UNIF_MOE_OK;
 }
 
@@ -875,19 +1030,30 @@ int backward_run(unif_moe_layer* L, const void* x, const void* dy, int T, const 
   // hidden gradients
   {
     HiddenParams p;
-    p.n_tiles = w.n_tiles; p.tile_group = w.tile_group; p.tile_row0 = w.tile_row0;
-    p.tile_rows = w.tile_rows; p.row_tok = w.row_tok; p.row_w = w.row_w;
+    p.counts = w.grp_cnt; p.G = L->G; p.region = L->region_rows;
+    p.row_tok = w.row_tok; p.row_w = w.row_w;
     p.x = static_cast<const __nv_bfloat16*>(x);
     p.dy = static_cast<const __nv_bfloat16*>(dy);
-    p.da = static_cast<__nv_bfloat16*>(w.da);
-    p.hw = static_cast<__nv_bfloat16*>(w.hw);
     p.dwt = w.dwt;
     p.n_sub = L->up_nsub; p.bn = L->up_bn; p.num_kb = L->d / tc::kBK;
     p.B = L->B; p.M = L->M; p.H = L->H; p.d = L->d; p.K1 = K1;
+    p.stages = L->bwd_hidden_stages;
     p.status = w.status;
     p.wait_limit = gemm_wait_limit();
-    bwd_hidden_kernel<<<L->n_sm, kThreads, L->bwd_hidden_smem, s>>>(L->tm_wup, L->tm_wdownT, p);
-    CKB(cudaGetLastError());
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(2 * L->bwd_pairs);
+    cfg.blockDim = dim3(kHThreads);
+    cfg.dynamicSmemBytes = L->bwd_hidden_smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    CKB(cudaLaunchKernelEx(&cfg, bwd_hidden_kernel, L->tm_wup_half, L->tm_wdownT, L->tm_da_st,
+                           L->tm_hw_st, p));
   }
   // dL/dx from the experts: DA K_e (the down kernel on the transposed keys)
   CKB(launch_down_streaming(L, L->tm_da, L->tm_wupT, nullptr, dx, s));

@@ -573,15 +573,16 @@ __device__ void group_rows_expert(const GroupArgs& a, int tid, int t0, uint64_t 
   }
 }
 
-// The tiles of the groups whose sizes (clamped to the region) are in
+// The tiles (TR rows) of the groups whose sizes (clamped to the region) are in
 // cnt_s[0..G): first_s[g] = first tile of group g (first_s[G] = all tiles).
 // Run by one warp; shared arrays of G + 1 and G ints.
+template <int TR = 128>
 __device__ __forceinline__ void tile_scan(int G, int lane, int32_t* first_s,
                                           const int32_t* cnt_s) {
   int carry = 0;
   for (int g0 = 0; g0 < G; g0 += 32) {
     const int g = g0 + lane;
-    const int nt = g < G ? (cnt_s[g] + 127) / 128 : 0;
+    const int nt = g < G ? (cnt_s[g] + TR - 1) / TR : 0;
     int inc = nt;
     for (int o = 1; o < 32; o <<= 1) {
       const int v = __shfl_up_sync(0xffffffffu, inc, o);

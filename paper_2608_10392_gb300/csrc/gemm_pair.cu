@@ -145,20 +145,8 @@ pair_up_kernel(const __grid_constant__ CUtensorMap tmB, Params p) {
   __syncthreads();
   if (warp == 0) {
     tile_scan(p.G, lane, first128_s, cnt_s);
-  } else if (warp == 1) {  // the same in pair tiles
-    int carry = 0;
-    for (int g0 = 0; g0 < p.G; g0 += 32) {
-      const int g = g0 + lane;
-      const int nt = g < p.G ? (cnt_s[g] + kPairRows - 1) / kPairRows : 0;
-      int inc = nt;
-      for (int o = 1; o < 32; o <<= 1) {
-        const int v = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o) inc += v;
-      }
-      if (g < p.G) first_s[g] = carry + inc - nt;
-      carry += __shfl_sync(0xffffffffu, inc, 31);
-    }
-    if (lane == 0) first_s[p.G] = carry;
+  } else if (warp == 1) {
+    tile_scan<kPairRows>(p.G, lane, first_s, cnt_s);
   }
   __syncwarp();
   tc_fence_before();

@@ -199,12 +199,14 @@ struct unif_moe_layer {
   int ffn_per_cta = 0, ffn_slots = 0;  // pair tiles per pair (run table), ring half-slabs
   uint32_t ffn_smem = 0;
   // backward: transposed weights and the per-row gradient buffers
-  CUtensorMap tm_wdownT;    // w_downT [(K+1) H][d], boxes of 64 x up_bn
+  CUtensorMap tm_wdownT;    // w_downT [(K+1) H][d], boxes of 64 x up_bn / 2
   CUtensorMap tm_wupT;      // w_upT [(K+1) d][H], boxes of 64 x down_bn
   CUtensorMap tm_da;        // da [max_rows][M], boxes of 64 x 128 (dx GEMM A operand)
+  CUtensorMap tm_da_st, tm_hw_st;  // da, hw, store boxes of 32 x 32 (64-byte swizzle)
   CUtensorMap tm_da_q;      // da, boxes of 64 x 32 (weight-gradient operand)
   CUtensorMap tm_hw_q;      // hw, boxes of 64 x 32
   uint32_t bwd_hidden_smem = 0, bwd_wgrad_smem = 0;
+  int bwd_hidden_stages = 0, bwd_pairs = 0;  // ring depth and CTA pairs of the hidden kernel
   // Pipelined host-buffer forwards (UNIF_MOE_FEATURE_HOST_IO): the handle's
   // copy streams, and per staging slot the events that order its reuse
   // (input landed, kernels done, output copied out).
