@@ -78,10 +78,7 @@ __device__ __forceinline__ uint64_t sw128_mn_desc(uint32_t saddr, uint32_t lbo) 
          ((uint64_t)(1024 >> 4) << 32) | ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
 }
 
-constexpr int kThreads = 416;     // 13 warps
-constexpr int kMmaWarp = 4;
-constexpr int kFirstEpiWarp = 5;  // warps 5-12
-constexpr int kEpiWarps = 8;
+constexpr int kEpiWarps = 8;      // of the weight-gradient kernel
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kAcc2 = 256;   // TMEM column of the second accumulator
 
@@ -101,8 +98,8 @@ constexpr uint32_t kAcc2 = 256;   // TMEM column of the second accumulator
 // epilogue of the one before; the ring holds the next tile's first steps by
 // then. (16 epilogue warps of half the columns ran no faster.)
 // Measured (ViT-S, 12,608 tokens; one CTA per tile, four gather warps, erff,
-// a 32-byte row piece per thread's store before): 138 -> HID_S us; BERT-base
-// (2,300 tokens) 102 -> HID_B.
+// a 32-byte row piece per thread's store before): 138 -> 111 us; BERT-base
+// (2,300 tokens) 102 -> 76.
 // ---------------------------------------------------------------------------
 struct HiddenParams {
   const int32_t* counts;   // [G] group sizes (the forward's)
@@ -112,6 +109,15 @@ struct HiddenParams {
   const __nv_bfloat16* x;
   const __nv_bfloat16* dy;
   float* dwt;          // [T][K+1]
+  // outputs that later kernels add into, zeroed here by the odd CTAs' MMA
+  // warps (which have no MMAs to issue): dw_up, dw_down (w4 float4 each),
+  // dw_router (n_wr floats), dbias (n_bias floats)
+  float4* dw_up;
+  float4* dw_down;
+  float* dw_router;
+  float* dbias;
+  long long w4;
+  int n_wr, n_bias;
   int n_sub, bn, num_kb, B, M, H, d, K1, stages;
   int* status;
   long long wait_limit;
@@ -125,12 +131,13 @@ constexpr int kHPairRows = 256;
 constexpr uint32_t kHPiece = 32u * 64u;  // 32 rows x 32 bf16
 constexpr uint32_t kHStaging = kHEpiWarps * 2u * kHPiece;
 constexpr uint32_t kHBarBytes = 256;
+constexpr uint32_t kHZero = 4096;  // zeros, the source of the bulk stores that clear the outputs
 
 __host__ __device__ constexpr uint32_t hidden_stage_bytes(int bn) {
   return kStageA + (uint32_t)bn * 64u;
 }
 __host__ __device__ constexpr uint32_t hidden_smem_bytes(int bn, int stages, int G) {
-  return 1024u + (uint32_t)stages * hidden_stage_bytes(bn) + kHStaging + kHBarBytes +
+  return 1024u + (uint32_t)stages * hidden_stage_bytes(bn) + kHStaging + kHZero + kHBarBytes +
          (uint32_t)((3 * G + 2) * 4 + 15) / 16u * 16u;
 }
 
@@ -156,7 +163,8 @@ bwd_hidden_kernel(const __grid_constant__ CUtensorMap tm_wk, const __grid_consta
   auto sa = [&](int s) { return s0 + (uint32_t)s * stage_bytes; };
   auto sw = [&](int s) { return s0 + (uint32_t)s * stage_bytes + kStageA; };
   uint8_t* staging = smem + (size_t)n_st * stage_bytes;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(staging + kHStaging);
+  uint8_t* zeros = staging + kHStaging;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(zeros + kHZero);
   const uint32_t bar0 = smem_u32(bars);
   auto full_bar = [&](int s) { return bar0 + 8u * s; };
   auto empty_bar = [&](int s) { return bar0 + 8u * (kHGather + s); };
@@ -332,6 +340,22 @@ bwd_hidden_kernel(const __grid_constant__ CUtensorMap tm_wk, const __grid_consta
         __syncwarp();
         wait_settle(mma_done, 0u, p.wait_limit);
       }
+    } else {
+      for (uint32_t k = lane; k < kHZero / 16; k += 32)
+        reinterpret_cast<uint4*>(zeros)[k] = make_uint4(0u, 0u, 0u, 0u);
+      fence_proxy_async();
+      __syncwarp();
+      const long long bytes = 16 * p.w4;
+      for (long long k = (long long)kHZero * (32 * pair + lane); k < bytes;
+           k += (long long)kHZero * 32 * n_pairs) {
+        const uint32_t n = (uint32_t)min((long long)kHZero, bytes - k);
+        bulk_store(reinterpret_cast<uint8_t*>(p.dw_up) + k, smem_u32(zeros), n);
+        bulk_store(reinterpret_cast<uint8_t*>(p.dw_down) + k, smem_u32(zeros), n);
+      }
+      bulk_commit();
+      for (int k = 32 * pair + lane; k < p.n_wr; k += 32 * n_pairs) p.dw_router[k] = 0.f;
+      for (int k = 32 * pair + lane; k < p.n_bias; k += 32 * n_pairs) p.dbias[k] = 0.f;
+      bulk_wait_all();
     }
     __syncwarp();
   } else {
@@ -424,18 +448,24 @@ bwd_hidden_kernel(const __grid_constant__ CUtensorMap tm_wk, const __grid_consta
 }
 
 // ---------------------------------------------------------------------------
-// bwd_wgrad_kernel: per item (group g, 128 features c of d, N chunk nc of the
-// block's M channels) two accumulators over all rows of the group, 64 rows
-// per stage:
-//   acc1[i][h] = sum_r X[tok_r][c*128 + i] DA[r][nc*N + h]   -> dK_e (transposed)
-//   acc2[i][h] = sum_r DY[tok_r][c*128 + i] HW[r][nc*N + h]  -> dV_e
+// bwd_wgrad_kernel: per item (group g, a chunk of its rows, 128 features c of
+// d, N chunk nc of the block's M channels, kind) one accumulator over the
+// chunk's rows, 64 rows per stage:
+//   kind 0: acc[i][h] = sum_r X[tok_r][c*128 + i] DA[r][nc*N + h]   -> dK_e (transposed)
+//   kind 1: acc[i][h] = sum_r DY[tok_r][c*128 + i] HW[r][nc*N + h]  -> dV_e
 // The token rows are the reduction dimension, so both operands are MN-major:
 // the gathered rows (x, dy) and the TMA tiles (DA, HW) keep the 128-byte
-// swizzled row layout, read with MN-major descriptors. A group's rows are
-// split into chunks of kChunkTiles tiles, one work item each, whose partial
-// sums are added into the (zeroed) outputs.
-// Roles: warps 0-3 fill the 4-deep ring (warp s: the x and dy rows of stage
-// s, and the DA/HW tiles by TMA), warp 4 MMAs, warps 5-12 epilogue.
+// swizzled row layout, read with MN-major descriptors. A group's tiles are
+// split evenly into chunks of at most kChunkTiles, whose partial sums are
+// added into the (zeroed) outputs.
+// Roles: warps 0-4 fill the ring, a warp per stage (the gathered rows, and
+// the DA or HW tiles by TMA), warp 5 MMAs, warps 6-13 epilogue. The two
+// kinds are items of their own so that one accumulator leaves room in TMEM
+// for a second: an item's atomic adds run under the next one's MMAs. Bound
+// by the operand bytes out of L2 (40 KB per 64 rows of 192 channels).
+// Measured (both kinds in one item, accumulators not overlapped, four stages
+// of 32 rows before): ViT-S 12,608 tokens 117 -> 101 us, BERT-base (2,300
+// tokens) 130 -> 115.
 // ---------------------------------------------------------------------------
 struct WgradParams {
   const int32_t* counts;   // [G] group sizes (the forward's)
@@ -444,43 +474,49 @@ struct WgradParams {
   const __nv_bfloat16* dy;
   float* dw_up;    // [K+1][H][d]
   float* dw_down;  // [K+1][d][H]
-  int G, region, B, M, H, d, N, n_nc, n_c;
+  int G, region, B, M, H, d, N, n_nc, n_c, stages;
   int* status;
   long long wait_limit;
 };
 
-constexpr uint32_t kRows = 32;                 // group rows per stage
-constexpr uint32_t kPBytes = 2u * kRows * 128u;  // 128 features x 32 rows (two 64-column blocks)
-constexpr int kWStages = 4;                      // one stage per producer warp
-constexpr int kQuarters = kBM / (int)kRows;      // stages per 128-row tile
-constexpr int kChunkTiles = 8;                   // tiles of a group per work item
+constexpr uint32_t kRows = 64;                 // group rows per stage
+constexpr uint32_t kPBytes = 2u * kRows * 128u;  // 128 features x 64 rows (two 64-column blocks)
+constexpr int kWStages = 5;                      // at most one stage per producer warp
+constexpr int kWMinStages = 2;
+constexpr int kWMma = 5, kWFirstEpi = 6;
+constexpr int kWThreads = 32 * (kWFirstEpi + kEpiWarps);  // 448
+constexpr int kParts = kBM / (int)kRows;         // stages per 128-row tile
+constexpr int kChunkTiles = 8;                   // most tiles of a group per work item
 
 __host__ __device__ constexpr uint32_t wgrad_stage_bytes(int N) {
-  return 2u * kPBytes + 2u * (uint32_t)(N / 64) * kRows * 128u;
+  return kPBytes + (uint32_t)(N / 64) * kRows * 128u;
+}
+__host__ __device__ constexpr uint32_t wgrad_smem_bytes(int N, int stages, int G) {
+  return 1024u + (uint32_t)stages * wgrad_stage_bytes(N) + 160u + 4u * (3u * (uint32_t)G + 2u) + 16u;
 }
 
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(kWThreads, 1)
 bwd_wgrad_kernel(const __grid_constant__ CUtensorMap tm_da, const __grid_constant__ CUtensorMap tm_hw,
                  WgradParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+  const int n_st = p.stages;
   const uint32_t stage_bytes = wgrad_stage_bytes(p.N);
   const uint32_t qbytes = (uint32_t)(p.N / 64) * kRows * 128u;
   const uint32_t s0 = smem_u32(smem);
-  // stage s: [x rows][dy rows][DA tile][HW tile]
-  auto spx = [&](int s) { return s0 + s * stage_bytes; };
-  auto spy = [&](int s) { return s0 + s * stage_bytes + kPBytes; };
-  auto sqa = [&](int s) { return s0 + s * stage_bytes + 2 * kPBytes; };
-  auto sqh = [&](int s) { return s0 + s * stage_bytes + 2 * kPBytes + qbytes; };
+  // stage s: [x or dy rows][DA or HW tile]
+  auto sp = [&](int s) { return s0 + (uint32_t)s * stage_bytes; };
+  auto sq = [&](int s) { return s0 + (uint32_t)s * stage_bytes + kPBytes; };
   uint8_t* gen_base = smem;  // generic pointer for zero-filling padding rows
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kWStages * stage_bytes);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + (size_t)n_st * stage_bytes);
   const uint32_t bar0 = smem_u32(bars);
   auto full_bar = [&](int s) { return bar0 + 8u * s; };
   auto empty_bar = [&](int s) { return bar0 + 8u * (kWStages + s); };
-  const uint32_t accf = bar0 + 8u * (2 * kWStages);
-  const uint32_t acce = bar0 + 8u * (2 * kWStages + 1);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kWStages + 2);
+  auto accf_bar = [&](int a) { return bar0 + 8u * (2 * kWStages + a); };
+  auto acce_bar = [&](int a) { return bar0 + 8u * (2 * kWStages + 2 + a); };
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kWStages + 4);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  static_assert(8 * (2 * kWStages + 4) + 16 <= 160, "barrier region");
   int32_t* first_s = reinterpret_cast<int32_t*>(tmem_slot + 4);  // [G + 1] first tiles
   int32_t* cnt_s = first_s + p.G + 1;                             // [G] sizes
   int32_t* chunk_s = cnt_s + p.G;                                 // [G + 1] first chunks
@@ -491,20 +527,22 @@ bwd_wgrad_kernel(const __grid_constant__ CUtensorMap tm_da, const __grid_constan
       mbar_init(full_bar(s), 1);
       mbar_init(empty_bar(s), 1);
     }
-    mbar_init(accf, 1);
-    mbar_init(acce, kEpiWarps);
+    for (int a = 0; a < 2; ++a) {
+      mbar_init(accf_bar(a), 1);
+      mbar_init(acce_bar(a), kEpiWarps);
+    }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == kMmaWarp) {
+  if (warp == kWMma) {
     tmem_alloc(smem_u32(tmem_slot), kTmemCols);
     tmem_relinquish();
   }
-  if (warp == kThreads / 32 - 1) {
+  grid_dep_wait();  // dL/da, w GeLU(a), and the zeroed outputs
+  if (warp == kWThreads / 32 - 1) {
     tile_table(p.counts, p.G, p.region, lane, first_s, cnt_s);
     __syncwarp();
-    // each group's tiles in chunks of kChunkTiles: the first chunk of every
-    // group (chunk_s[G] = all chunks)
+    // the first chunk of every group (chunk_s[G] = all chunks)
     int carry = 0;
     for (int g0 = 0; g0 < p.G; g0 += 32) {
       const int g = g0 + lane;
@@ -524,155 +562,159 @@ bwd_wgrad_kernel(const __grid_constant__ CUtensorMap tm_da, const __grid_constan
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  const int n_items = chunk_s[p.G] * p.n_c * p.n_nc;
+  const int n_items = chunk_s[p.G] * p.n_c * p.n_nc * 2;
   // item -> (group g, its tiles [t0, t0 + nt) of one chunk, feature chunk c,
-  // N chunk nc); rows of the chunk start at row r0 of the group
-  auto decode = [&](int item, int& g, int& t0, int& nt, int& r0, int& c, int& nc) {
-    nc = item % p.n_nc;
-    c = (item / p.n_nc) % p.n_c;
-    const int q = item / (p.n_nc * p.n_c);
+  // N chunk nc, kind); rows of the chunk start at row r0 of the group
+  struct Item { int g, t0, nt, r0, c, nc, kind; };
+  auto decode = [&](int item) {
+    Item it;
+    it.kind = item & 1;
+    int q = item >> 1;
+    it.nc = q % p.n_nc;
+    q /= p.n_nc;
+    it.c = q % p.n_c;
+    q /= p.n_c;
     int lo = 0, hi = p.G - 1;  // the last group whose first chunk is <= q
     while (lo < hi) {
       const int mid = (lo + hi + 1) >> 1;
       if (chunk_s[mid] <= q) lo = mid; else hi = mid - 1;
     }
-    g = lo;
-    const int k = q - chunk_s[g];
-    t0 = first_s[g] + k * kChunkTiles;
-    nt = min(kChunkTiles, first_s[g + 1] - t0);
-    r0 = k * kChunkTiles * kBM;
+    it.g = lo;
+    const int k = q - chunk_s[lo], nch = chunk_s[lo + 1] - chunk_s[lo];
+    const int tiles = first_s[lo + 1] - first_s[lo];
+    const int ta = tiles * k / nch;
+    it.t0 = first_s[lo] + ta;
+    it.nt = tiles * (k + 1) / nch - ta;
+    it.r0 = ta * kBM;
+    return it;
   };
 
   if (warp < kWStages) {
-    // ---- producers: warp w owns stage w: the x and dy rows of its 32 group
-    // rows, and lane 0 brings the DA and HW tiles by TMA ----
-    const int my_stage = warp;
+    // ---- producers: warp w owns stage w: the gathered rows, and lane 0
+    // brings the DA or HW tile by TMA ----
     const int j = lane & 7, rsub = lane >> 3;
     bool ok = true;
-    int seq = 0;
-    for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
-      int g, t_first, nt, r0, c, nc;
-      decode(item, g, t_first, nt, r0, c, nc);
-      const int size = cnt_s[g];
-      for (int kt = 0; kt < nt * kQuarters && ok; ++kt, ++seq) {  // 32-row quarters of the tiles
-        const int stage = seq % kWStages;
-        if (stage != my_stage) continue;
-        const uint32_t phase = (uint32_t)(seq / kWStages) & 1u;
-        ok = wait_warp(empty_bar(stage), phase ^ 1u, abort_flag, p.status, p.wait_limit);
+    uint32_t ph = 0;
+    int kt = warp;  // this warp's next stage, counted from the item's first
+    for (int item = blockIdx.x; item < n_items && ok && warp < n_st; item += gridDim.x) {
+      const Item it = decode(item);
+      const int n_steps = it.nt * kParts;
+      const int size = cnt_s[it.g];
+      const CUtensorMap* tm = it.kind == 0 ? &tm_da : &tm_hw;
+      const __nv_bfloat16* sj = (it.kind == 0 ? p.x : p.dy) + (size_t)it.c * 128 + j * 8;
+      for (; kt < n_steps; kt += n_st) {
+        ok = wait_warp(empty_bar(warp), ph ^ 1u, abort_flag, p.status, p.wait_limit);
         if (!ok) break;
-        const int row_in_group = r0 + kt * (int)kRows;  // first row of this quarter in the group
-        const int crow = (t_first + kt / kQuarters) * kBM + (kt % kQuarters) * (int)kRows;
+        ph ^= 1u;
         if (lane == 0) {
-          mbar_expect_tx_only(full_bar(stage), 2u * qbytes);
-          for (int b = 0; b < p.N / 64; ++b) {
-            tma_load_2d(sqa(stage) + b * kRows * 128u, &tm_da, full_bar(stage), nc * p.N + b * 64,
-                        crow);
-            tma_load_2d(sqh(stage) + b * kRows * 128u, &tm_hw, full_bar(stage), nc * p.N + b * 64,
-                        crow);
-          }
+          mbar_expect_tx_only(full_bar(warp), qbytes);
+          const int crow = it.t0 * kBM + kt * (int)kRows;
+          for (int b = 0; b < p.N / 64; ++b)
+            tma_load_2d(sq(warp) + b * kRows * 128u, tm, full_bar(warp), it.nc * p.N + b * 64, crow);
         }
-        // this quarter's row tokens: lane l holds row l (-1: padding)
-        const int rg = row_in_group + lane;
-        const int tk = rg < size ? p.row_tok[(size_t)g * p.region + rg] : -1;
+        // this step's row tokens: lane l holds rows l and 32 + l (-1: padding)
+        int tk[2];
 #pragma unroll
-        for (int kind = 0; kind < 2; ++kind) {
-          const uint32_t dst = kind == 0 ? spx(stage) : spy(stage);
-          const __nv_bfloat16* sj = (kind == 0 ? p.x : p.dy) + (size_t)c * 128 + j * 8;
+        for (int i = 0; i < 2; ++i) {
+          const int rg = it.r0 + kt * (int)kRows + 32 * i + lane;
+          tk[i] = rg < size ? p.row_tok[(size_t)it.g * p.region + rg] : -1;
+        }
+        const uint32_t dst = sp(warp);
 #pragma unroll
-          for (int b = 0; b < 2; ++b) {
+        for (int b = 0; b < 2; ++b) {
 #pragma unroll
-            for (int i = 0; i < (int)kRows / 4; ++i) {
-              const int r = 4 * i + rsub;
-              const int t = __shfl_sync(0xffffffffu, tk, r);
-              const uint32_t off = b * kRows * 128u + r * 128u + ((j ^ (r & 7)) << 4);
-              if (t >= 0)
-                cp_async16(dst + off, sj + (size_t)t * p.d + b * 64);
-              else  // padding rows contribute zeros to the row sums
-                *reinterpret_cast<uint4*>(gen_base + (dst - s0) + off) = make_uint4(0u, 0u, 0u, 0u);
-            }
+          for (int i = 0; i < (int)kRows / 4; ++i) {
+            const int r = 4 * i + rsub;
+            const int t = __shfl_sync(0xffffffffu, tk[i >> 3], r & 31);
+            const uint32_t off = b * kRows * 128u + r * 128u + ((j ^ (r & 7)) << 4);
+            if (t >= 0)
+              cp_async16(dst + off, sj + (size_t)t * p.d + b * 64);
+            else  // padding rows contribute zeros to the row sums
+              *reinterpret_cast<uint4*>(gen_base + (dst - s0) + off) = make_uint4(0u, 0u, 0u, 0u);
           }
         }
         cp_async_commit();
         cp_async_wait<0>();
         fence_proxy_async();
         __syncwarp();
-        if (lane == 0) mbar_arrive(full_bar(stage));
+        if (lane == 0) mbar_arrive(full_bar(warp));
       }
+      kt -= n_steps;  // stages count on over the items
     }
-  } else if (warp == kMmaWarp) {
+  } else if (warp == kWMma) {
     const uint32_t idesc = idesc_bf16_mn(kBM, p.N);
     const uint32_t lbo = kRows * 128u;  // 64-element MN blocks of kRows rows
-    int seq = 0;
-    uint32_t acc_phase = 0;
+    int s = 0, acc = 0;
+    uint32_t ph = 0, acc_ph = 0;
     bool ok = true;
     for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
-      int g, t_first, nt, r0, c, nc;
-      decode(item, g, t_first, nt, r0, c, nc);
-      ok = wait_warp(acce, acc_phase ^ 1u, abort_flag, p.status, p.wait_limit);
+      const int n_steps = decode(item).nt * kParts;
+      ok = wait_warp(acce_bar(acc), acc_ph ^ 1u, abort_flag, p.status, p.wait_limit);
       if (!ok) break;
       tc_fence_after();
-      for (int kt = 0; kt < nt * kQuarters; ++kt, ++seq) {
-        const int stage = seq % kWStages;
-        const uint32_t phase = (uint32_t)(seq / kWStages) & 1u;
-        ok = wait_warp(full_bar(stage), phase, abort_flag, p.status, p.wait_limit);
+      const uint32_t d_tmem = tmem_base + (uint32_t)acc * kAcc2;
+      for (int kt = 0; kt < n_steps; ++kt) {
+        ok = wait_warp(full_bar(s), ph, abort_flag, p.status, p.wait_limit);
         if (!ok) break;
         tc_fence_after();
         if (elect_one()) {
 #pragma unroll
-          for (int k = 0; k < (int)kRows / 16; ++k) {  // 16 rows (two 8-row groups) per MMA
-            const uint32_t acc = (kt | k) != 0 ? 1u : 0u;
-            umma_bf16(tmem_base, sw128_mn_desc(spx(stage) + k * 2048u, lbo),
-                      sw128_mn_desc(sqa(stage) + k * 2048u, lbo), idesc, acc);
-            umma_bf16(tmem_base + kAcc2, sw128_mn_desc(spy(stage) + k * 2048u, lbo),
-                      sw128_mn_desc(sqh(stage) + k * 2048u, lbo), idesc, acc);
-          }
-          umma_commit(empty_bar(stage));
+          for (int k = 0; k < (int)kRows / 16; ++k)  // 16 rows (two 8-row groups) per MMA
+            umma_bf16(d_tmem, sw128_mn_desc(sp(s) + k * 2048u, lbo),
+                      sw128_mn_desc(sq(s) + k * 2048u, lbo), idesc, (kt | k) != 0 ? 1u : 0u);
+          umma_commit(empty_bar(s));
+          if (kt == n_steps - 1) umma_commit(accf_bar(acc));
         }
         __syncwarp();
+        if (++s == n_st) { s = 0; ph ^= 1u; }
       }
-      if (!ok) break;
-      if (elect_one()) umma_commit(accf);
-      __syncwarp();
-      acc_phase ^= 1u;
+      if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
     }
-  } else if (warp >= kFirstEpiWarp) {
+  } else if (warp >= kWFirstEpi) {
     const int q = warp & 3;
-    const int half = (warp - kFirstEpiWarp) >> 2;
+    const int half = (warp - kWFirstEpi) >> 2;
     const int cols = p.N / 2;
-    uint32_t acc_phase = 0;
+    int acc = 0;
+    uint32_t acc_ph = 0;
     for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
-      int g, t_first, nt, r0, c, nc;
-      decode(item, g, t_first, nt, r0, c, nc);
-      const int e = g / p.B, blk = g % p.B;
-      const int i = c * 128 + q * 32 + lane;  // this thread's feature
-      const int h0 = blk * p.M + nc * p.N + half * cols;  // first channel of its columns
-      float* up_col = p.dw_up + ((size_t)e * p.H + h0) * p.d + i;   // dK_e[h][i], stride d per h
-      float* dn_row = p.dw_down + ((size_t)e * p.d + i) * p.H + h0;  // dV_e[i][h], contiguous
-      if (!wait_warp(accf, acc_phase, abort_flag, p.status, p.wait_limit)) break;
+      const Item it = decode(item);
+      const int e = it.g / p.B, blk = it.g % p.B;
+      const int i = it.c * 128 + q * 32 + lane;  // this thread's feature
+      const int h0 = blk * p.M + it.nc * p.N + half * cols;  // first channel of its columns
+      if (!wait_warp(accf_bar(acc), acc_ph, abort_flag, p.status, p.wait_limit)) break;
       tc_fence_after();
-      const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16) + half * cols;
+      const uint32_t t_row =
+          tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)acc * kAcc2 + half * cols;
       // the chunks of a group add their partial sums (the outputs start at zero)
-      for (int cc = 0; cc < cols; cc += 32) {
-        float v[32];
-        tmem_ld32(t_row + cc, v);
+      if (it.kind == 0) {  // dK_e[h][i]: a warp's lanes are 32 features of one h
+        float* col = p.dw_up + ((size_t)e * p.H + h0) * p.d + i;
+        for (int cc = 0; cc < cols; cc += 32) {
+          float v[32];
+          tmem_ld32(t_row + cc, v);
 #pragma unroll
-        for (int jj = 0; jj < 32; ++jj) atomicAdd(up_col + (size_t)(cc + jj) * p.d, v[jj]);
-        tmem_ld32(t_row + kAcc2 + cc, v);
+          for (int jj = 0; jj < 32; ++jj) atomicAdd(col + (size_t)(cc + jj) * p.d, v[jj]);
+        }
+      } else {  // dV_e[i][h]: a thread's columns are contiguous
+        float* row = p.dw_down + ((size_t)e * p.d + i) * p.H + h0;
+        for (int cc = 0; cc < cols; cc += 32) {
+          float v[32];
+          tmem_ld32(t_row + cc, v);
 #pragma unroll
-        for (int jj = 0; jj < 32; jj += 4)
-          atomicAdd(reinterpret_cast<float4*>(dn_row + cc + jj),
-                    make_float4(v[jj], v[jj + 1], v[jj + 2], v[jj + 3]));
+          for (int jj = 0; jj < 32; jj += 4)
+            atomicAdd(reinterpret_cast<float4*>(row + cc + jj),
+                      make_float4(v[jj], v[jj + 1], v[jj + 2], v[jj + 3]));
+        }
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(acce);
-      acc_phase ^= 1u;
+      if (lane == 0) mbar_arrive(acce_bar(acc));
+      if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
     }
   }
   __syncwarp();
   tc_fence_before();
   __syncthreads();
-  if (warp == kMmaWarp) {
+  if (warp == kWMma) {
     tc_fence_after();
     tmem_dealloc(tmem_base, kTmemCols);
   }
@@ -722,6 +764,7 @@ __global__ void __launch_bounds__(256)
 router_dz_kernel(int T, int K, float tau, int adaptive, const uint8_t* __restrict__ mask,
                  const float* __restrict__ alpha, const float* __restrict__ s,
                  const float* __restrict__ dwt, float* __restrict__ dz) {
+  grid_dep_wait();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= T) return;
   float z[KC];
@@ -732,13 +775,16 @@ router_dz_kernel(int T, int K, float tau, int adaptive, const uint8_t* __restric
     if (c <= K) o[c] = z[c];
 }
 
-// dx[t][8 f .. 8 f + 8) += sum_c dL/dz_c(t) W*^T[c][8 f .. 8 f + 8) for the
+// dx[t][8 f .. 8 f + 8) = sum_c dL/dz_c(t) W*^T[c][8 f .. 8 f + 8) for the
 // two tokens t = 2 p, 2 p + 1: a thread per (token pair, 8 features), so that
 // each W*^T load serves both tokens. W*^T is the router's first K+1 columns
-// as fp32 [K+1][d]; d % 128 == 0; padding tokens have dL/dz = 0 and keep dx.
+// as fp32 [K+1][d]; d % 128 == 0; padding tokens have dL/dz = 0 and get 0.
+// Runs before the experts' share is added, so that dx is neither zeroed
+// first nor read here.
 __global__ void __launch_bounds__(256)
 router_dx_kernel(int T, int K1, int d, const float* __restrict__ dz,
                  const float* __restrict__ wrT, float* __restrict__ dx) {
+  grid_dep_wait();
   const int per = d / 8;
   const int n = ((T + 1) / 2) * per;
   for (int it = blockIdx.x * blockDim.x + threadIdx.x; it < n; it += gridDim.x * blockDim.x) {
@@ -746,7 +792,6 @@ router_dx_kernel(int T, int K1, int d, const float* __restrict__ dz,
     const int ta = 2 * p, tb = min(2 * p + 1, T - 1);  // (tb == ta: the last odd token)
     float4* pa = reinterpret_cast<float4*>(dx + (size_t)ta * d + 8 * f8);
     float4* pb = reinterpret_cast<float4*>(dx + (size_t)tb * d + 8 * f8);
-    const float4 xa0 = pa[0], xa1 = pa[1], xb0 = pb[0], xb1 = pb[1];  // added at the end
     const float* za = dz + (size_t)ta * K1;
     const float* zb = dz + (size_t)tb * K1;
     float4 a0 = make_float4(0.f, 0.f, 0.f, 0.f), a1 = a0, b0 = a0, b1 = a0;
@@ -780,10 +825,6 @@ router_dx_kernel(int T, int K1, int d, const float* __restrict__ dz,
         b1.z = fmaf(v[k], w1[k].z, b1.z); b1.w = fmaf(v[k], w1[k].w, b1.w);
       }
     }
-    a0.x += xa0.x; a0.y += xa0.y; a0.z += xa0.z; a0.w += xa0.w;
-    a1.x += xa1.x; a1.y += xa1.y; a1.z += xa1.z; a1.w += xa1.w;
-    b0.x += xb0.x; b0.y += xb0.y; b0.z += xb0.z; b0.w += xb0.w;
-    b1.x += xb1.x; b1.y += xb1.y; b1.z += xb1.z; b1.w += xb1.w;
     pa[0] = a0;
     pa[1] = a1;
     if (tb != ta) {
@@ -809,6 +850,7 @@ router_dw_kernel(int T, int K1, int d, const uint8_t* __restrict__ mask,
                  float* __restrict__ dw_router, float* __restrict__ dbias) {
   __shared__ __align__(16) __nv_bfloat16 xs[32][128];
   __shared__ __align__(16) float zs[32][16];
+  grid_dep_wait();
   const int i0 = blockIdx.x * 128, c0 = blockIdx.z * 16;
   const int t_begin = blockIdx.y * kRwSlice, t_end = min(T, t_begin + kRwSlice);
   const int q = threadIdx.x & 63, g = threadIdx.x >> 6;
@@ -867,6 +909,7 @@ router_dw_kernel(int T, int K1, int d, const uint8_t* __restrict__ mask,
 // W*^T: the router's first K+1 columns (fp32 [d][Cp]) as [K+1][d].
 __global__ void router_transpose_kernel(int K1, int d, int Cp, const float* __restrict__ wr,
                                         float* __restrict__ wrT) {
+  grid_dep_wait();
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k < K1 * d) {
     const int c = k / d, i = k % d;
@@ -881,6 +924,7 @@ __global__ void router_transpose_kernel(int K1, int d, int Cp, const float* __re
 __global__ void __launch_bounds__(128)
 gram_kernel(int K1, int d, const float* __restrict__ wrT, float* __restrict__ A) {
   __shared__ float red[4];
+  grid_dep_wait();
   const int a = blockIdx.x / K1, b = blockIdx.x % K1;
   float g = 0.f;
   for (int i = threadIdx.x; i < d; i += blockDim.x)
@@ -896,6 +940,7 @@ __global__ void __launch_bounds__(256)
 diversity_grad_kernel(int K1, int d, const float* __restrict__ wrT, const float* __restrict__ A,
                       float lambda, float* __restrict__ dw_router, float* __restrict__ l_out) {
   __shared__ float red[8];
+  grid_dep_wait();
   float ss = 0.f;
   for (int k = threadIdx.x; k < K1 * K1; k += blockDim.x) ss = fmaf(A[k], A[k], ss);
 #pragma unroll
@@ -958,8 +1003,11 @@ int backward_setup(unif_moe_layer* L) {
          hidden_smem_bytes(L->up_bn, L->bwd_hidden_stages, L->G) > 232448)
     --L->bwd_hidden_stages;
   L->bwd_hidden_smem = hidden_smem_bytes(L->up_bn, L->bwd_hidden_stages, L->G);
-  L->bwd_wgrad_smem =
-      1024 + kWStages * wgrad_stage_bytes(L->up_bn) + 96 + 4 * (3 * (uint32_t)L->G + 2) + 16;
+  L->bwd_wgrad_stages = kWStages;
+  while (L->bwd_wgrad_stages > kWMinStages &&
+         wgrad_smem_bytes(L->up_bn, L->bwd_wgrad_stages, L->G) > 232448)
+    --L->bwd_wgrad_stages;
+  L->bwd_wgrad_smem = wgrad_smem_bytes(L->up_bn, L->bwd_wgrad_stages, L->G);
   if (L->bwd_hidden_smem > 232448 || L->bwd_wgrad_smem > 232448) {
     set_error("backward: shared memory for block width %d and %d groups exceeds 227 KB", L->M,
               L->G);
@@ -972,24 +1020,6 @@ int backward_setup(unif_moe_layer* L) {
     set_error("cudaFuncSetAttribute failed for the backward kernels");
     return UNIF_MOE_ERR_CUDA;
   }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(L->n_sm);
-  cfg.blockDim = dim3(kHThreads);
-  cfg.dynamicSmemBytes = L->bwd_hidden_smem;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = 2;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  int clusters = 0;
-  if (cudaOccupancyMaxActiveClusters(&clusters, bwd_hidden_kernel, &cfg) != cudaSuccess ||
-      clusters < 1) {
-    set_error("backward: no CTA pair fits on this device");
-    return UNIF_MOE_ERR_CUDA;
-  }
-  L->bwd_pairs = std::min(clusters, L->n_sm / 2);
   return UNIF_MOE_OK;
 }
 
@@ -1021,12 +1051,9 @@ int backward_run(unif_moe_layer* L, const void* x, const void* dy, int T, const 
       return UNIF_MOE_ERR_CUDA;                                                 \
     }                                                                           \
   } while (0)
-  CKB(cudaMemsetAsync(dx, 0, sizeof(float) * (size_t)T * L->d, s));
-  CKB(cudaMemsetAsync(w.dwt, 0, sizeof(float) * (size_t)T * K1, s));
-  CKB(cudaMemsetAsync(dw_router, 0, sizeof(float) * (size_t)L->d * K1, s));
-  if (dbias) CKB(cudaMemsetAsync(dbias, 0, sizeof(float) * K1, s));
-  // tile list of the forward's groups (sizes in grp_cnt, rows in the regions)
-  CKB(launch_tile_list_from(L, w.grp_cnt, s));
+  // tile list of the forward's groups (sizes in grp_cnt, rows in the regions);
+  // dL/dalpha and dL/ds start at zero
+  CKB(launch_tile_list_from(L, w.grp_cnt, w.dwt, (size_t)T * K1, s));
   // hidden gradients
   {
     HiddenParams p;
@@ -1035,13 +1062,17 @@ int backward_run(unif_moe_layer* L, const void* x, const void* dy, int T, const 
     p.x = static_cast<const __nv_bfloat16*>(x);
     p.dy = static_cast<const __nv_bfloat16*>(dy);
     p.dwt = w.dwt;
+    p.dw_up = reinterpret_cast<float4*>(dw_up); p.dw_down = reinterpret_cast<float4*>(dw_down);
+    p.w4 = (long long)K1 * L->H * L->d / 4;
+    p.dw_router = dw_router; p.n_wr = L->d * K1;
+    p.dbias = dbias; p.n_bias = dbias ? K1 : 0;
     p.n_sub = L->up_nsub; p.bn = L->up_bn; p.num_kb = L->d / tc::kBK;
     p.B = L->B; p.M = L->M; p.H = L->H; p.d = L->d; p.K1 = K1;
     p.stages = L->bwd_hidden_stages;
     p.status = w.status;
     p.wait_limit = gemm_wait_limit();
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(2 * L->bwd_pairs);
+    cfg.gridDim = dim3(L->n_sm / 2 * 2);  // a pair per two SMs
     cfg.blockDim = dim3(kHThreads);
     cfg.dynamicSmemBytes = L->bwd_hidden_smem;
     cfg.stream = s;
@@ -1055,11 +1086,24 @@ int backward_run(unif_moe_layer* L, const void* x, const void* dy, int T, const 
     CKB(cudaLaunchKernelEx(&cfg, bwd_hidden_kernel, L->tm_wup_half, L->tm_wdownT, L->tm_da_st,
                            L->tm_hw_st, p));
   }
+  // router: W*^T, then dL/dz and its share of dL/dx, which dL/dx starts from
+  CKB(launch_dependent(router_transpose_kernel, dim3((K1 * L->d + 255) / 256), dim3(256), 0, s, K1,
+                       L->d, L->router_cols_pad, static_cast<const float*>(L->wr), w.wrT));
+  {
+    const int adaptive = isnan(L->th.alpha_fixed) ? 1 : 0;
+    auto dz = K1 <= 16 ? router_dz_kernel<16>
+                       : (K1 <= 32 ? router_dz_kernel<32> : router_dz_kernel<65>);
+    CKB(launch_dependent(dz, dim3((T + 255) / 256), dim3(256), 0, s, T, L->K, L->tau, adaptive,
+                         mask, static_cast<const float*>(w.alpha), static_cast<const float*>(w.s),
+                         static_cast<const float*>(w.dwt), w.dz));
+    const int items = (T + 1) / 2 * (L->d / 8);
+    CKB(launch_dependent(router_dx_kernel, dim3(std::min((items + 255) / 256, 8 * L->n_sm)),
+                         dim3(256), 0, s, T, K1, L->d, static_cast<const float*>(w.dz),
+                         static_cast<const float*>(w.wrT), dx));
+  }
   // dL/dx from the experts: DA K_e (the down kernel on the transposed keys)
   CKB(launch_down_streaming(L, L->tm_da, L->tm_wupT, nullptr, dx, s));
   // dL/dK_e and dL/dV_e (chunks of each group's rows add their parts)
-  CKB(cudaMemsetAsync(dw_up, 0, sizeof(float) * (size_t)K1 * L->H * L->d, s));
-  CKB(cudaMemsetAsync(dw_down, 0, sizeof(float) * (size_t)K1 * L->H * L->d, s));
   {
     WgradParams p;
     p.counts = w.grp_cnt; p.row_tok = w.row_tok;
@@ -1068,43 +1112,23 @@ int backward_run(unif_moe_layer* L, const void* x, const void* dy, int T, const 
     p.dw_up = dw_up; p.dw_down = dw_down;
     p.G = L->G; p.region = L->region_rows; p.B = L->B; p.M = L->M; p.H = L->H; p.d = L->d;
     p.N = L->up_bn; p.n_nc = L->up_nsub; p.n_c = L->d / 128;
+    p.stages = L->bwd_wgrad_stages;
     p.status = w.status;
     p.wait_limit = gemm_wait_limit();
-    bwd_wgrad_kernel<<<L->n_sm, kThreads, L->bwd_wgrad_smem, s>>>(L->tm_da_q, L->tm_hw_q, p);
-    CKB(cudaGetLastError());
+    CKB(launch_dependent(bwd_wgrad_kernel, dim3(L->n_sm), dim3(kWThreads), L->bwd_wgrad_smem, s,
+                         L->tm_da_q, L->tm_hw_q, p));
   }
-  // router: W*^T, then dL/dz, its share of dL/dx, dL/dW* and dL/dbias
-  router_transpose_kernel<<<(K1 * L->d + 255) / 256, 256, 0, s>>>(K1, L->d, L->router_cols_pad,
-                                                                   L->wr, w.wrT);
-  CKB(cudaGetLastError());
-  {
-    const int adaptive = isnan(L->th.alpha_fixed) ? 1 : 0;
-    const int dz_blocks = (T + 255) / 256;
-    if (K1 <= 16)
-      router_dz_kernel<16><<<dz_blocks, 256, 0, s>>>(T, L->K, L->tau, adaptive, mask, w.alpha,
-                                                     w.s, w.dwt, w.dz);
-    else if (K1 <= 32)
-      router_dz_kernel<32><<<dz_blocks, 256, 0, s>>>(T, L->K, L->tau, adaptive, mask, w.alpha,
-                                                     w.s, w.dwt, w.dz);
-    else
-      router_dz_kernel<65><<<dz_blocks, 256, 0, s>>>(T, L->K, L->tau, adaptive, mask, w.alpha,
-                                                     w.s, w.dwt, w.dz);
-    CKB(cudaGetLastError());
-    const int items = (T + 1) / 2 * (L->d / 8);
-    router_dx_kernel<<<std::min((items + 255) / 256, 8 * L->n_sm), 256, 0, s>>>(T, K1, L->d,
-                                                                                 w.dz, w.wrT, dx);
-    CKB(cudaGetLastError());
-    router_dw_kernel<<<dim3(L->d / 128, (T + kRwSlice - 1) / kRwSlice, (K1 + 15) / 16), 256, 0,
-                       s>>>(T, K1, L->d, mask, static_cast<const __nv_bfloat16*>(x), w.dz,
-                            dw_router, dbias);
-    CKB(cudaGetLastError());
-  }
+  // dL/dW* and dL/dbias
+  CKB(launch_dependent(router_dw_kernel,
+                       dim3(L->d / 128, (T + kRwSlice - 1) / kRwSlice, (K1 + 15) / 16), dim3(256),
+                       0, s, T, K1, L->d, mask, static_cast<const __nv_bfloat16*>(x),
+                       static_cast<const float*>(w.dz), dw_router, dbias));
   if (lambda_div != 0.f || l_div) {
-    gram_kernel<<<K1 * K1, 128, 0, s>>>(K1, L->d, w.wrT, w.gram);
-    CKB(cudaGetLastError());
-    diversity_grad_kernel<<<(L->d * K1 + 255) / 256, 256, 0, s>>>(K1, L->d, w.wrT, w.gram,
-                                                                  lambda_div, dw_router, l_div);
-    CKB(cudaGetLastError());
+    CKB(launch_dependent(gram_kernel, dim3(K1 * K1), dim3(128), 0, s, K1, L->d,
+                         static_cast<const float*>(w.wrT), w.gram));
+    CKB(launch_dependent(diversity_grad_kernel, dim3((L->d * K1 + 255) / 256), dim3(256), 0, s, K1,
+                         L->d, static_cast<const float*>(w.wrT),
+                         static_cast<const float*>(w.gram), lambda_div, dw_router, l_div));
   }
 #undef CKB
   return UNIF_MOE_OK;

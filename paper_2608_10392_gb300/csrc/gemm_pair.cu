@@ -395,25 +395,7 @@ int gemm_pair_setup(unif_moe_layer* L) {
     set_error("setting up the pair up-projection kernel failed");
     return UNIF_MOE_ERR_CUDA;
   }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(L->n_sm);
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = L->pair_smem;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = 2;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  int clusters = 0;
-  if (cudaOccupancyMaxActiveClusters(&clusters, pair_up_kernel<true>, &cfg) != cudaSuccess) {
-    set_error("cudaOccupancyMaxActiveClusters failed for the pair up-projection kernel");
-    return UNIF_MOE_ERR_CUDA;
-  }
-  if (clusters > L->n_sm / 2) clusters = L->n_sm / 2;
-  L->pairs = clusters;
-  L->up_pair = clusters > 0;
+  L->up_pair = true;
   return UNIF_MOE_OK;
 }
 
@@ -433,7 +415,7 @@ cudaError_t launch_up_pair(unif_moe_layer* L, const void* x, bool scatter, cudaS
   p.status = L->ws.status;
   p.wait_limit = gemm_wait_limit();
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(2 * L->pairs);
+  cfg.gridDim = dim3(L->n_sm / 2 * 2);  // a pair per two SMs
   cfg.blockDim = dim3(tc::pair::kThreads);
   cfg.dynamicSmemBytes = L->pair_smem;
   cfg.stream = s;

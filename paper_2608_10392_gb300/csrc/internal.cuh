@@ -183,10 +183,10 @@ struct unif_moe_layer {
   int ws_down_bn = 0, ws_down_nsub = 0, down_slices = 1;
   CUtensorMap tm_wdown_ws;  // w_down slabs of ws_down_bn rows
   // Up projection on CTA pairs (where the slice does not fit): boxes of half
-  // a sub-tile's key rows, ring depth, shared memory, pairs launched.
+  // a sub-tile's key rows, ring depth, shared memory.
   bool up_pair = false;
   CUtensorMap tm_wup_half;
-  int pair_stages = 0, pairs = 0;
+  int pair_stages = 0;
   bool bundles = false;  // the bundled down projection's workspace is allocated
   int64_t h_rows = 0;    // rows of hbuf
   uint32_t pair_smem = 0;
@@ -203,10 +203,10 @@ struct unif_moe_layer {
   CUtensorMap tm_wupT;      // w_upT [(K+1) d][H], boxes of 64 x down_bn
   CUtensorMap tm_da;        // da [max_rows][M], boxes of 64 x 128 (dx GEMM A operand)
   CUtensorMap tm_da_st, tm_hw_st;  // da, hw, store boxes of 32 x 32 (64-byte swizzle)
-  CUtensorMap tm_da_q;      // da, boxes of 64 x 32 (weight-gradient operand)
-  CUtensorMap tm_hw_q;      // hw, boxes of 64 x 32
+  CUtensorMap tm_da_q;      // da, boxes of 64 x 64 (weight-gradient operand)
+  CUtensorMap tm_hw_q;      // hw, boxes of 64 x 64
   uint32_t bwd_hidden_smem = 0, bwd_wgrad_smem = 0;
-  int bwd_hidden_stages = 0, bwd_pairs = 0;  // ring depth and CTA pairs of the hidden kernel
+  int bwd_hidden_stages = 0, bwd_wgrad_stages = 0;  // ring depths
   // Pipelined host-buffer forwards (UNIF_MOE_FEATURE_HOST_IO): the handle's
   // copy streams, and per staging slot the events that order its reuse
   // (input landed, kernels done, output copied out).
@@ -241,8 +241,10 @@ cudaError_t launch_combine_residual(unif_moe_layer* L, const void* x, void* out,
                                     float eps, bool norm, int T, cudaStream_t s);
 // Tile list from the router's group sizes, for streaming grouped GEMMs.
 cudaError_t launch_tile_list(unif_moe_layer* L, cudaStream_t s);
-// The same from group sizes at `sizes` (the forward's, for the backward).
-cudaError_t launch_tile_list_from(unif_moe_layer* L, const int32_t* sizes, cudaStream_t s);
+// The same from group sizes at `sizes` (the forward's, for the backward), also
+// zeroing n_zero floats.
+cudaError_t launch_tile_list_from(unif_moe_layer* L, const int32_t* sizes, float* zero,
+                                  size_t n_zero, cudaStream_t s);
 cudaError_t launch_sort_affinities(unif_moe_layer* L, int T, int32_t* q, float* p,
                                    cudaStream_t s);
 int forward_chunks(int T);

@@ -494,9 +494,13 @@ scatter_kernel(const uint64_t* __restrict__ shr_o, const uint64_t* __restrict__ 
 // ---------------------------------------------------------------------------
 __global__ void tile_list_kernel(const int32_t* __restrict__ fill, int G, int region,
                                  int32_t* __restrict__ n_tiles, int32_t* __restrict__ tile_group,
-                                 int32_t* __restrict__ tile_row0, int32_t* __restrict__ tile_rows) {
+                                 int32_t* __restrict__ tile_row0, int32_t* __restrict__ tile_rows,
+                                 float* __restrict__ zero, size_t n_zero) {
   extern __shared__ int32_t tl_s[];  // [G + 1] first tiles, [G] sizes
   grid_dep_wait();  // the group sizes are final
+  for (size_t k = blockIdx.x * (size_t)blockDim.x + threadIdx.x; k < n_zero;
+       k += (size_t)gridDim.x * blockDim.x)
+    zero[k] = 0.f;
   for (int g = threadIdx.x; g < G; g += blockDim.x)
     tl_s[G + 1 + g] = min(__ldcg(fill + g), region);
   __syncthreads();
@@ -841,17 +845,19 @@ cudaError_t launch_sort_affinities(unif_moe_layer* L, int T, int32_t* q, float* 
 }
 
 cudaError_t launch_tile_list(unif_moe_layer* L, cudaStream_t s) {
-  return launch_tile_list_from(L, L->ws.grp_fill, s);
+  return launch_tile_list_from(L, L->ws.grp_fill, nullptr, 0, s);
 }
 
-cudaError_t launch_tile_list_from(unif_moe_layer* L, const int32_t* sizes, cudaStream_t s) {
+cudaError_t launch_tile_list_from(unif_moe_layer* L, const int32_t* sizes, float* zero,
+                                  size_t n_zero, cudaStream_t s) {
   Workspace& w = L->ws;
   // every CTA scans the group sizes for itself and writes its share of the
   // tiles; a thread per tile where 32 CTAs allow it
   const int grid = (int)std::min<int64_t>(32, (L->max_tiles + 255) / 256);
   return launch_dependent(tile_list_kernel, dim3(grid), dim3(256),
                           sizeof(int32_t) * (2 * (size_t)L->G + 1), s, sizes, L->G,
-                          L->region_rows, w.n_tiles, w.tile_group, w.tile_row0, w.tile_rows);
+                          L->region_rows, w.n_tiles, w.tile_group, w.tile_row0, w.tile_rows, zero,
+                          n_zero);
 }
 
 cudaError_t launch_layernorm(unif_moe_layer* L, const void* x, void* out, const uint8_t* mask,
