@@ -48,21 +48,22 @@ constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kAccStride = 256;  // TMEM columns per accumulator buffer
 constexpr int kMaxBN = 256;
 constexpr uint32_t kStageB = kMaxBN * kBK * 2;   // 32 KB
-constexpr int kStageRow = 36;                    // fp32 per staged row (32 + 4 pad, 16 B aligned)
 constexpr uint32_t kHStageRow = 80;              // bytes per staged h row (64 + 16 pad)
 
-// Per-kernel shared memory: the up kernel keeps 4 operand stages; the down
-// kernel keeps 3 and a per-warp 32 x 32 fp32 staging tile that turns its
-// row-per-thread accumulator into row-contiguous, coalesced atomic adds.
+// Per-kernel shared memory: 4 operand stages; the down kernels also a 32 x 32
+// fp32 tile per epilogue warp (128-byte rows, 16-byte chunk c of row r at
+// c ^ (r & 7)) that turns its row-per-thread accumulator into row-contiguous,
+// coalesced atomic adds. (Padded rows left room for 3 stages: 2,776 us per
+// forward of 65,536 tokens of d = 1024 against 2,700.)
 template <int MODE>
 struct Cfg {
-  static constexpr int kStages = MODE == 0 ? 4 : 3;
+  static constexpr int kStages = 4;
   // up: 32 rows x 32 bf16 per warp (80-byte rows); down: 32 rows x 32 fp32
-  static constexpr uint32_t kStaging =
-      MODE == 0 ? kEpiWarps * 32u * kHStageRow : kEpiWarps * 32u * kStageRow * 4u;
+  static constexpr uint32_t kStaging = MODE == 0 ? kEpiWarps * 32u * kHStageRow : kEpiWarps * 4096u;
   static constexpr uint32_t kTokens = MODE == 0 ? kProducerWarps * kBM * 4u : 0u;
   static constexpr size_t kSmem = 1024 + kStages * (kStageA + kStageB) + kStaging + kTokens + 256;
 };
+static_assert(Cfg<0>::kSmem <= 232448 && Cfg<1>::kSmem <= 232448, "shared memory of a CTA");
 
 struct Params {
   const int32_t* n_tiles;
@@ -378,26 +379,27 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         // y[tok] += w * acc: each thread scales its row, the warp stages 32 rows x
         // 32 columns in shared memory and adds them back row-contiguously (8 lanes
         // x 16 B per row, 4 rows per instruction).
-        float* stg = staging + (size_t)(warp - kFirstEpiWarp) * 32 * kStageRow;
+        float* stg = staging + (size_t)(warp - kFirstEpiWarp) * 1024;
         const int t = t_cur;
         const float wt = w_cur;
-        const int r_sub = lane >> 3, c_sub = (lane & 7) * 4;
+        const int r_sub = lane >> 3, chunk = lane & 7;
         for (int c = 0; c < cols; c += 32) {
           float v[32];
           tmem_ld32(t_row + c_begin + c, v);
 #pragma unroll
           for (int j = 0; j < 32; j += 4)
-            *reinterpret_cast<float4*>(stg + lane * kStageRow + j) =
+            *reinterpret_cast<float4*>(stg + lane * 32 + (((j >> 2) ^ (lane & 7)) << 2)) =
                 make_float4(wt * v[j], wt * v[j + 1], wt * v[j + 2], wt * v[j + 3]);
           __syncwarp();
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
             const int r = 4 * i + r_sub;
             const int tr = __shfl_sync(0xffffffffu, t, r);
-            const float4 val = *reinterpret_cast<const float4*>(stg + r * kStageRow + c_sub);
+            const float4 val =
+                *reinterpret_cast<const float4*>(stg + r * 32 + ((chunk ^ (r & 7)) << 2));
             if (tr >= 0)
               atomicAdd(reinterpret_cast<float4*>(p.y32 + (size_t)tr * p.d + ns * p.bn + c_begin +
-                                                  c + c_sub),
+                                                  c + 4 * chunk),
                         val);
           }
           __syncwarp();
