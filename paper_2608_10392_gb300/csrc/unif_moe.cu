@@ -659,6 +659,71 @@ static void* mapped_host(void* p) {
   return at.devicePointer;
 }
 
+// Whether p is page-locked host memory.
+static bool pinned_host(const void* p) {
+  cudaPointerAttributes at;
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return at.type == cudaMemoryTypeHost;
+}
+
+// The host-buffer forward in three parts of tokens (a quarter, a half, a
+// quarter), each a pass of its own: the later parts' inputs and the first
+// two's outputs move under the kernels, which a single pass leaves waiting
+// for the whole input and then storing the whole output over the link. Each
+// part costs its own router, launches and copy latencies, though (ViT-S
+// layer, us, one pass against three parts: 8,000 tokens 168 and 191, 12,608
+// 235 and 231, 16,000 286 and 254, 40,000 641 and 502), so it is taken from
+// kHostPartTokens on. x_host and out_host are pinned, out_dev is out_host's
+// device address; T <= pass_tokens.
+constexpr int kHostPartTokens = 14336;
+static int forward_host_parts(unif_moe_t L, const void* x_host, void* out_host, char* out_dev, int T,
+                              const uint8_t* mask_host, int32_t* b_dev, int32_t* k_dev,
+                              cudaStream_t s) {
+  unif::Workspace& w = L->ws;
+  const size_t row = elt_size(L) * (size_t)L->d;
+  const int cut[4] = {0, (T / 4 + 127) / 128 * 128, (T / 4 * 3 + 127) / 128 * 128, T};
+  const char* xh = static_cast<const char*>(x_host);
+  char* xd = static_cast<char*>(w.x_stage[0]);
+  char* od = static_cast<char*>(w.out_stage[0]);
+  // the first part's input on the caller's stream, the others' on the copy
+  // stream once that stream has done what came before this call
+  CK(cudaEventRecord(L->ev_comp[0], s));
+  CK(cudaStreamWaitEvent(L->copy_in, L->ev_comp[0], 0));
+  CK(cudaMemcpyAsync(xd, xh, (size_t)cut[1] * row, cudaMemcpyHostToDevice, s));
+  if (mask_host) CK(cudaMemcpyAsync(w.mask_stage[0], mask_host, (size_t)T, cudaMemcpyHostToDevice, s));
+  for (int i = 0; i < 3; ++i) {
+    const int t0 = cut[i], n = cut[i + 1] - t0;
+    const size_t off = (size_t)t0 * row;
+    if (i > 0) CK(cudaStreamWaitEvent(s, L->ev_in[i - 1], 0));
+    // the last part's output is stored by the combine itself
+    const int rc = forward_pass(L, xd + off, i == 2 ? out_dev + off : od + off, n, t0,
+                                mask_host ? w.mask_stage[0] + t0 : nullptr,
+                                b_dev ? b_dev + t0 : nullptr, k_dev ? k_dev + t0 : nullptr, s,
+                                nullptr, i == 2);
+    L->rec0 = 0;
+    if (rc != UNIF_MOE_OK) return rc;
+    if (i == 0)
+      for (int q = 0; q < 2; ++q) {
+        const size_t o = (size_t)cut[q + 1] * row;
+        CK(cudaMemcpyAsync(xd + o, xh + o, (size_t)(cut[q + 2] - cut[q + 1]) * row,
+                           cudaMemcpyHostToDevice, L->copy_in));
+        CK(cudaEventRecord(L->ev_in[q], L->copy_in));
+      }
+    if (i == 2) break;
+    CK(cudaEventRecord(L->ev_comp[i], s));
+    CK(cudaStreamWaitEvent(L->copy_out, L->ev_comp[i], 0));
+    CK(cudaMemcpyAsync(static_cast<char*>(out_host) + off, od + off, (size_t)n * row,
+                       cudaMemcpyDeviceToHost, L->copy_out));
+  }
+  CK(cudaEventRecord(L->ev_comp[0], s));
+  L->last_T = T;
+  L->last_pass_T = T;  // (the group table follows from the routing records)
+  return UNIF_MOE_OK;
+}
+
 int unif_moe_forward_host(unif_moe_t L, const void* x_host, void* out_host, int T,
                           const uint8_t* mask_host, int32_t* b_host, int32_t* k_host,
                           void* stream) {
@@ -683,14 +748,30 @@ int unif_moe_forward_host(unif_moe_t L, const void* x_host, void* out_host, int 
   // slot 0 may still be in use by pipelined forwards
   CK(cudaStreamSynchronize(L->copy_in));
   CK(cudaStreamSynchronize(L->copy_out));
-  CK(cudaMemcpyAsync(w.x_stage[0], x_host, xb, cudaMemcpyHostToDevice, s));
-  if (mask_host) CK(cudaMemcpyAsync(w.mask_stage[0], mask_host, (size_t)T, cudaMemcpyHostToDevice, s));
   // Outputs in pinned host memory that the device can address are written
   // there by the kernels themselves (the combine, the router), without a
   // staging buffer and a copy back.
   void* out_dev = mapped_host(out_host);
   int32_t* b_dev = static_cast<int32_t*>(mapped_host(b_host));
   int32_t* k_dev = static_cast<int32_t*>(mapped_host(k_host));
+  // In parts from kHostPartTokens on, where pinned buffers let the copies run
+  // beside the kernels, for layers whose group table follows from the routing
+  // records (the expert-tile FFN).
+  if (L->ffn_fused && T >= kHostPartTokens && T <= L->pass_tokens && out_dev &&
+      pinned_host(x_host) && (!b_host || b_dev) && (!k_host || k_dev)) {
+    // a failure leaves no copy of the caller's buffers in flight
+    const int rc = forward_host_parts(L, x_host, out_host, static_cast<char*>(out_dev), T,
+                                      mask_host, b_dev, k_dev, s);
+    const cudaError_t e1 = cudaStreamSynchronize(L->copy_in), e2 = cudaStreamSynchronize(s),
+                      e3 = cudaStreamSynchronize(L->copy_out);
+    if (rc != UNIF_MOE_OK) return rc;
+    CK(e1);
+    CK(e2);
+    CK(e3);
+    return UNIF_MOE_OK;
+  }
+  CK(cudaMemcpyAsync(w.x_stage[0], x_host, xb, cudaMemcpyHostToDevice, s));
+  if (mask_host) CK(cudaMemcpyAsync(w.mask_stage[0], mask_host, (size_t)T, cudaMemcpyHostToDevice, s));
   int rc = unif_moe_forward(L, w.x_stage[0], out_dev ? out_dev : w.out_stage[0], T,
                             mask_host ? w.mask_stage[0] : nullptr,
                             b_host ? (b_dev ? b_dev : w.b_stage[0]) : nullptr,

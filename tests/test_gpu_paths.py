@@ -120,3 +120,27 @@ def test_bundled_down_projection(shape, kw):
     assert (few.b == g.b[:200]).all() and (few.k == g.k[:200]).all()
     again = run_gpu(wl, layer=g.layer)
     assert np.abs(again.y - g.y).max() <= 2e-2 * np.abs(g.y).max()
+
+
+@pytest.mark.parametrize("T,masked", [(14335, False), (14336, True), (20011, False)])
+def test_host_forward_in_parts(T, masked):
+    """From 14,336 tokens on, a forward of pinned buffers runs in three parts:
+    outputs, counts, records and the group table as of one pass."""
+    s = small(tokens=T, n_experts=2, d_ff=256, **(dict(seq_len=50, min_len=1) if masked else {}))
+    wl = workloads.make_workload(s)
+    g = run_gpu(wl)
+    counts, offsets, tok, w = g.layer.groups()
+    out = torch.empty_like(wl.x).pin_memory()
+    b = torch.empty(T, dtype=torch.int32).pin_memory()
+    k = torch.empty(T, dtype=torch.int32).pin_memory()
+    mask = None if wl.mask is None else wl.mask.pin_memory()
+    for _ in range(2):  # both accumulators
+        out.fill_(7.0)
+        g.layer.forward_host(wl.x.pin_memory(), out, mask, b, k)
+        assert g.layer.sync_status() == 0
+        assert (b.numpy() == g.b).all() and (k.numpy() == g.k).all()
+        y = out.float().numpy()
+        assert np.abs(y - g.y).max() <= 2.0 ** -7 * np.abs(g.y).max()
+    again = g.layer.groups()
+    assert torch.equal(again[0], counts) and torch.equal(again[2], tok)
+    assert torch.equal(again[3], w)
