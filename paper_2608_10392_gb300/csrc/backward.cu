@@ -82,6 +82,17 @@ constexpr int kEpiWarps = 8;      // of the weight-gradient kernel
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kAcc2 = 256;   // TMEM column of the second accumulator
 
+// Most 128-row tiles of a group in one weight-gradient item, `total` tiles in
+// `parts` items each (features x channels x kinds) on `ctas` CTAs: as many as
+// leave every CTA two items, so that most groups are one chunk, whose sums
+// are stored instead of added into zeroed outputs. (ViT-S, 25 tiles per
+// group: chunks of at most 8 took 101 us, this 91; BERT-base, 5
+// tiles: 115 and 95, its 170 MB of gradients being more than L2 holds
+// between the clearing and the adds.)
+__device__ __forceinline__ int chunk_tiles(int total, int parts, int ctas) {
+  return max(8, (int)(((long long)total * parts + 2 * ctas - 1) / (2 * ctas)));
+}
+
 // ---------------------------------------------------------------------------
 // bwd_hidden_kernel: per 256-row tile of a group and N sub-tile, on a pair of
 // CTAs (tcgen05 cta_group::2, M = 256, 128 rows each), acc_a = X[rows]
@@ -110,13 +121,14 @@ struct HiddenParams {
   const __nv_bfloat16* dy;
   float* dwt;          // [T][K+1]
   // outputs that later kernels add into, zeroed here by the odd CTAs' MMA
-  // warps (which have no MMAs to issue): dw_up, dw_down (w4 float4 each),
-  // dw_router (n_wr floats), dbias (n_bias floats)
-  float4* dw_up;
-  float4* dw_down;
+  // warps (which have no MMAs to issue): dw_up and dw_down of the experts with
+  // a group that is no single weight-gradient chunk (w_parts items per chunk
+  // on w_ctas CTAs), dw_router (n_wr floats), dbias (n_bias floats)
+  float* dw_up;
+  float* dw_down;
   float* dw_router;
   float* dbias;
-  long long w4;
+  int w_parts, w_ctas;
   int n_wr, n_bias;
   int n_sub, bn, num_kb, B, M, H, d, K1, stages;
   int* status;
@@ -345,12 +357,26 @@ bwd_hidden_kernel(const __grid_constant__ CUtensorMap tm_wk, const __grid_consta
         reinterpret_cast<uint4*>(zeros)[k] = make_uint4(0u, 0u, 0u, 0u);
       fence_proxy_async();
       __syncwarp();
-      const long long bytes = 16 * p.w4;
-      for (long long k = (long long)kHZero * (32 * pair + lane); k < bytes;
-           k += (long long)kHZero * 32 * n_pairs) {
-        const uint32_t n = (uint32_t)min((long long)kHZero, bytes - k);
-        bulk_store(reinterpret_cast<uint8_t*>(p.dw_up) + k, smem_u32(zeros), n);
-        bulk_store(reinterpret_cast<uint8_t*>(p.dw_down) + k, smem_u32(zeros), n);
+      const int most = chunk_tiles(first128_s[p.G], p.w_parts, p.w_ctas);
+      const long long bytes = (long long)p.H * p.d * 4;  // of one expert's dK or dV
+      for (int e = 0; e < p.G / p.B; ++e) {
+        // an expert with a block whose group is empty or split is cleared
+        // whole (its other blocks are overwritten): its dV rows interleave
+        // the blocks, and clearing them block by block took 50 us more
+        bool clear = false;
+        for (int blk = lane; blk < p.B; blk += 32) {
+          const int nt = first128_s[e * p.B + blk + 1] - first128_s[e * p.B + blk];
+          clear |= nt == 0 || nt > most;
+        }
+        if (!__any_sync(0xffffffffu, clear)) continue;
+        uint8_t* up = reinterpret_cast<uint8_t*>(p.dw_up) + e * bytes;
+        uint8_t* dn = reinterpret_cast<uint8_t*>(p.dw_down) + e * bytes;
+        for (long long k = (long long)kHZero * (32 * pair + lane); k < bytes;
+             k += (long long)kHZero * 32 * n_pairs) {
+          const uint32_t n = (uint32_t)min((long long)kHZero, bytes - k);
+          bulk_store(up + k, smem_u32(zeros), n);
+          bulk_store(dn + k, smem_u32(zeros), n);
+        }
       }
       bulk_commit();
       for (int k = 32 * pair + lane; k < p.n_wr; k += 32 * n_pairs) p.dw_router[k] = 0.f;
@@ -456,16 +482,16 @@ bwd_hidden_kernel(const __grid_constant__ CUtensorMap tm_wk, const __grid_consta
 // The token rows are the reduction dimension, so both operands are MN-major:
 // the gathered rows (x, dy) and the TMA tiles (DA, HW) keep the 128-byte
 // swizzled row layout, read with MN-major descriptors. A group's tiles are
-// split evenly into chunks of at most kChunkTiles, whose partial sums are
-// added into the (zeroed) outputs.
+// one chunk, whose sums are stored, or split evenly into chunks of at most
+// chunk_tiles, whose partial sums are added into the (zeroed) outputs.
 // Roles: warps 0-4 fill the ring, a warp per stage (the gathered rows, and
 // the DA or HW tiles by TMA), warp 5 MMAs, warps 6-13 epilogue. The two
 // kinds are items of their own so that one accumulator leaves room in TMEM
 // for a second: an item's atomic adds run under the next one's MMAs. Bound
 // by the operand bytes out of L2 (40 KB per 64 rows of 192 channels).
 // Measured (both kinds in one item, accumulators not overlapped, four stages
-// of 32 rows before): ViT-S 12,608 tokens 117 -> 101 us, BERT-base (2,300
-// tokens) 130 -> 115.
+// of 32 rows before): ViT-S 12,608 tokens 117 -> 91 us, BERT-base (2,300
+// tokens) 130 -> 95.
 // ---------------------------------------------------------------------------
 struct WgradParams {
   const int32_t* counts;   // [G] group sizes (the forward's)
@@ -486,7 +512,6 @@ constexpr int kWMinStages = 2;
 constexpr int kWMma = 5, kWFirstEpi = 6;
 constexpr int kWThreads = 32 * (kWFirstEpi + kEpiWarps);  // 448
 constexpr int kParts = kBM / (int)kRows;         // stages per 128-row tile
-constexpr int kChunkTiles = 8;                   // most tiles of a group per work item
 
 __host__ __device__ constexpr uint32_t wgrad_stage_bytes(int N) {
   return kPBytes + (uint32_t)(N / 64) * kRows * 128u;
@@ -543,10 +568,11 @@ bwd_wgrad_kernel(const __grid_constant__ CUtensorMap tm_da, const __grid_constan
     tile_table(p.counts, p.G, p.region, lane, first_s, cnt_s);
     __syncwarp();
     // the first chunk of every group (chunk_s[G] = all chunks)
+    const int most = chunk_tiles(first_s[p.G], p.n_c * p.n_nc * 2, (int)gridDim.x);
     int carry = 0;
     for (int g0 = 0; g0 < p.G; g0 += 32) {
       const int g = g0 + lane;
-      const int nch = g < p.G ? (first_s[g + 1] - first_s[g] + kChunkTiles - 1) / kChunkTiles : 0;
+      const int nch = g < p.G ? (first_s[g + 1] - first_s[g] + most - 1) / most : 0;
       int inc = nch;
       for (int o = 1; o < 32; o <<= 1) {
         const int v = __shfl_up_sync(0xffffffffu, inc, o);
@@ -565,7 +591,7 @@ bwd_wgrad_kernel(const __grid_constant__ CUtensorMap tm_da, const __grid_constan
   const int n_items = chunk_s[p.G] * p.n_c * p.n_nc * 2;
   // item -> (group g, its tiles [t0, t0 + nt) of one chunk, feature chunk c,
   // N chunk nc, kind); rows of the chunk start at row r0 of the group
-  struct Item { int g, t0, nt, r0, c, nc, kind; };
+  struct Item { int g, t0, nt, r0, c, nc, kind; bool whole; };  // whole: the group's only chunk
   auto decode = [&](int item) {
     Item it;
     it.kind = item & 1;
@@ -585,6 +611,7 @@ bwd_wgrad_kernel(const __grid_constant__ CUtensorMap tm_da, const __grid_constan
     const int ta = tiles * k / nch;
     it.t0 = first_s[lo] + ta;
     it.nt = tiles * (k + 1) / nch - ta;
+    it.whole = nch == 1;
     it.r0 = ta * kBM;
     return it;
   };
@@ -674,6 +701,8 @@ bwd_wgrad_kernel(const __grid_constant__ CUtensorMap tm_da, const __grid_constan
     const int q = warp & 3;
     const int half = (warp - kWFirstEpi) >> 2;
     const int cols = p.N / 2;
+    // (the caller's buffer need only be 16-byte aligned)
+    const bool wide = (reinterpret_cast<uintptr_t>(p.dw_down) & 31u) == 0;
     int acc = 0;
     uint32_t acc_ph = 0;
     for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
@@ -685,24 +714,45 @@ bwd_wgrad_kernel(const __grid_constant__ CUtensorMap tm_da, const __grid_constan
       tc_fence_after();
       const uint32_t t_row =
           tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)acc * kAcc2 + half * cols;
-      // the chunks of a group add their partial sums (the outputs start at zero)
+      // a whole group's sums are stored; the chunks of a split one add theirs
+      // (those outputs start at zero)
       if (it.kind == 0) {  // dK_e[h][i]: a warp's lanes are 32 features of one h
         float* col = p.dw_up + ((size_t)e * p.H + h0) * p.d + i;
         for (int cc = 0; cc < cols; cc += 32) {
           float v[32];
           tmem_ld32(t_row + cc, v);
+          if (it.whole) {
 #pragma unroll
-          for (int jj = 0; jj < 32; ++jj) atomicAdd(col + (size_t)(cc + jj) * p.d, v[jj]);
+            for (int jj = 0; jj < 32; ++jj) col[(size_t)(cc + jj) * p.d] = v[jj];
+          } else {
+#pragma unroll
+            for (int jj = 0; jj < 32; ++jj) atomicAdd(col + (size_t)(cc + jj) * p.d, v[jj]);
+          }
         }
       } else {  // dV_e[i][h]: a thread's columns are contiguous
         float* row = p.dw_down + ((size_t)e * p.d + i) * p.H + h0;
         for (int cc = 0; cc < cols; cc += 32) {
           float v[32];
           tmem_ld32(t_row + cc, v);
+          if (it.whole && wide) {  // whole 32-byte sectors per lane
 #pragma unroll
-          for (int jj = 0; jj < 32; jj += 4)
-            atomicAdd(reinterpret_cast<float4*>(row + cc + jj),
-                      make_float4(v[jj], v[jj + 1], v[jj + 2], v[jj + 3]));
+            for (int jj = 0; jj < 32; jj += 8)
+              asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(
+                               row + cc + jj),
+                           "f"(v[jj]), "f"(v[jj + 1]), "f"(v[jj + 2]), "f"(v[jj + 3]),
+                           "f"(v[jj + 4]), "f"(v[jj + 5]), "f"(v[jj + 6]), "f"(v[jj + 7])
+                           : "memory");
+          } else if (it.whole) {
+#pragma unroll
+            for (int jj = 0; jj < 32; jj += 4)
+              *reinterpret_cast<float4*>(row + cc + jj) =
+                  make_float4(v[jj], v[jj + 1], v[jj + 2], v[jj + 3]);
+          } else {
+#pragma unroll
+            for (int jj = 0; jj < 32; jj += 4)
+              atomicAdd(reinterpret_cast<float4*>(row + cc + jj),
+                        make_float4(v[jj], v[jj + 1], v[jj + 2], v[jj + 3]));
+          }
         }
       }
       tc_fence_before();
@@ -1062,8 +1112,8 @@ int backward_run(unif_moe_layer* L, const void* x, const void* dy, int T, const 
     p.x = static_cast<const __nv_bfloat16*>(x);
     p.dy = static_cast<const __nv_bfloat16*>(dy);
     p.dwt = w.dwt;
-    p.dw_up = reinterpret_cast<float4*>(dw_up); p.dw_down = reinterpret_cast<float4*>(dw_down);
-    p.w4 = (long long)K1 * L->H * L->d / 4;
+    p.dw_up = dw_up; p.dw_down = dw_down;
+    p.w_parts = L->d / 128 * L->up_nsub * 2; p.w_ctas = L->n_sm;
     p.dw_router = dw_router; p.n_wr = L->d * K1;
     p.dbias = dbias; p.n_bias = dbias ? K1 : 0;
     p.n_sub = L->up_nsub; p.bn = L->up_bn; p.num_kb = L->d / tc::kBK;

@@ -144,3 +144,30 @@ def test_host_forward_in_parts(T, masked):
     again = g.layer.groups()
     assert torch.equal(again[0], counts) and torch.equal(again[2], tok)
     assert torch.equal(again[3], w)
+
+
+@pytest.mark.parametrize("kw", [
+    dict(tokens=3000, n_experts=2),                   # groups of more than one chunk: added
+    dict(tokens=900, n_experts=3, d_ff=768),          # single chunks: stored (M = 192)
+    dict(tokens=900, n_experts=3, alpha_fixed=1.0),   # empty groups: cleared
+    dict(tokens=1100, n_experts=2, d_model=768, d_ff=1536),  # two N chunks, six feature chunks
+])
+def test_weight_gradient_chunks(kw):
+    """Weight gradients of groups that are one chunk, several, or empty, the
+    buffers filled with NaN before: every entry is written."""
+    from test_gpu_backward import check, run_case
+    wl, got, ref, L = run_case(small(**kw))
+    check(wl, got, ref)
+    dev = torch.device("cuda")
+    x, dy = wl.x.to(dev), torch.ones_like(wl.x, device=dev)
+    a = L.backward(x, dy, want_bias=True)
+    # the same into buffers on 16-byte, not 32-byte boundaries
+    def odd(t):
+        flat = torch.full((t.numel() + 4,), float("nan"), device=dev)
+        return flat[4:].view(t.shape)
+    b = L.backward(x, dy, want_bias=True, out={k: odd(v) for k, v in a.items()})
+    torch.cuda.synchronize()
+    for k in ("dx", "dw_up", "dw_down", "dw_router", "dbias"):
+        assert torch.isfinite(b[k]).all(), k
+        # (two runs: fp32 sums in another order, of up to 3,000 terms)
+        assert (a[k] - b[k]).abs().max() <= 1e-4 * a[k].abs().max(), k
