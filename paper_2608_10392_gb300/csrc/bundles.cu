@@ -11,9 +11,14 @@
 // The tokens of equal (e, c, s) form a group whose rows go through the
 // |s| blocks of s as one reduction of |s| M channels, so that a token adds
 // one output row per bundle it touches (25.5 instead of 54.3 on ViT-B) and
-// no block is computed that it does not run. The price is smaller groups
-// (15 patterns per bundle), whose last 128-row tiles are partly padding:
-// bundles_apply.
+// no block is computed that it does not run: 378 -> 268 us, bound by the
+// operand bytes out of L2 and the reductions together (without the
+// reductions 194). Sharing each tile's h among a cluster of CTAs by TMA
+// multicast was slower (497 -> 525 us per forward: 138 of 152 SMs, in
+// lockstep), and so were contiguous runs of tiles per CTA (570: neighbouring
+// tiles at the same time keep an expert's values in L2). The price is smaller
+// groups (15 patterns per bundle), whose last 128-row tiles are partly
+// padding: bundles_apply.
 //
 // h keeps its rows of M channels: the tiles of all bundle groups are numbered
 // in units of 128 rows x M, |s| units per tile (one per block of s, in
@@ -191,12 +196,12 @@ __global__ void __launch_bounds__(kTilesThreads) bundle_tiles_kernel(TilesArgs a
 
 }  // namespace
 
-// Bundles can be used by a layer: whole bundles, tables that fit in shared
-// memory, list indexes within int32.
+// Bundles can be used by a layer: its up projection is the pair kernel's,
+// whole bundles, tables that fit in shared memory, list indexes within int32.
 bool bundles_fit(const unif_moe_layer* L) {
   const int64_t G = (int64_t)(L->K + 1) * (L->B / kBundle) * kPatterns;
-  return L->fused_group && !L->ffn_fused && !L->gemm_streaming && L->B % kBundle == 0 &&
-         G <= 4096 && G * L->region_rows < ((int64_t)1 << 31) &&
+  return L->fused_group && !L->ffn_fused && !L->gemm_streaming && up_ws_bytes(L) == 0 &&
+         L->B % kBundle == 0 && G <= 4096 && G * L->region_rows < ((int64_t)1 << 31) &&
          (int64_t)L->pass_tokens * (L->K + 1) * (L->B / kBundle) < ((int64_t)1 << 31) &&
          bundle_h_rows(L) < ((int64_t)1 << 31);
 }
@@ -219,13 +224,20 @@ int64_t bundle_max_tiles(const unif_moe_layer* L) {
   return rows / kTileRows + bundle_groups(L) + 1;
 }
 
-// A pass of T tokens bundles its rows where the groups are at least one tile
-// on average: T (1 + k) / (K + 1) tokens per expert over 15 patterns, k the
-// fixed count or else about K / 3. BUNDLE_MEASURED
+// A pass of T tokens bundles its rows where the groups hold at least M^2 / 500
+// tokens on average: T (1 + k) / (K + 1) tokens per expert over 15 patterns, k
+// the fixed count or else about K / 3. Narrow blocks gain most (an output
+// row per M channels of work), and small groups lose to padding. Measured, us
+// per forward without and with bundles: d = 768, K = 16, M = 192: 2,500
+// tokens (62 per group) 167 and 172, 4,000 228 and 203, 12,608 583 and 497;
+// with two experts per token 5,000 (59) 153 and 168, 12,608 288 and 250; K =
+// 10, M = 256: 4,000 (105) 163 and 149; K = 8, M = 384: 7,000 (190) 172 and
+// 177, 14,000 319 and 305; d = 1024, skewed, K = 32, M = 256: 6,000 (141) 412
+// and 415, 9,000 546 and 502; K = 12, M = 512: 20,000 (512) 414 and 420.
 bool bundles_apply(const unif_moe_layer* L, int T) {
   if (!L->bundles) return false;
   const double k = L->th.topk_fixed > 0 ? L->th.topk_fixed : L->K / 3.0;
-  return (double)T * (1.0 + k) >= (double)kTileRows * kPatterns * (L->K + 1);
+  return (double)T * (1.0 + k) * 500.0 >= (double)L->M * L->M * kPatterns * (L->K + 1);
 }
 
 cudaError_t bundles_setup(const unif_moe_layer* L) {

@@ -565,6 +565,24 @@ ws_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 }  // namespace ws
 }  // namespace tc
 
+// The weight-stationary kernels' table in shared memory (first tile and size
+// of every group, the tiles of one CTA's run), after the barriers.
+static uint64_t ws_table_bytes(const unif_moe_layer* L) {
+  const uint64_t per_cta = (uint64_t)((L->max_tiles + L->n_sm - 1) / L->n_sm);
+  return L->fused_group ? ((uint64_t)(2 * L->G + 1 + 3 * per_cta) * 4 + 15) / 16 * 16 : 0;
+}
+
+// Shared memory of the weight-stationary up projection of a bf16 layer, 0
+// where it does not apply.
+uint64_t up_ws_bytes(const unif_moe_layer* L) {
+  using namespace tc::ws;
+  int bn = 0, nsub = 0;
+  if (L->gemm_streaming || !tc::pick_split(L->M, &bn, &nsub) || nsub != 1) return 0;
+  const uint64_t slabs = (uint64_t)(L->d / tc::kBK);
+  const uint64_t smem = Cfg<0>::kFixed + slabs * (uint64_t)bn * tc::kBK * 2 + ws_table_bytes(L);
+  return slabs <= (uint64_t)kMaxSlabs && smem <= kMaxSmem ? smem : 0;
+}
+
 // Chooses the weight-stationary kernels where their shapes and shared memory
 // allow: the up projection needs the whole block width in one accumulator
 // (M <= 256); the down projection reuses each h tile across all output
@@ -574,15 +592,9 @@ int gemm_ws_setup(unif_moe_layer* L) {
   using namespace tc::ws;
   L->up_ws = L->down_ws = false;
   if (L->gemm_streaming) return UNIF_MOE_OK;
-  // the tile table (first tile and size of every group, the tiles of one
-  // CTA's run) follows the barriers
-  const uint64_t per_cta = (uint64_t)((L->max_tiles + L->n_sm - 1) / L->n_sm);
-  const uint64_t table =
-      L->fused_group ? ((uint64_t)(2 * L->G + 1 + 3 * per_cta) * 4 + 15) / 16 * 16 : 0;
-  const uint64_t up_slabs = (uint64_t)L->up_nsub * (L->d / tc::kBK);
-  const uint64_t up_smem =
-      Cfg<0>::kFixed + up_slabs * (uint64_t)L->up_bn * tc::kBK * 2 + table;
-  if (L->up_nsub == 1 && up_slabs <= (uint64_t)kMaxSlabs && up_smem <= kMaxSmem) {
+  const uint64_t table = ws_table_bytes(L);
+  const uint64_t up_smem = up_ws_bytes(L);
+  if (up_smem > 0) {
     if (cudaFuncSetAttribute(ws_gemm_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)up_smem) != cudaSuccess) {
       set_error("cudaFuncSetAttribute failed for the weight-stationary up kernel");

@@ -221,6 +221,10 @@ struct unif_moe_layer {
 
 namespace unif {
 
+namespace tc {
+bool pick_split(int n, int* bn, int* nsub);  // N sub-tiles of the tensor-core GEMMs
+}
+
 void set_error(const char* fmt, ...);
 
 // Load time.
@@ -256,6 +260,7 @@ int gemm_tc_setup(unif_moe_layer* L);  // tensor maps of weights and h; returns 
 cudaError_t launch_gemms_tc(unif_moe_layer* L, const void* x, int T, cudaEvent_t mid,
                             cudaStream_t s);
 cudaError_t launch_timeout_probe(unif_moe_layer* L, int timeout_us, cudaStream_t s);
+uint64_t up_ws_bytes(const unif_moe_layer* L);  // 0: no weight-stationary up projection
 int gemm_ws_setup(unif_moe_layer* L);  // picks the weight-stationary kernels where they fit
 cudaError_t launch_up_ws(unif_moe_layer* L, const void* x, cudaStream_t s);
 cudaError_t launch_down_ws(unif_moe_layer* L, cudaStream_t s);
