@@ -22,7 +22,8 @@
 //               must follow each step's copies waits for the later ones too,
 //               measured 1,200-1,800 cycles per step with four such warps.)
 //   warp 8      this CTA's half of the step's keys by TMA
-//   warp 9      TMEM allocation (both CTAs); MMA issue (even CTA)
+//   warp 9      TMEM allocation (both CTAs); MMA issue (even CTA); the tile
+//               list of a streaming down projection (odd CTAs)
 //   warps 10-17 epilogue: GeLU, bf16, h rows to device memory (warp w: TMEM
 //               lane quarter w % 4, one half of the columns)
 // The ring's full barriers are the even CTA's: the stage's owner warp of each
@@ -63,6 +64,11 @@ struct Params {
   __nv_bfloat16* h;        // [128-row tiles of all groups][M]
   int n_sub, bn, num_kb;   // N sub-tiles of bn columns, 64-deep steps
   int B, M, H, d, stages;
+  // the streaming down projection's tile list, written here (null: none)
+  int32_t* n_tiles;
+  int32_t* tile_group;
+  int32_t* tile_row0;
+  int32_t* tile_rows;
   // SCATTER: the place in h of every row (bundles.cu)
   const uint64_t* shr;     // [T] shared block sets
   const int32_t* dst;      // [T][K+1][B / kBundle]
@@ -284,6 +290,19 @@ pair_up_kernel(const __grid_constant__ CUtensorMap tmB, Params p) {
         __syncwarp();
         wait_settle(mma_done, 0u, p.wait_limit);
       }
+    } else if (p.n_tiles != nullptr) {
+      // the peer's MMA warp, which has no MMAs to issue, lists the 128-row
+      // tiles for the streaming down projection (a kernel of its own took
+      // 3.3 us of every forward)
+      const int nt = first128_s[p.G];
+      if (pair == 0 && lane == 0) *p.n_tiles = nt;
+      for (int k = 32 * pair + lane; k < nt; k += 32 * n_pairs) {
+        int g, row0, rows;
+        tile_lookup(k, first128_s, cnt_s, p.G, p.region, g, row0, rows);
+        p.tile_group[k] = g;
+        p.tile_row0[k] = row0;
+        p.tile_rows[k] = rows;
+      }
     }
     __syncwarp();
   } else {
@@ -410,6 +429,9 @@ cudaError_t launch_up_pair(unif_moe_layer* L, const void* x, bool scatter, cudaS
   p.n_sub = L->up_nsub; p.bn = L->up_bn; p.num_kb = L->d / tc::kBK;
   p.B = L->B; p.M = L->M; p.H = L->H; p.d = L->d;
   p.stages = L->pair_stages;
+  const bool list = !scatter && !L->down_ws;
+  p.n_tiles = list ? L->ws.n_tiles : nullptr;
+  p.tile_group = L->ws.tile_group; p.tile_row0 = L->ws.tile_row0; p.tile_rows = L->ws.tile_rows;
   p.shr = L->ws.shr_mask + L->rec0;
   p.dst = L->ws.bd_dst;
   p.status = L->ws.status;

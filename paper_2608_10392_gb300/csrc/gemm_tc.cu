@@ -728,7 +728,8 @@ int gemm_tc_setup(unif_moe_layer* L) {
       rc = UNIF_MOE_ERR_CUDA;
     }
   }
-  L->tile_list = L->fused_group && !L->ffn_fused && !((L->up_ws || L->up_pair) && L->down_ws);
+  // (the pair up projection writes the list itself)
+  L->tile_list = L->fused_group && !L->ffn_fused && !L->up_pair && !(L->up_ws && L->down_ws);
   return rc;
 }
 
