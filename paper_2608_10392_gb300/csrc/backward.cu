@@ -1040,6 +1040,8 @@ int backward_setup(unif_moe_layer* L) {
   if (!encode_bf16_map(&L->tm_wdownT, w.w_downT, L->d, E * L->H, tc::kBK, L->up_bn / 2, 128) ||
       !encode_bf16_map(&L->tm_wup_half, L->w_up, L->d, E * L->H, tc::kBK, L->up_bn / 2, 128) ||
       !encode_bf16_map(&L->tm_wupT, w.w_upT, L->H, E * L->d, tc::kBK, L->down_bn, 128) ||
+      (L->down_ws && !encode_bf16_map(&L->tm_wupT_ws, w.w_upT, L->H, E * L->d, tc::kBK,
+                                      (uint32_t)L->ws_down_bn, 128)) ||
       !encode_bf16_map(&L->tm_da, w.da, L->M, (uint64_t)L->max_rows, tc::kBK, tc::kBM, 128) ||
       !encode_bf16_map(&L->tm_da_st, w.da, L->M, (uint64_t)L->max_rows, 32, 32, 64) ||
       !encode_bf16_map(&L->tm_hw_st, w.hw, L->M, (uint64_t)L->max_rows, 32, 32, 64) ||
@@ -1152,7 +1154,12 @@ int backward_run(unif_moe_layer* L, const void* x, const void* dy, int T, const 
                          static_cast<const float*>(w.wrT), dx));
   }
   // dL/dx from the experts: DA K_e (the down kernel on the transposed keys)
-  CKB(launch_down_streaming(L, L->tm_da, L->tm_wupT, nullptr, dx, s));
+  // (weight-stationary where the forward's down projection is: ViT-S, 12,608
+  // tokens, 82 -> 71 us)
+  if (L->down_ws && T >= kWsTokens)
+    CKB(launch_down_ws_on(L, L->tm_da, L->tm_wupT_ws, dx, s));
+  else
+    CKB(launch_down_streaming(L, L->tm_da, L->tm_wupT, nullptr, dx, s));
   // dL/dK_e and dL/dV_e (chunks of each group's rows add their parts)
   {
     WgradParams p;

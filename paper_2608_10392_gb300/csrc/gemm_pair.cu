@@ -1,6 +1,6 @@
 // Up projection on CTA pairs (tcgen05 cta_group::2, M = 256) for bf16 layers
 // whose (expert, block) weight slice does not fit in shared memory (d = 768,
-// 1024): h[row] = GeLU(x[tok(row)] K_e[:, H_b]) over the router's groups
+// 1024), and for small passes of the others: h[row] = GeLU(x[tok(row)] K_e[:, H_b]) over the router's groups
 // (Eq. 16, inner part).
 //
 // What bounds it: operand bytes out of L2. The single-CTA streaming kernel
@@ -393,12 +393,12 @@ pair_up_kernel(const __grid_constant__ CUtensorMap tmB, Params p) {
 }  // namespace pair
 }  // namespace tc
 
-// Chooses the pair kernel for the up projection of layers that would stream
-// it: where the ring holds kMinStages stages beside the group tables.
+// Sets the pair kernel up for the up projection, where the ring holds
+// kMinStages stages beside the group tables.
 int gemm_pair_setup(unif_moe_layer* L) {
   using namespace tc::pair;
   L->up_pair = false;
-  if (!L->fused_group || L->up_ws || L->gemm_streaming || L->up_bn % 64 != 0) return UNIF_MOE_OK;
+  if (!L->fused_group || L->gemm_streaming || L->up_bn % 64 != 0) return UNIF_MOE_OK;
   const uint32_t fixed = smem_bytes(L->up_bn, 0, L->G);
   int stages = fixed < kMaxSmem ? (int)((kMaxSmem - fixed) / stage_bytes(L->up_bn)) : 0;
   if (stages > kMaxStages) stages = kMaxStages;
@@ -418,7 +418,8 @@ int gemm_pair_setup(unif_moe_layer* L) {
   return UNIF_MOE_OK;
 }
 
-cudaError_t launch_up_pair(unif_moe_layer* L, const void* x, bool scatter, cudaStream_t s) {
+cudaError_t launch_up_pair(unif_moe_layer* L, const void* x, bool list, bool scatter,
+                           cudaStream_t s) {
   tc::pair::Params p;
   p.fill = L->ws.grp_fill;
   p.G = L->G;
@@ -429,7 +430,6 @@ cudaError_t launch_up_pair(unif_moe_layer* L, const void* x, bool scatter, cudaS
   p.n_sub = L->up_nsub; p.bn = L->up_bn; p.num_kb = L->d / tc::kBK;
   p.B = L->B; p.M = L->M; p.H = L->H; p.d = L->d;
   p.stages = L->pair_stages;
-  const bool list = !scatter && !L->down_ws;
   p.n_tiles = list ? L->ws.n_tiles : nullptr;
   p.tile_group = L->ws.tile_group; p.tile_row0 = L->ws.tile_row0; p.tile_rows = L->ws.tile_rows;
   p.shr = L->ws.shr_mask + L->rec0;

@@ -728,8 +728,8 @@ int gemm_tc_setup(unif_moe_layer* L) {
       rc = UNIF_MOE_ERR_CUDA;
     }
   }
-  // (the pair up projection writes the list itself)
-  L->tile_list = L->fused_group && !L->ffn_fused && !L->up_pair && !(L->up_ws && L->down_ws);
+  // (the pair up projection writes the list itself; up_ws does not)
+  L->tile_list = needs_tile_list(L);
   return rc;
 }
 
@@ -754,10 +754,14 @@ cudaError_t launch_gemms_tc(unif_moe_layer* L, const void* x, int T, cudaEvent_t
   // up: N = M (block width), reduction over d
   p.n_sub = L->up_nsub; p.bn = L->up_bn; p.num_kb = L->d / tc::kBK;
   cudaError_t e;
-  if (L->up_ws) {
+  const bool bundled = bundles_apply(L, T);
+  // weight-stationary kernels: from kWsTokens on, or where nothing else
+  // numbers the tiles (up_pair lists them for the streaming down projection)
+  const bool ws = T >= kWsTokens || !L->up_pair;
+  if (L->up_ws && ws) {
     e = launch_up_ws(L, x, s);
   } else if (L->up_pair) {
-    e = launch_up_pair(L, x, bundles_apply(L, T), s);
+    e = launch_up_pair(L, x, !bundled && !(L->down_ws && ws), bundled, s);
   } else {
     e = launch_dependent(tc::grouped_gemm_kernel<0>, dim3(L->n_sm), dim3(tc::kThreads),
                          tc::Cfg<0>::kSmem, s, L->tm_h, L->tm_wup, p);
@@ -766,7 +770,7 @@ cudaError_t launch_gemms_tc(unif_moe_layer* L, const void* x, int T, cudaEvent_t
   if (mid) cudaEventRecord(mid, s);
   // down: N = d, reduction over the block's M channels (bundled: over the
   // blocks of each row's pattern)
-  if (bundles_apply(L, T)) {
+  if (bundled) {
     const Workspace& w = L->ws;
     p.n_tiles = w.bd_n_tiles; p.tile_group = w.bd_tile_group; p.tile_row0 = w.bd_tile_row0;
     p.tile_rows = w.bd_tile_rows; p.tile_unit = w.bd_tile_unit;
@@ -776,7 +780,7 @@ cudaError_t launch_gemms_tc(unif_moe_layer* L, const void* x, int T, cudaEvent_t
     return launch_dependent(tc::grouped_gemm_kernel<2>, dim3(L->n_sm), dim3(tc::kThreads),
                             tc::Cfg<2>::kSmem, s, L->tm_h, L->tm_wdown, p);
   }
-  if (L->down_ws) return launch_down_ws(L, s);
+  if (L->down_ws && ws) return launch_down_ws(L, s);
   p.n_sub = L->down_nsub; p.bn = L->down_bn; p.num_kb = L->M / tc::kBK;
   return launch_dependent(tc::grouped_gemm_kernel<1>, dim3(L->n_sm), dim3(tc::kThreads),
                           tc::Cfg<1>::kSmem, s, L->tm_h, L->tm_wdown, p);

@@ -80,7 +80,7 @@ struct Params {
   const int32_t* tile_row0;  // first row of each tile in row_tok / row_w
   const int32_t* tile_rows;  // rows of each tile that are not padding
   const int32_t* row_tok;
-  const float* row_w;
+  const float* row_w;      // null: every row's weight is 1
   int n_sub, bn, num_kb;
   int B, M, H, d;
   const __nv_bfloat16* x;
@@ -464,7 +464,7 @@ ws_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       tile_of(t_begin, gq, r0, n);
       if (q * 32 + lane < n) {
         t_nxt = p.row_tok[r0 + q * 32 + lane];
-        w_nxt = p.row_w[r0 + q * 32 + lane];
+        w_nxt = p.row_w ? p.row_w[r0 + q * 32 + lane] : 1.f;
       }
     }
     uint8_t* stg = staging + (size_t)(warp - kFirstEpiWarp) * 32 * Cfg<MODE>::kStageRowBytes;
@@ -477,7 +477,7 @@ ws_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       if (MODE == 1 && tile + 1 < t_end) {
         const int r = r0_nxt + q * 32 + lane;
         t_nxt = q * 32 + lane < n_nxt ? p.row_tok[r] : -1;
-        w_nxt = q * 32 + lane < n_nxt ? p.row_w[r] : 0.f;
+        w_nxt = q * 32 + lane < n_nxt ? (p.row_w ? p.row_w[r] : 1.f) : 0.f;
         if (tile + 2 < t_end) tile_of(tile + 2, gq, r0_nxt, n_nxt);
       }
       for (int ns = 0; ns < p.n_sub; ++ns) {
@@ -685,6 +685,21 @@ cudaError_t launch_down_ws(unif_moe_layer* L, cudaStream_t s) {
   p.n_slices = L->down_slices;
   return launch_dependent(tc::ws::ws_gemm_kernel<1>, dim3(L->n_sm), dim3(tc::ws::Cfg<1>::kThreads),
                           L->down_ws_smem, s, L->tm_h, L->tm_wdown_ws, p);
+}
+
+// The weight-stationary down projection on other operands (as
+// launch_down_streaming): out[tok] += A[row] B_e[H_b, :] over the groups of
+// the forward (sizes in grp_cnt), every row with weight 1.
+cudaError_t launch_down_ws_on(unif_moe_layer* L, const CUtensorMap& tmA, const CUtensorMap& tmB,
+                              float* out, cudaStream_t s) {
+  tc::ws::Params p = ws_params(L, nullptr);
+  p.fill = L->ws.grp_cnt;
+  p.row_w = nullptr;
+  p.y32 = out;
+  p.n_sub = L->ws_down_nsub; p.bn = L->ws_down_bn; p.num_kb = L->M / tc::kBK;
+  p.n_slices = L->down_slices;
+  return launch_dependent(tc::ws::ws_gemm_kernel<1>, dim3(L->n_sm), dim3(tc::ws::Cfg<1>::kThreads),
+                          L->down_ws_smem, s, tmA, tmB, p);
 }
 
 }  // namespace unif

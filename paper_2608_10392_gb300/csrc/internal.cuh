@@ -182,7 +182,7 @@ struct unif_moe_layer {
   // number of output column slices run as separate work items
   int ws_down_bn = 0, ws_down_nsub = 0, down_slices = 1;
   CUtensorMap tm_wdown_ws;  // w_down slabs of ws_down_bn rows
-  // Up projection on CTA pairs (where the slice does not fit): boxes of half
+  // Up projection on CTA pairs (where up_ws does not apply): boxes of half
   // a sub-tile's key rows, ring depth, shared memory.
   bool up_pair = false;
   CUtensorMap tm_wup_half;
@@ -201,6 +201,7 @@ struct unif_moe_layer {
   // backward: transposed weights and the per-row gradient buffers
   CUtensorMap tm_wdownT;    // w_downT [(K+1) H][d], boxes of 64 x up_bn / 2
   CUtensorMap tm_wupT;      // w_upT [(K+1) d][H], boxes of 64 x down_bn
+  CUtensorMap tm_wupT_ws;   // w_upT, boxes of 64 x ws_down_bn (where down_ws)
   CUtensorMap tm_da;        // da [max_rows][M], boxes of 64 x 128 (dx GEMM A operand)
   CUtensorMap tm_da_st, tm_hw_st;  // da, hw, store boxes of 32 x 32 (64-byte swizzle)
   CUtensorMap tm_da_q;      // da, boxes of 64 x 64 (weight-gradient operand)
@@ -220,6 +221,14 @@ struct unif_moe_layer {
 };
 
 namespace unif {
+
+// Whether a streaming GEMM needs the tile list of a kernel of its own: where
+// no pair kernel writes it, or the weight-stationary up projection runs
+// before a streaming down projection.
+inline bool needs_tile_list(const unif_moe_layer* L) {
+  if (!L->fused_group || L->ffn_fused) return false;
+  return L->up_ws ? !L->down_ws : !L->up_pair;
+}
 
 namespace tc {
 bool pick_split(int n, int* bn, int* nsub);  // N sub-tiles of the tensor-core GEMMs
@@ -260,12 +269,22 @@ int gemm_tc_setup(unif_moe_layer* L);  // tensor maps of weights and h; returns 
 cudaError_t launch_gemms_tc(unif_moe_layer* L, const void* x, int T, cudaEvent_t mid,
                             cudaStream_t s);
 cudaError_t launch_timeout_probe(unif_moe_layer* L, int timeout_us, cudaStream_t s);
+// The weight-stationary kernels take passes of at least this many tokens: with
+// fewer, a CTA has a tile or two per weight slice and loading the slice first
+// only delays it. (us with the pair and streaming kernels and with these:
+// ViT-S training step of 1,000 tokens 115 and 126, 3,500 186 and 193, 5,000
+// 236 and 230; ViT-B forward of 1,000 tokens 104 and 114.)
+constexpr int kWsTokens = 4096;
 uint64_t up_ws_bytes(const unif_moe_layer* L);  // 0: no weight-stationary up projection
 int gemm_ws_setup(unif_moe_layer* L);  // picks the weight-stationary kernels where they fit
 cudaError_t launch_up_ws(unif_moe_layer* L, const void* x, cudaStream_t s);
 cudaError_t launch_down_ws(unif_moe_layer* L, cudaStream_t s);
+cudaError_t launch_down_ws_on(unif_moe_layer* L, const CUtensorMap& tmA, const CUtensorMap& tmB,
+                              float* out, cudaStream_t s);
 int gemm_pair_setup(unif_moe_layer* L);  // picks the pair up projection where the slice streams
-cudaError_t launch_up_pair(unif_moe_layer* L, const void* x, bool scatter, cudaStream_t s);
+// list: also write the 128-row tile list; scatter: h rows to the bundles' places
+cudaError_t launch_up_pair(unif_moe_layer* L, const void* x, bool list, bool scatter,
+                           cudaStream_t s);
 // Bundled down projection (bundles.cu).
 bool bundles_fit(const unif_moe_layer* L);
 int bundle_groups(const unif_moe_layer* L);

@@ -352,7 +352,7 @@ int unif_moe_create_ex(unif_moe_t* out, int d_model, int d_ff, int n_experts, in
     // explicit EXPERT_TILE request fails instead
     if (rc != UNIF_MOE_OK && o.gemm_kernels == UNIF_MOE_GEMM_AUTO) {
       L->ffn_fused = false;
-      L->tile_list = L->fused_group && !L->up_pair && !(L->up_ws && L->down_ws);
+      L->tile_list = unif::needs_tile_list(L);
       cudaGetLastError();  // a failed attribute call must not surface at a later launch
       rc = UNIF_MOE_OK;
     }

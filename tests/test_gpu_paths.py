@@ -151,6 +151,7 @@ def test_host_forward_in_parts(T, masked):
     dict(tokens=900, n_experts=3, d_ff=768),          # single chunks: stored (M = 192)
     dict(tokens=900, n_experts=3, alpha_fixed=1.0),   # empty groups: cleared
     dict(tokens=1100, n_experts=2, d_model=768, d_ff=1536),  # two N chunks, six feature chunks
+    dict(tokens=4200, n_experts=2),                   # dL/dx by the weight-stationary kernel
 ])
 def test_weight_gradient_chunks(kw):
     """Weight gradients of groups that are one chunk, several, or empty, the
@@ -171,3 +172,17 @@ def test_weight_gradient_chunks(kw):
         assert torch.isfinite(b[k]).all(), k
         # (two runs: fp32 sums in another order, of up to 3,000 terms)
         assert (a[k] - b[k]).abs().max() <= 1e-4 * a[k].abs().max(), k
+
+
+@pytest.mark.parametrize("shape", [
+    dict(d_model=128, d_ff=512, n_blocks=4),   # both projections weight-stationary
+    dict(d_model=768, d_ff=768, n_blocks=4),   # the down projection alone, in column slices
+    dict(d_model=256, d_ff=1536, n_blocks=4),  # two sub-tiles per block: the up projection streams
+])
+@pytest.mark.parametrize("T", [4095, 4096, 4321])
+def test_grouped_kernels_around_the_weight_stationary_switch(shape, T):
+    """Below 4,096 tokens grouped layers run the pair and streaming kernels,
+    from there on the weight-stationary ones where they fit."""
+    wl = workloads.make_workload(small(tokens=T, n_experts=2, topk_fixed=1, **shape))
+    g = run_gpu(wl, gemm_kernels="grouped")
+    assert_parity(wl, g, compare(wl, g))
