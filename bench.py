@@ -523,7 +523,10 @@ def main():
     # affinities; b and k also to the caller) and, when it groups the pairs,
     # one (token, weight) row per pair; the permute writes those rows; the
     # combine reads the fp32 accumulator and writes the output
-    fused = layer.kernels_per_forward() <= 5 and s.dtype == "bf16"
+    fused = s.dtype == "bf16"
+    # six kernels of a bf16 layer: two of them group the down projection's
+    # rows by bundle after the router's own grouping
+    bundled = fused and layer.kernels_per_forward() == 6
     # (grouped by expert: one row per (token, expert), 1[b > 0] + k per token)
     n_rows_last = cb_last
     if expert_tile:
@@ -545,6 +548,7 @@ def main():
     stages = {
         "router": hbm_stage(stage_ms["router"], router_bytes),
         "permute": (hbm_stage(stage_ms["permute"], permute_bytes) if not fused else
+                    {"ms": stage_ms["permute"], "kernels": "bundle rows and tiles"} if bundled else
                     {"ms": 0.0, "fused_into": "router", "event_gap_ms": stage_ms["permute"]}),
         **({"ffn": {"ms": ffn_ms, "TFLOP/s": ach, "frac_of_burst_bf16": ach / peak_tf,
                     "kernel": "expert-tile FFN (both projections, rows grouped by expert)",
@@ -607,11 +611,10 @@ def main():
             "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
             "ms_per_step": statistics.fmean(e2e_ms),
             "kind": "unif_moe_forward_host, one synchronous call at a time, CUDA events"},
-        # (a norm-first sublayer adds its layer-normalisation kernel)
         # (a norm-first sublayer adds its layer-normalisation kernel; a
-        # training step the backward's seven kernels)
+        # training step the backward's ten kernels)
         "gpu_launches": (layer.kernels_per_forward() * n_pass + (args.sublayer == "pre") +
-                         (7 if args.train else 0)) * K,
+                         (10 if args.train else 0)) * K,
         "clocks": clocks,
     }
     if args.train:

@@ -209,8 +209,11 @@ UNIF_MOE_API int unif_moe_sublayer_forward(unif_moe_t h, const void* x_dev, void
  * residual_counts_host (each may be NULL), and synchronises `stream` before
  * returning. Host buffers should be pinned for asynchronous copies; output
  * buffers (out_host and the counts) in pinned host memory the device can
- * address are written by the kernels directly, with no copy back. The
- * staging buffers are allocated at create time (UNIF_MOE_FEATURE_HOST_IO;
+ * address are written by the kernels directly, with no copy back. Large
+ * batches of pinned buffers (layers with the expert-tile FFN) run in three
+ * parts of tokens, whose copies overlap one another's kernels on the handle's
+ * copy streams; results and records are those of one pass. The staging
+ * buffers are allocated at create time (UNIF_MOE_FEATURE_HOST_IO;
  * ERR_STATE on a handle created without it). */
 UNIF_MOE_API int unif_moe_forward_host(unif_moe_t h, const void* x_host, void* out_host, int T,
                           const uint8_t* token_mask_host, int32_t* shared_counts_host,
@@ -355,12 +358,15 @@ UNIF_MOE_API int64_t unif_moe_max_rows(unif_moe_t h);
  * in one pass; -1 for a NULL handle. */
 UNIF_MOE_API int unif_moe_pass_tokens(unif_moe_t h);
 
-/* Number of kernels one pass of unif_moe_forward launches (a forward of
- * T > 0 tokens runs ceil(T / unif_moe_pass_tokens) passes): 4 for bf16
- * layers whose router also groups the pairs (router, up projection, down
- * projection, combine), 5 when a streaming GEMM reads a tile list, else 6
- * (router, group scan, group scatter, up, down, combine). -1 for a NULL
- * handle. */
+/* Number of kernels a full pass (unif_moe_pass_tokens tokens) of
+ * unif_moe_forward launches (a forward of T > 0 tokens runs
+ * ceil(T / unif_moe_pass_tokens) passes): 3 with the expert-tile FFN (router,
+ * FFN, combine), 4 for other bf16 layers whose router also groups the pairs
+ * (router, up projection, down projection, combine), 5 when a streaming GEMM
+ * reads a tile list, 6 where the down projection's rows are bundled (router,
+ * bundle rows, bundle tiles, up, down, combine; smaller passes of such a layer
+ * launch 4) and for fp32 layers (router, group scan, group scatter, up, down,
+ * combine). -1 for a NULL handle. */
 UNIF_MOE_API int unif_moe_kernels_per_forward(unif_moe_t h);
 
 /* Waits for `stream`, then reads and clears the handle's device status word.

@@ -91,6 +91,27 @@ void free_all(unif_moe_layer* L) {
   if (L->copy_out) cudaStreamDestroy(L->copy_out);
 }
 
+// Takes a handle back to the unbundled down projection after an allocation for
+// the bundled one failed.
+void drop_bundles(unif_moe_layer* L) {
+  void** ptrs[] = {reinterpret_cast<void**>(&L->ws.bd_fill),
+                   reinterpret_cast<void**>(&L->ws.bd_row_tok),
+                   reinterpret_cast<void**>(&L->ws.bd_row_w),
+                   reinterpret_cast<void**>(&L->ws.bd_dst),
+                   reinterpret_cast<void**>(&L->ws.bd_n_tiles),
+                   reinterpret_cast<void**>(&L->ws.bd_tile_group),
+                   reinterpret_cast<void**>(&L->ws.bd_tile_row0),
+                   reinterpret_cast<void**>(&L->ws.bd_tile_rows),
+                   reinterpret_cast<void**>(&L->ws.bd_tile_unit)};
+  for (void** q : ptrs) {
+    if (*q) cudaFree(*q);
+    *q = nullptr;
+  }
+  L->bundles = false;
+  L->h_rows = L->max_rows;
+  cudaGetLastError();  // the failed allocation must not surface at a later launch
+}
+
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 size_t elt_size(const unif_moe_layer* L) { return L->dtype == UNIF_MOE_BF16 ? 2 : 4; }
@@ -252,9 +273,10 @@ int unif_moe_create_ex(unif_moe_t* out, int d_model, int d_ff, int n_experts, in
   ALLOC(w.row_tok, row_cap); ALLOC(w.row_w, row_cap);
   if (L->fused_group) ALLOC(w.grp_fill, (size_t)L->G);
   // wide layers' passes of many tokens: the down projection's rows bundled
-  // over four blocks, h in their layout
+  // over four blocks, h in their layout; without room for the tables (at most
+  // 1.4 GB) the layer keeps its unbundled kernels
   L->bundles = true;
-  L->bundles = dtype == UNIF_MOE_BF16 && unif::bundles_fit(L) &&
+  L->bundles = rc == UNIF_MOE_OK && dtype == UNIF_MOE_BF16 && unif::bundles_fit(L) &&
                unif::bundles_apply(L, L->pass_tokens);
   L->h_rows = L->max_rows;
   if (L->bundles) {
@@ -265,9 +287,17 @@ int unif_moe_create_ex(unif_moe_t* out, int d_model, int d_ff, int n_experts, in
     ALLOC(w.bd_dst, (size_t)L->pass_tokens * E * (n_blocks / unif::kBundle));
     ALLOC(w.bd_n_tiles, 1); ALLOC(w.bd_tile_group, nt); ALLOC(w.bd_tile_row0, nt);
     ALLOC(w.bd_tile_rows, nt); ALLOC(w.bd_tile_unit, nt);
+    if (rc != UNIF_MOE_OK) {
+      drop_bundles(L);
+      rc = UNIF_MOE_OK;
+    }
   }
   void* hb = nullptr;
   if (rc == UNIF_MOE_OK) rc = dalloc(reinterpret_cast<char**>(&hb), es * (size_t)L->h_rows * M);
+  if (rc != UNIF_MOE_OK && L->bundles) {  // h in the unbundled layout is smaller
+    drop_bundles(L);
+    rc = dalloc(reinterpret_cast<char**>(&hb), es * (size_t)L->h_rows * M);
+  }
   w.hbuf = hb;
   ALLOC(w.y32, (size_t)L->pass_tokens * d_model);
   if (L->ffn_fused) ALLOC(w.y32_b, (size_t)L->pass_tokens * d_model);
