@@ -4,8 +4,9 @@ import numpy as np
 import pytest
 import torch
 
+import oracle
 import workloads
-from gpu_helpers import assert_parity, compare, make_layer, run_gpu
+from gpu_helpers import assert_parity, compare, make_layer, oracle_routing, run_gpu
 
 pytestmark = pytest.mark.gpu
 
@@ -186,3 +187,26 @@ def test_grouped_kernels_around_the_weight_stationary_switch(shape, T):
     wl = workloads.make_workload(small(tokens=T, n_experts=2, topk_fixed=1, **shape))
     g = run_gpu(wl, gemm_kernels="grouped")
     assert_parity(wl, g, compare(wl, g))
+
+
+@pytest.mark.parametrize("K,B,T,kw", [
+    (16, 12, 1, dict()),                         # one token
+    (8, 16, 5003, dict()),                       # two chunks per CTA, a ragged last one
+    (15, 8, 12001, dict(topk_fixed=1)),          # three; 128 groups
+    (7, 20, 700, dict()),                        # more blocks than the unrolled loop takes
+    (2, 64, 300, dict(seq_len=100, min_len=1)),  # whole block masks, padding
+    (16, 16, 700, dict(alpha_fixed=0.0, topk_fixed=16)),  # more rows than fit: one by one
+])
+def test_router_rows_staged(K, B, T, kw):
+    """Group rows put together in shared memory (from 128 groups on): outputs,
+    and the group table against the decisions."""
+    wl = workloads.make_workload(small(tokens=T, d_ff=64 * B, n_experts=K, n_blocks=B, **kw))
+    g = run_gpu(wl, gemm_kernels="grouped")
+    assert_parity(wl, g, compare(wl, g))
+    counts, offsets, tok, w = (v.numpy() for v in g.layer.groups())
+    r = oracle.with_decisions(oracle_routing(wl), g.shr, g.em, B)
+    c_ref, tok_ref, w_ref = oracle.groups(r, K, B, *([] if wl.mask is None else [wl.mask.numpy()]))
+    assert counts.tolist() == c_ref.tolist()
+    real = tok >= 0
+    assert tok[real].tolist() == tok_ref.tolist()
+    np.testing.assert_allclose(w[real], w_ref, rtol=1e-5, atol=1e-7)
