@@ -79,8 +79,9 @@ struct Params {
   const __nv_bfloat16* x;  // up: tokens [T][d] (rows gathered with cp.async)
   __nv_bfloat16* h;  // up: [rows][M]
   float* y32;        // down: [T][d]
-  // bundled down projection: the tiles' first units of h, and the group
-  // counters to zero for the next pass
+  // bundled down projection: rows as (token, weight) pairs, the tiles' first
+  // units of h, and the group counters to zero for the next pass
+  const int2* rows;
   const int32_t* tile_unit;
   int32_t* bd_fill;
   int bd_groups;
@@ -323,12 +324,20 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     // down: this thread's row token and weight, fetched one tile ahead
     int t_nxt = -1;
     float w_nxt = 0.f;
-    // (row_w == nullptr: every row's weight is 1)
+    auto row_of = [&](int r, int& t, float& w) {
+      if (MODE == 2) {
+        const int2 v = p.rows[r];
+        t = v.x;
+        w = __int_as_float(v.y);
+      } else {  // (row_w == nullptr: every row's weight is 1)
+        t = p.row_tok[r];
+        w = p.row_w ? p.row_w[r] : 1.f;
+      }
+    };
     if (MODE >= 1 && blockIdx.x < n_items &&
         q * 32 + lane < p.tile_rows[blockIdx.x / p.n_sub]) {
       const int r = p.tile_row0[blockIdx.x / p.n_sub] + q * 32 + lane;
-      t_nxt = p.row_tok[r];
-      w_nxt = p.row_w ? p.row_w[r] : 1.f;
+      row_of(r, t_nxt, w_nxt);
     }
     for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
       const int tile = item / p.n_sub, ns = item % p.n_sub;
@@ -339,8 +348,9 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         const int nt = (item + gridDim.x) / p.n_sub;
         const int r = p.tile_row0[nt] + q * 32 + lane;
         const bool real = q * 32 + lane < p.tile_rows[nt];
-        t_nxt = real ? p.row_tok[r] : -1;
-        w_nxt = real ? (p.row_w ? p.row_w[r] : 1.f) : 0.f;
+        t_nxt = -1;
+        w_nxt = 0.f;
+        if (real) row_of(r, t_nxt, w_nxt);
       }
       if (!wait_warp(accf_bar(acc), acc_phase, abort_flag, p.status, p.wait_limit)) break;
       tc_fence_after();
@@ -781,7 +791,7 @@ cudaError_t launch_gemms_tc(unif_moe_layer* L, const void* x, int T, cudaEvent_t
     const Workspace& w = L->ws;
     p.n_tiles = w.bd_n_tiles; p.tile_group = w.bd_tile_group; p.tile_row0 = w.bd_tile_row0;
     p.tile_rows = w.bd_tile_rows; p.tile_unit = w.bd_tile_unit;
-    p.row_tok = w.bd_row_tok; p.row_w = w.bd_row_w;
+    p.rows = w.bd_rows;
     p.bd_fill = w.bd_fill; p.bd_groups = bundle_groups(L);
     p.n_sub = L->down_nsub; p.bn = L->down_bn; p.num_kb = L->M / tc::kBK;
     return launch_dependent(tc::grouped_gemm_kernel<2>, dim3(L->n_sm), dim3(tc::kThreads),

@@ -90,8 +90,7 @@ struct Workspace {
   void* wv_slabs = nullptr;      // V_e: [K+1][H/128][2][d/128] slabs
   // Down-projection rows bundled over four blocks (bundles.cu), G2 groups.
   int32_t* bd_fill = nullptr;       // [G2] rows per group, 0 between passes
-  int32_t* bd_row_tok = nullptr;    // [G2][region]
-  float* bd_row_w = nullptr;        // same layout
+  int2* bd_rows = nullptr;          // [G2][region] (token, bits of the fp32 weight)
   int32_t* bd_dst = nullptr;        // [pass_tokens][K+1][B/4] h row of the bundle's first block
   int32_t* bd_n_tiles = nullptr;    // [1]
   int32_t* bd_tile_group = nullptr; // per 128-row tile: group, first list row, real rows,

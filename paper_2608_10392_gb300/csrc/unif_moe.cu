@@ -77,7 +77,7 @@ void free_all(unif_moe_layer* L) {
                   L->ws.dwt, L->ws.dz, L->ws.wrT, L->ws.gram, L->ws.diag_sets,
                   L->ws.diag_counts, L->ws.diag_pair, L->ws.diag_wts, L->ws.diag_q,
                   L->ws.diag_E, L->ws.diag_ES, L->ws.wk_slabs, L->ws.wv_slabs, L->ws.y32_b,
-                  L->ws.bd_fill, L->ws.bd_row_tok, L->ws.bd_row_w, L->ws.bd_dst,
+                  L->ws.bd_fill, L->ws.bd_rows, L->ws.bd_dst,
                   L->ws.bd_n_tiles, L->ws.bd_tile_group, L->ws.bd_tile_row0,
                   L->ws.bd_tile_rows, L->ws.bd_tile_unit};
   for (void* q : ptrs)
@@ -95,8 +95,7 @@ void free_all(unif_moe_layer* L) {
 // the bundled one failed.
 void drop_bundles(unif_moe_layer* L) {
   void** ptrs[] = {reinterpret_cast<void**>(&L->ws.bd_fill),
-                   reinterpret_cast<void**>(&L->ws.bd_row_tok),
-                   reinterpret_cast<void**>(&L->ws.bd_row_w),
+                   reinterpret_cast<void**>(&L->ws.bd_rows),
                    reinterpret_cast<void**>(&L->ws.bd_dst),
                    reinterpret_cast<void**>(&L->ws.bd_n_tiles),
                    reinterpret_cast<void**>(&L->ws.bd_tile_group),
@@ -283,7 +282,7 @@ int unif_moe_create_ex(unif_moe_t* out, int d_model, int d_ff, int n_experts, in
     const size_t G2 = (size_t)unif::bundle_groups(L), nt = (size_t)unif::bundle_max_tiles(L);
     L->h_rows = std::max(L->h_rows, unif::bundle_h_rows(L));
     ALLOC(w.bd_fill, G2);
-    ALLOC(w.bd_row_tok, G2 * L->region_rows); ALLOC(w.bd_row_w, G2 * L->region_rows);
+    ALLOC(w.bd_rows, G2 * L->region_rows);
     ALLOC(w.bd_dst, (size_t)L->pass_tokens * E * (n_blocks / unif::kBundle));
     ALLOC(w.bd_n_tiles, 1); ALLOC(w.bd_tile_group, nt); ALLOC(w.bd_tile_row0, nt);
     ALLOC(w.bd_tile_rows, nt); ALLOC(w.bd_tile_unit, nt);
