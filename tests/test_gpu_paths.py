@@ -66,6 +66,16 @@ def test_decisions_of_tokens_that_are_not_finite(K):
     assert (bad.shr[keep] == clean.shr[keep]).all() and (bad.em[keep] == clean.em[keep]).all()
 
 
+@pytest.mark.parametrize("K", [5, 8, 12, 16, 32])
+def test_equal_affinities_go_to_the_lower_expert(K):
+    """A zero token's logits are all equal: the first experts are its own."""
+    wl = workloads.make_workload(small(n_experts=K, topk_fixed=3))
+    x = wl.x.clone()
+    x[11] = 0
+    g = run_gpu(wl, x=x)
+    assert g.k[11] == 3 and int(g.em[11]) == 0b111
+
+
 @pytest.mark.parametrize("T", [152 * 128, 152 * 128 + 1, 40001])
 def test_router_two_ctas_per_sm(T):
     """One wave of 128-token router CTAs, one token more, and a ragged count
