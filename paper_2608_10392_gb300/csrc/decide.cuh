@@ -157,9 +157,10 @@ __device__ __forceinline__ void store_affinities(float* dst, const float (&e)[KC
 // of decide_token_rt. For KC > 8 the experts are taken one at a time, largest
 // first, until their mass reaches beta: k steps over the K experts in place
 // of K^2 comparisons (two passes of 32,768 tokens, K = 32: 18 us less), each
-// found by a tree of comparisons of integer keys (another 26 us less than one
-// logit after the other; K = 16, 12,608 tokens: 1.5). The mass of the experts
-// taken is summed in index order, as there. Logits that are not finite numbers
+// found by a tree of comparisons of integer keys (one logit after the other
+// before: 1,500 tokens, d = 1024, K = 32 252.9 -> 250.8 us per forward, 3,000
+// of K = 16 99.0 -> 98.5). The mass of the experts taken is summed in index
+// order, as there. Logits that are not finite numbers
 // (the softmax's sum is then NaN) are left to decide_token_rt (returns false).
 template <int KC, int BC, bool EXACT>
 __device__ __forceinline__ bool decide_token_ct(const DecideArgs& a, int t, bool valid, float* z,
