@@ -1065,10 +1065,8 @@ int backward_setup(unif_moe_layer* L) {
               L->G);
     return UNIF_MOE_ERR_SHAPE;
   }
-  if (cudaFuncSetAttribute(bwd_hidden_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)L->bwd_hidden_smem) != cudaSuccess ||
-      cudaFuncSetAttribute(bwd_wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)L->bwd_wgrad_smem) != cudaSuccess ) {
+  if (allow_smem(bwd_hidden_kernel, L->bwd_hidden_smem) != cudaSuccess ||
+      allow_smem(bwd_wgrad_kernel, L->bwd_wgrad_smem) != cudaSuccess) {
     set_error("cudaFuncSetAttribute failed for the backward kernels");
     return UNIF_MOE_ERR_CUDA;
   }

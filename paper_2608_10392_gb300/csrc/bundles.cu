@@ -262,8 +262,7 @@ bool bundles_apply(const unif_moe_layer* L, int T) {
 }
 
 cudaError_t bundles_setup(const unif_moe_layer* L) {
-  return cudaFuncSetAttribute(bundle_tiles_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (3 * bundle_groups(L) + 1) * (int)sizeof(int32_t));
+  return allow_smem(bundle_tiles_kernel, (3 * bundle_groups(L) + 1) * sizeof(int32_t));
 }
 
 cudaError_t launch_bundles(unif_moe_layer* L, int T, cudaStream_t s) {

@@ -788,8 +788,7 @@ int gemm_fused_setup(unif_moe_layer* L) {
   }
   L->ffn_slots = slots;
   L->ffn_smem = smem_bytes(num_kb, slots, G, per_pair_guess);
-  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)L->ffn_smem) != cudaSuccess ||
+  if (allow_smem(kernel, L->ffn_smem) != cudaSuccess ||
       cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 0) !=
           cudaSuccess) {
     set_error("cudaFuncSetAttribute failed for the expert-tile FFN kernel");
@@ -827,8 +826,7 @@ int gemm_fused_setup(unif_moe_layer* L) {
                 L->ffn_per_cta);
       return UNIF_MOE_ERR_SHAPE;
     }
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)L->ffn_smem) != cudaSuccess) {
+    if (allow_smem(kernel, L->ffn_smem) != cudaSuccess) {
       set_error("cudaFuncSetAttribute failed for the expert-tile FFN kernel");
       return UNIF_MOE_ERR_CUDA;
     }

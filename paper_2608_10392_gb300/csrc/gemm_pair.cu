@@ -407,10 +407,8 @@ int gemm_pair_setup(unif_moe_layer* L) {
   L->pair_smem = smem_bytes(L->up_bn, stages, L->G);
   if (!encode_bf16_map(&L->tm_wup_half, L->w_up, L->d, (uint64_t)(L->K + 1) * L->H, tc::kBK,
                        (uint32_t)L->up_bn / 2, 128) ||
-      cudaFuncSetAttribute(pair_up_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)L->pair_smem) != cudaSuccess ||
-      cudaFuncSetAttribute(pair_up_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)L->pair_smem) != cudaSuccess) {
+      allow_smem(pair_up_kernel<false>, L->pair_smem) != cudaSuccess ||
+      allow_smem(pair_up_kernel<true>, L->pair_smem) != cudaSuccess) {
     set_error("setting up the pair up-projection kernel failed");
     return UNIF_MOE_ERR_CUDA;
   }

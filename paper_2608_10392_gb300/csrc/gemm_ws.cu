@@ -595,8 +595,7 @@ int gemm_ws_setup(unif_moe_layer* L) {
   const uint64_t table = ws_table_bytes(L);
   const uint64_t up_smem = up_ws_bytes(L);
   if (up_smem > 0) {
-    if (cudaFuncSetAttribute(ws_gemm_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)up_smem) != cudaSuccess) {
+    if (allow_smem(ws_gemm_kernel<0>, up_smem) != cudaSuccess) {
       set_error("cudaFuncSetAttribute failed for the weight-stationary up kernel");
       return UNIF_MOE_ERR_CUDA;
     }
@@ -635,8 +634,7 @@ int gemm_ws_setup(unif_moe_layer* L) {
     }
   }
   if (bn > 0) {
-    if (cudaFuncSetAttribute(ws_gemm_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem) != cudaSuccess) {
+    if (allow_smem(ws_gemm_kernel<1>, smem) != cudaSuccess) {
       set_error("cudaFuncSetAttribute failed for the weight-stationary down kernel");
       return UNIF_MOE_ERR_CUDA;
     }

@@ -235,6 +235,17 @@ bool pick_split(int n, int* bn, int* nsub);  // N sub-tiles of the tensor-core G
 
 void set_error(const char* fmt, ...);
 
+// Lets kernel `fn` be launched with `need` bytes of dynamic shared memory. The
+// limit belongs to the kernel, not to a handle, and the value set last holds
+// for all launches: it is always the most that the device allows beside the
+// kernel's static shared memory, so that handles of different shapes leave one
+// another's launches alone. An error where `need` is above that.
+cudaError_t allow_smem(const void* fn, size_t need);
+template <typename... P>
+cudaError_t allow_smem(void (*fn)(P...), size_t need) {
+  return allow_smem(reinterpret_cast<const void*>(fn), need);
+}
+
 // Load time.
 cudaError_t launch_prototypes(unif_moe_layer* L, const void* w_router, const float* bias,
                               cudaStream_t s);

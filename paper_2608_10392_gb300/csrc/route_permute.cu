@@ -817,11 +817,9 @@ static size_t scatter_smem(const unif_moe_layer* L) {
 }
 
 cudaError_t router_setup(unif_moe_layer* L) {
-  cudaError_t e = cudaFuncSetAttribute(router_entry(L), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)router_smem(L));
+  const cudaError_t e = allow_smem(router_entry(L), router_smem(L));
   if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(group_scatter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)scatter_smem(L));
+  return allow_smem(group_scatter_kernel, scatter_smem(L));
 }
 
 cudaError_t launch_permute(unif_moe_layer* L, int T, cudaStream_t s) {

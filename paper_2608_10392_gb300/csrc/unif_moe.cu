@@ -26,6 +26,19 @@ void set_error(const char* fmt, ...) {
   va_end(ap);
 }
 
+cudaError_t allow_smem(const void* fn, size_t need) {
+  cudaFuncAttributes at;
+  int dev = 0, most = 0;
+  cudaError_t e = cudaFuncGetAttributes(&at, fn);
+  if (e == cudaSuccess) e = cudaGetDevice(&dev);
+  if (e == cudaSuccess)
+    e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e != cudaSuccess) return e;
+  most -= (int)at.sharedSizeBytes;
+  if (most < 0 || need > (size_t)most) return cudaErrorInvalidValue;
+  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+}
+
 }  // namespace unif
 
 using unif::set_error;
