@@ -36,26 +36,16 @@ namespace unif {
 namespace tc {
 namespace bwd {
 
-// GeLU (exact erf form, Sec. II-A) and its derivative Phi(a) + a phi(a). Phi
-// from the erf approximation 7.1.26 of Abramowitz and Stegun (Handbook of
-// Mathematical Functions, 1964): erfc(z) = (b1 t + ... + b5 t^5) exp(-z^2),
-// t = 1 / (1 + p z), z >= 0, error at most 1.5e-7; with z = |a| / sqrt 2 its
-// exponential is the one that phi needs, so one value takes about 17
-// instructions in place of the 45 that erff and the exponential took. (The
-// same in packed fp32x2 arithmetic ran 8 us slower per ViT-S backward.)
+// GeLU (exact erf form, Sec. II-A) and its derivative Phi(a) + a phi(a), from
+// one evaluation of Phi. GeLU's value is not rounded to bf16 everywhere (it goes
+// into dL/dalpha and dL/ds in fp32), so Phi is erff's, whose error stays near
+// that of the last rounding (6e-8 in Phi). A five-term approximation of erfc
+// that shared the exponential took 17 instructions instead of 45, and four
+// times that error.
 __device__ __forceinline__ void gelu_and_grad(float a, float& g, float& dg) {
-  float e, t;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(a * a * -0.72134752044448170f));  // exp(-a^2/2)
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t) : "f"(fmaf(fabsf(a), 0.23164188819f, 1.0f)));
-  // -erfc / 2: the coefficients halved and negated
-  float q = fmaf(-0.5307027145f, t, 0.7265760135f);
-  q = fmaf(q, t, -0.7107068705f);
-  q = fmaf(q, t, 0.142248368f);
-  q = fmaf(q, t, -0.127414796f);
-  // Phi = 1/2 + sign(a) (1/2 - erfc / 2)
-  const float cdf = 0.5f + copysignf(fmaf(q * t, e, 0.5f), a);
+  const float cdf = 0.5f * (1.0f + erff(a * 0.70710678118654752f));
   g = a * cdf;
-  dg = fmaf(a * 0.39894228040143268f, e, cdf);
+  dg = cdf + a * 0.39894228040143268f * __expf(-0.5f * a * a);
 }
 
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {

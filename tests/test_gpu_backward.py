@@ -164,3 +164,44 @@ def test_backward_argument_errors():
     assert e.value.code == -6
     torch.cuda.synchronize()
     assert L.sync_status() == 0
+
+
+def test_gelu_of_the_router_gradient_in_fp32():
+    """dL/dalpha takes GeLU(a) in fp32. Token t has x = a_t in feature 0, whose
+    key is 1 in the shared expert's first channel, and 1 in feature 1 + t; dy V^T
+    is 1 in that channel; alpha = 1/2 (zero router, tau = 0, one of two blocks
+    shared): dL/dW*[1 + t][0] = GeLU(a_t) / 4, all other factors and terms being
+    exact. For every bf16 a_t of [2^-6, 8) and both signs.
+
+    Bound: erff within 2 ulp (its documented error) of values below 1 (2^-23),
+    its argument's two roundings (2^-23 z erf'(z) <= 2^-24), the sum 1 + erf
+    (2^-24), halved: 2^-23 |a| at most; the product's rounding, 2^-24 |GeLU|."""
+    from scipy.stats import norm
+
+    from paper_2608_10392_gb300 import FEATURE_BACKWARD, FEATURES_DEFAULT, Layer
+    dev, d, H, T = torch.device("cuda"), 1024, 128, 1000
+    L = Layer(d, H, 1, 2, max_tokens=T, tau=0.0, prefix_blocks=1,
+              features=FEATURES_DEFAULT | FEATURE_BACKWARD)
+    zeros = dict(dtype=torch.bfloat16, device=dev)
+    w_up, w_down = torch.zeros(2, H, d, **zeros), torch.zeros(2, d, H, **zeros)
+    w_up[0, 0, 0] = w_down[0, 0, 0] = 1
+    L.load_weights(torch.zeros(d, 2, **zeros), w_up, w_down)
+    mag = (torch.arange(128, dtype=torch.float64) / 128 + 1) * 2.0 ** torch.arange(
+        -6, 3, dtype=torch.float64)[:, None]
+    values = torch.cat([mag.flatten(), -mag.flatten()])
+    dy = torch.zeros(T, d, **zeros)
+    dy[:, 0] = 1
+    worst = 0.0
+    for a in values.split(T):
+        x = torch.zeros(T, d, **zeros)
+        x[:a.numel(), 0] = a.to(dev, torch.bfloat16)
+        x[torch.arange(T), 1 + torch.arange(T)] = 1
+        L.forward(x)
+        dw = L.backward(x, dy)["dw_router"]
+        torch.cuda.synchronize()
+        assert L.sync_status() == 0
+        got = 4 * dw[1:1 + a.numel(), 0].double().cpu().numpy()
+        ref = a.numpy() * norm.cdf(a.numpy())
+        bound = 2.0 ** -23 * np.abs(a.numpy()) + 2.0 ** -24 * np.abs(ref)
+        worst = max(worst, float((np.abs(got - ref) / bound).max()))
+    assert worst <= 1.0, worst
