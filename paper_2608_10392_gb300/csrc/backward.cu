@@ -69,18 +69,22 @@ __device__ __forceinline__ uint64_t sw128_mn_desc(uint32_t saddr, uint32_t lbo) 
 }
 
 constexpr int kEpiWarps = 8;      // of the weight-gradient kernel
+// Most 128-row tiles that one accumulation of the weight gradients runs over:
+// the tensor cores truncate the accumulator at every 16 rows, so the error grows
+// with the number of rows. A group's sums beyond that are added in fp32.
+constexpr int kSumTiles = 8;
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kAcc2 = 256;   // TMEM column of the second accumulator
 
 // Most 128-row tiles of a group in one weight-gradient item, `total` tiles in
 // `parts` items each (features x channels x kinds) on `ctas` CTAs: as many as
-// leave every CTA two items, so that most groups are one chunk, whose sums
-// are stored instead of added into zeroed outputs. (ViT-S, 25 tiles per
+// leave every CTA two items, so that most groups are one chunk, whose first
+// sums are stored instead of added into zeroed outputs. (ViT-S, 25 tiles per
 // group: chunks of at most 8 took 101 us, this 91; BERT-base, 5
 // tiles: 115 and 95, its 170 MB of gradients being more than L2 holds
 // between the clearing and the adds.)
 __device__ __forceinline__ int chunk_tiles(int total, int parts, int ctas) {
-  return max(8, (int)(((long long)total * parts + 2 * ctas - 1) / (2 * ctas)));
+  return max(kSumTiles, (int)(((long long)total * parts + 2 * ctas - 1) / (2 * ctas)));
 }
 
 // ---------------------------------------------------------------------------
@@ -472,8 +476,11 @@ bwd_hidden_kernel(const __grid_constant__ CUtensorMap tm_wk, const __grid_consta
 // The token rows are the reduction dimension, so both operands are MN-major:
 // the gathered rows (x, dy) and the TMA tiles (DA, HW) keep the 128-byte
 // swizzled row layout, read with MN-major descriptors. A group's tiles are
-// one chunk, whose sums are stored, or split evenly into chunks of at most
-// chunk_tiles, whose partial sums are added into the (zeroed) outputs.
+// one chunk or split evenly into chunks of at most chunk_tiles. A chunk's rows
+// are summed in accumulations of at most kSumTiles tiles, each in the TMEM
+// accumulator that the one before left free: the first of a group that is one
+// chunk is stored, all others are added into the outputs (zeroed where a group
+// is several chunks), in fp32 and by the thread that stored.
 // Roles: warps 0-4 fill the ring, a warp per stage (the gathered rows, and
 // the DA or HW tiles by TMA), warp 5 MMAs, warps 6-13 epilogue. The two
 // kinds are items of their own so that one accumulator leaves room in TMEM
@@ -581,7 +588,15 @@ bwd_wgrad_kernel(const __grid_constant__ CUtensorMap tm_da, const __grid_constan
   const int n_items = chunk_s[p.G] * p.n_c * p.n_nc * 2;
   // item -> (group g, its tiles [t0, t0 + nt) of one chunk, feature chunk c,
   // N chunk nc, kind); rows of the chunk start at row r0 of the group
-  struct Item { int g, t0, nt, r0, c, nc, kind; bool whole; };  // whole: the group's only chunk
+  struct Item {
+    int g, t0, nt, r0, c, nc, kind;
+    bool whole;  // the group's only chunk
+    __device__ __forceinline__ int sums() const { return (nt + kSumTiles - 1) / kSumTiles; }
+    // tiles of its j-th accumulation
+    __device__ __forceinline__ int tiles(int j) const {
+      return nt * (j + 1) / sums() - nt * j / sums();
+    }
+  };
   auto decode = [&](int item) {
     Item it;
     it.kind = item & 1;
@@ -665,27 +680,30 @@ bwd_wgrad_kernel(const __grid_constant__ CUtensorMap tm_da, const __grid_constan
     uint32_t ph = 0, acc_ph = 0;
     bool ok = true;
     for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
-      const int n_steps = decode(item).nt * kParts;
-      ok = wait_warp(acce_bar(acc), acc_ph ^ 1u, abort_flag, p.status, p.wait_limit);
-      if (!ok) break;
-      tc_fence_after();
-      const uint32_t d_tmem = tmem_base + (uint32_t)acc * kAcc2;
-      for (int kt = 0; kt < n_steps; ++kt) {
-        ok = wait_warp(full_bar(s), ph, abort_flag, p.status, p.wait_limit);
+      const Item it = decode(item);
+      for (int j = 0; j < it.sums() && ok; ++j) {
+        const int n_steps = it.tiles(j) * kParts;
+        ok = wait_warp(acce_bar(acc), acc_ph ^ 1u, abort_flag, p.status, p.wait_limit);
         if (!ok) break;
         tc_fence_after();
-        if (elect_one()) {
+        const uint32_t d_tmem = tmem_base + (uint32_t)acc * kAcc2;
+        for (int kt = 0; kt < n_steps; ++kt) {
+          ok = wait_warp(full_bar(s), ph, abort_flag, p.status, p.wait_limit);
+          if (!ok) break;
+          tc_fence_after();
+          if (elect_one()) {
 #pragma unroll
-          for (int k = 0; k < (int)kRows / 16; ++k)  // 16 rows (two 8-row groups) per MMA
-            umma_bf16(d_tmem, sw128_mn_desc(sp(s) + k * 2048u, lbo),
-                      sw128_mn_desc(sq(s) + k * 2048u, lbo), idesc, (kt | k) != 0 ? 1u : 0u);
-          umma_commit(empty_bar(s));
-          if (kt == n_steps - 1) umma_commit(accf_bar(acc));
+            for (int k = 0; k < (int)kRows / 16; ++k)  // 16 rows (two 8-row groups) per MMA
+              umma_bf16(d_tmem, sw128_mn_desc(sp(s) + k * 2048u, lbo),
+                        sw128_mn_desc(sq(s) + k * 2048u, lbo), idesc, (kt | k) != 0 ? 1u : 0u);
+            umma_commit(empty_bar(s));
+            if (kt == n_steps - 1) umma_commit(accf_bar(acc));
+          }
+          __syncwarp();
+          if (++s == n_st) { s = 0; ph ^= 1u; }
         }
-        __syncwarp();
-        if (++s == n_st) { s = 0; ph ^= 1u; }
+        if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
       }
-      if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
     }
   } else if (warp >= kWFirstEpi) {
     const int q = warp & 3;
@@ -695,60 +713,63 @@ bwd_wgrad_kernel(const __grid_constant__ CUtensorMap tm_da, const __grid_constan
     const bool wide = (reinterpret_cast<uintptr_t>(p.dw_down) & 31u) == 0;
     int acc = 0;
     uint32_t acc_ph = 0;
-    for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
+    bool ok = true;
+    for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
       const Item it = decode(item);
       const int e = it.g / p.B, blk = it.g % p.B;
       const int i = it.c * 128 + q * 32 + lane;  // this thread's feature
       const int h0 = blk * p.M + it.nc * p.N + half * cols;  // first channel of its columns
-      if (!wait_warp(accf_bar(acc), acc_ph, abort_flag, p.status, p.wait_limit)) break;
-      tc_fence_after();
-      const uint32_t t_row =
-          tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)acc * kAcc2 + half * cols;
-      // a whole group's sums are stored; the chunks of a split one add theirs
-      // (those outputs start at zero)
-      if (it.kind == 0) {  // dK_e[h][i]: a warp's lanes are 32 features of one h
-        float* col = p.dw_up + ((size_t)e * p.H + h0) * p.d + i;
-        for (int cc = 0; cc < cols; cc += 32) {
-          float v[32];
-          tmem_ld32(t_row + cc, v);
-          if (it.whole) {
+      for (int j = 0; j < it.sums() && ok; ++j) {
+        ok = wait_warp(accf_bar(acc), acc_ph, abort_flag, p.status, p.wait_limit);
+        if (!ok) break;
+        tc_fence_after();
+        const uint32_t t_row =
+            tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)acc * kAcc2 + half * cols;
+        const bool store = it.whole && j == 0;
+        if (it.kind == 0) {  // dK_e[h][i]: a warp's lanes are 32 features of one h
+          float* col = p.dw_up + ((size_t)e * p.H + h0) * p.d + i;
+          for (int cc = 0; cc < cols; cc += 32) {
+            float v[32];
+            tmem_ld32(t_row + cc, v);
+            if (store) {
 #pragma unroll
-            for (int jj = 0; jj < 32; ++jj) col[(size_t)(cc + jj) * p.d] = v[jj];
-          } else {
+              for (int jj = 0; jj < 32; ++jj) col[(size_t)(cc + jj) * p.d] = v[jj];
+            } else {
 #pragma unroll
-            for (int jj = 0; jj < 32; ++jj) atomicAdd(col + (size_t)(cc + jj) * p.d, v[jj]);
+              for (int jj = 0; jj < 32; ++jj) atomicAdd(col + (size_t)(cc + jj) * p.d, v[jj]);
+            }
+          }
+        } else {  // dV_e[i][h]: a thread's columns are contiguous
+          float* row = p.dw_down + ((size_t)e * p.d + i) * p.H + h0;
+          for (int cc = 0; cc < cols; cc += 32) {
+            float v[32];
+            tmem_ld32(t_row + cc, v);
+            if (store && wide) {  // whole 32-byte sectors per lane
+#pragma unroll
+              for (int jj = 0; jj < 32; jj += 8)
+                asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(
+                                 row + cc + jj),
+                             "f"(v[jj]), "f"(v[jj + 1]), "f"(v[jj + 2]), "f"(v[jj + 3]),
+                             "f"(v[jj + 4]), "f"(v[jj + 5]), "f"(v[jj + 6]), "f"(v[jj + 7])
+                             : "memory");
+            } else if (store) {
+#pragma unroll
+              for (int jj = 0; jj < 32; jj += 4)
+                *reinterpret_cast<float4*>(row + cc + jj) =
+                    make_float4(v[jj], v[jj + 1], v[jj + 2], v[jj + 3]);
+            } else {
+#pragma unroll
+              for (int jj = 0; jj < 32; jj += 4)
+                atomicAdd(reinterpret_cast<float4*>(row + cc + jj),
+                          make_float4(v[jj], v[jj + 1], v[jj + 2], v[jj + 3]));
+            }
           }
         }
-      } else {  // dV_e[i][h]: a thread's columns are contiguous
-        float* row = p.dw_down + ((size_t)e * p.d + i) * p.H + h0;
-        for (int cc = 0; cc < cols; cc += 32) {
-          float v[32];
-          tmem_ld32(t_row + cc, v);
-          if (it.whole && wide) {  // whole 32-byte sectors per lane
-#pragma unroll
-            for (int jj = 0; jj < 32; jj += 8)
-              asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(
-                               row + cc + jj),
-                           "f"(v[jj]), "f"(v[jj + 1]), "f"(v[jj + 2]), "f"(v[jj + 3]),
-                           "f"(v[jj + 4]), "f"(v[jj + 5]), "f"(v[jj + 6]), "f"(v[jj + 7])
-                           : "memory");
-          } else if (it.whole) {
-#pragma unroll
-            for (int jj = 0; jj < 32; jj += 4)
-              *reinterpret_cast<float4*>(row + cc + jj) =
-                  make_float4(v[jj], v[jj + 1], v[jj + 2], v[jj + 3]);
-          } else {
-#pragma unroll
-            for (int jj = 0; jj < 32; jj += 4)
-              atomicAdd(reinterpret_cast<float4*>(row + cc + jj),
-                        make_float4(v[jj], v[jj + 1], v[jj + 2], v[jj + 3]));
-          }
-        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(acce_bar(acc));
+        if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
       }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(acce_bar(acc));
-      if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
     }
   }
   __syncwarp();

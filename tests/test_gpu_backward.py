@@ -205,3 +205,41 @@ def test_gelu_of_the_router_gradient_in_fp32():
         bound = 2.0 ** -23 * np.abs(a.numpy()) + 2.0 ** -24 * np.abs(ref)
         worst = max(worst, float((np.abs(got - ref) / bound).max()))
     assert worst <= 1.0, worst
+
+
+@pytest.mark.parametrize("T,alpha,topk,shape", [
+    # 57 groups of 99 tiles, one item per group: 13 sums, stored and added
+    (12608, 0.125, 8, dict(d_model=384, d_ff=1536, n_experts=8, n_blocks=8)),
+    # 9 tiles per group
+    (1025, 0.125, 8, dict(d_model=384, d_ff=1536, n_experts=8, n_blocks=8)),
+    # 3 groups of 313 tiles, 13 items per group, 4 sums each
+    (40003, 0.5, 2, dict(d_model=512, d_ff=256, n_experts=2, n_blocks=2)),
+])
+def test_weight_gradient_accumulation_error(T, alpha, topk, shape):
+    """dV over groups of T rows, all rows of w GeLU(a) being equal (the same x for
+    every token): dV[i][h] = (sum_t dy[t][i]) hw[h], with hw an exact bf16 number
+    that the results give themselves. dy > 0, so that nothing cancels.
+
+    Bound: 1,024 rows are 64 accumulations, each truncated below the last bit
+    of the sum (2^-23 of it, half of that on average over a growing sum), then
+    at most T / 1,024 fp32 additions of 2^-24 each."""
+    from paper_2608_10392_gb300 import FEATURE_BACKWARD, FEATURES_DEFAULT
+    s = small(tokens=T, alpha_fixed=alpha, topk_fixed=topk, **shape)
+    wl = workloads.make_workload(s)
+    dev = torch.device("cuda")
+    L = make_layer(s, features=FEATURES_DEFAULT | FEATURE_BACKWARD)
+    L.load_weights(wl.w_router.to(dev), wl.w_up.to(dev), wl.w_down.to(dev))
+    x = wl.x[:1].to(dev).expand(T, -1).contiguous()
+    g = torch.Generator().manual_seed(3)
+    dy = torch.rand(T, s.d_model, generator=g).to(torch.bfloat16).to(dev)
+    L.forward(x)
+    dv = L.backward(x, dy)["dw_down"].double()
+    torch.cuda.synchronize()
+    assert L.sync_status() == 0
+    total = dy.double().sum(0)
+    hw = (dv / total[None, :, None]).mean(1).to(torch.bfloat16).double()  # [K + 1][H]
+    assert (hw != 0).any(dim=1).sum() == 1 + topk  # the experts that run
+    ref = total[None, :, None] * hw[:, None, :]
+    err = ((dv - ref).abs() / ref.abs())[ref != 0].max()
+    assert (dv[ref == 0] == 0).all()
+    assert err <= 64 * 2.0 ** -24 + T / 1024 * 2.0 ** -24, float(err)
