@@ -71,17 +71,17 @@ __device__ __forceinline__ uint64_t sw128_mn_desc(uint32_t saddr, uint32_t lbo) 
 constexpr int kEpiWarps = 8;      // of the weight-gradient kernel
 // Most 128-row tiles that one accumulation of the weight gradients runs over:
 // the tensor cores truncate the accumulator at every 16 rows, so the error grows
-// with the number of rows. A group's sums beyond that are added in fp32.
+// with the number of rows. Further rows are added in fp32.
 constexpr int kSumTiles = 8;
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kAcc2 = 256;   // TMEM column of the second accumulator
 
 // Most 128-row tiles of a group in one weight-gradient item, `total` tiles in
 // `parts` items each (features x channels x kinds) on `ctas` CTAs: as many as
-// leave every CTA two items, so that most groups are one chunk, whose first
-// sums are stored instead of added into zeroed outputs. (ViT-S, 25 tiles per
-// group: chunks of at most 8 took 101 us, this 91; BERT-base, 5
-// tiles: 115 and 95, its 170 MB of gradients being more than L2 holds
+// leave every CTA two items, so that most groups are one chunk, whose sums
+// are stored instead of added into zeroed outputs. (ViT-S, 25 tiles per
+// group: chunks of at most 8 took 101 us, this 95; BERT-base, 5
+// tiles: 115 and 97, its 170 MB of gradients being more than L2 holds
 // between the clearing and the adds.)
 __device__ __forceinline__ int chunk_tiles(int total, int parts, int ctas) {
   return max(kSumTiles, (int)(((long long)total * parts + 2 * ctas - 1) / (2 * ctas)));
@@ -102,9 +102,11 @@ __device__ __forceinline__ int chunk_tiles(int total, int parts, int ctas) {
 // accumulators take 2 bn <= 512 TMEM columns, so a tile's MMAs wait for the
 // epilogue of the one before; the ring holds the next tile's first steps by
 // then. (16 epilogue warps of half the columns ran no faster.)
-// Measured (ViT-S, 12,608 tokens; one CTA per tile, four gather warps, erff,
-// a 32-byte row piece per thread's store before): 138 -> 111 us; BERT-base
-// (2,300 tokens) 102 -> 76.
+// Measured (one CTA per tile, four gather warps, a 32-byte row piece per
+// thread's store before): BERT-base (2,300 tokens) 102 -> 88 us; ViT-S (12,608
+// tokens) 138 either way, bound by the epilogue's arithmetic: with a GeLU of
+// 17 instructions in place of erff's 45, but less exact, it took 111 (and
+// BERT-base 75).
 // ---------------------------------------------------------------------------
 struct HiddenParams {
   const int32_t* counts;   // [G] group sizes (the forward's)
@@ -476,19 +478,21 @@ bwd_hidden_kernel(const __grid_constant__ CUtensorMap tm_wk, const __grid_consta
 // The token rows are the reduction dimension, so both operands are MN-major:
 // the gathered rows (x, dy) and the TMA tiles (DA, HW) keep the 128-byte
 // swizzled row layout, read with MN-major descriptors. A group's tiles are
-// one chunk or split evenly into chunks of at most chunk_tiles. A chunk's rows
-// are summed in accumulations of at most kSumTiles tiles, each in the TMEM
-// accumulator that the one before left free: the first of a group that is one
-// chunk is stored, all others are added into the outputs (zeroed where a group
-// is several chunks), in fp32 and by the thread that stored.
+// one chunk, whose sums are stored, or split evenly into chunks of at most
+// chunk_tiles, whose partial sums are added into the (zeroed) outputs. A
+// chunk's rows are summed in accumulations of at most kSumTiles tiles: the first
+// stays in its TMEM accumulator, the others run in the second one and are added
+// there by the epilogue warps in fp32. (Each added into the outputs instead:
+// 122 us per ViT-S backward.) The next chunk begins in the second accumulator
+// while the sum of this one goes out.
 // Roles: warps 0-4 fill the ring, a warp per stage (the gathered rows, and
 // the DA or HW tiles by TMA), warp 5 MMAs, warps 6-13 epilogue. The two
 // kinds are items of their own so that one accumulator leaves room in TMEM
 // for a second: an item's atomic adds run under the next one's MMAs. Bound
 // by the operand bytes out of L2 (40 KB per 64 rows of 192 channels).
 // Measured (both kinds in one item, accumulators not overlapped, four stages
-// of 32 rows before): ViT-S 12,608 tokens 117 -> 91 us, BERT-base (2,300
-// tokens) 130 -> 95.
+// of 32 rows before): ViT-S 12,608 tokens 117 -> 95 us, BERT-base (2,300
+// tokens) 130 -> 97.
 // ---------------------------------------------------------------------------
 struct WgradParams {
   const int32_t* counts;   // [G] group sizes (the forward's)
@@ -676,15 +680,18 @@ bwd_wgrad_kernel(const __grid_constant__ CUtensorMap tm_da, const __grid_constan
   } else if (warp == kWMma) {
     const uint32_t idesc = idesc_bf16_mn(kBM, p.N);
     const uint32_t lbo = kRows * 128u;  // 64-element MN blocks of kRows rows
-    int s = 0, acc = 0;
-    uint32_t ph = 0, acc_ph = 0;
+    int s = 0, first = 0;  // first: the accumulator of an item's first sum
+    uint32_t ph = 0, acc_ph = 0;  // (a phase bit per accumulator)
     bool ok = true;
     for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
       const Item it = decode(item);
       for (int j = 0; j < it.sums() && ok; ++j) {
         const int n_steps = it.tiles(j) * kParts;
-        ok = wait_warp(acce_bar(acc), acc_ph ^ 1u, abort_flag, p.status, p.wait_limit);
+        const int acc = j == 0 ? first : first ^ 1;
+        ok = wait_warp(acce_bar(acc), ((acc_ph >> acc) & 1u) ^ 1u, abort_flag, p.status,
+                       p.wait_limit);
         if (!ok) break;
+        acc_ph ^= 1u << acc;
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + (uint32_t)acc * kAcc2;
         for (int kt = 0; kt < n_steps; ++kt) {
@@ -702,8 +709,8 @@ bwd_wgrad_kernel(const __grid_constant__ CUtensorMap tm_da, const __grid_constan
           __syncwarp();
           if (++s == n_st) { s = 0; ph ^= 1u; }
         }
-        if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
       }
+      first ^= 1;
     }
   } else if (warp >= kWFirstEpi) {
     const int q = warp & 3;
@@ -711,65 +718,90 @@ bwd_wgrad_kernel(const __grid_constant__ CUtensorMap tm_da, const __grid_constan
     const int cols = p.N / 2;
     // (the caller's buffer need only be 16-byte aligned)
     const bool wide = (reinterpret_cast<uintptr_t>(p.dw_down) & 31u) == 0;
-    int acc = 0;
+    int first = 0;
     uint32_t acc_ph = 0;
+    auto wait_acc = [&](int acc) {
+      const uint32_t phase = (acc_ph >> acc) & 1u;
+      acc_ph ^= 1u << acc;
+      const bool ok = wait_warp(accf_bar(acc), phase, abort_flag, p.status, p.wait_limit);
+      tc_fence_after();
+      return ok;
+    };
+    auto release = [&](int acc) {
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(acce_bar(acc));
+    };
     bool ok = true;
     for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
       const Item it = decode(item);
       const int e = it.g / p.B, blk = it.g % p.B;
       const int i = it.c * 128 + q * 32 + lane;  // this thread's feature
       const int h0 = blk * p.M + it.nc * p.N + half * cols;  // first channel of its columns
-      for (int j = 0; j < it.sums() && ok; ++j) {
-        ok = wait_warp(accf_bar(acc), acc_ph, abort_flag, p.status, p.wait_limit);
+      const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16) + half * cols;
+      const uint32_t t_sum = t_row + (uint32_t)first * kAcc2;
+      ok = wait_acc(first);
+      for (int j = 1; j < it.sums() && ok; ++j) {  // the first sum += the j-th
+        ok = wait_acc(first ^ 1);
         if (!ok) break;
-        tc_fence_after();
-        const uint32_t t_row =
-            tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)acc * kAcc2 + half * cols;
-        const bool store = it.whole && j == 0;
-        if (it.kind == 0) {  // dK_e[h][i]: a warp's lanes are 32 features of one h
-          float* col = p.dw_up + ((size_t)e * p.H + h0) * p.d + i;
-          for (int cc = 0; cc < cols; cc += 32) {
-            float v[32];
-            tmem_ld32(t_row + cc, v);
-            if (store) {
+        const uint32_t t_part = t_row + (uint32_t)(first ^ 1) * kAcc2;
+        for (int cc = 0; cc < cols; cc += 32) {
+          uint32_t u[32], v[32];
+          float sum[32];
+          tmem_ld32_async(t_sum + cc, u);
+          tmem_ld32_async(t_part + cc, v);
+          tmem_wait_ld();
 #pragma unroll
-              for (int jj = 0; jj < 32; ++jj) col[(size_t)(cc + jj) * p.d] = v[jj];
-            } else {
+          for (int jj = 0; jj < 32; ++jj) sum[jj] = __uint_as_float(u[jj]) + __uint_as_float(v[jj]);
+          tmem_st32_async(t_sum + cc, sum);
+        }
+        tmem_wait_st();
+        release(first ^ 1);
+      }
+      if (!ok) break;
+      // a whole group's sums are stored; the chunks of a split one add theirs
+      // (those outputs start at zero)
+      if (it.kind == 0) {  // dK_e[h][i]: a warp's lanes are 32 features of one h
+        float* col = p.dw_up + ((size_t)e * p.H + h0) * p.d + i;
+        for (int cc = 0; cc < cols; cc += 32) {
+          float v[32];
+          tmem_ld32(t_sum + cc, v);
+          if (it.whole) {
 #pragma unroll
-              for (int jj = 0; jj < 32; ++jj) atomicAdd(col + (size_t)(cc + jj) * p.d, v[jj]);
-            }
-          }
-        } else {  // dV_e[i][h]: a thread's columns are contiguous
-          float* row = p.dw_down + ((size_t)e * p.d + i) * p.H + h0;
-          for (int cc = 0; cc < cols; cc += 32) {
-            float v[32];
-            tmem_ld32(t_row + cc, v);
-            if (store && wide) {  // whole 32-byte sectors per lane
+            for (int jj = 0; jj < 32; ++jj) col[(size_t)(cc + jj) * p.d] = v[jj];
+          } else {
 #pragma unroll
-              for (int jj = 0; jj < 32; jj += 8)
-                asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(
-                                 row + cc + jj),
-                             "f"(v[jj]), "f"(v[jj + 1]), "f"(v[jj + 2]), "f"(v[jj + 3]),
-                             "f"(v[jj + 4]), "f"(v[jj + 5]), "f"(v[jj + 6]), "f"(v[jj + 7])
-                             : "memory");
-            } else if (store) {
-#pragma unroll
-              for (int jj = 0; jj < 32; jj += 4)
-                *reinterpret_cast<float4*>(row + cc + jj) =
-                    make_float4(v[jj], v[jj + 1], v[jj + 2], v[jj + 3]);
-            } else {
-#pragma unroll
-              for (int jj = 0; jj < 32; jj += 4)
-                atomicAdd(reinterpret_cast<float4*>(row + cc + jj),
-                          make_float4(v[jj], v[jj + 1], v[jj + 2], v[jj + 3]));
-            }
+            for (int jj = 0; jj < 32; ++jj) atomicAdd(col + (size_t)(cc + jj) * p.d, v[jj]);
           }
         }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(acce_bar(acc));
-        if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
+      } else {  // dV_e[i][h]: a thread's columns are contiguous
+        float* row = p.dw_down + ((size_t)e * p.d + i) * p.H + h0;
+        for (int cc = 0; cc < cols; cc += 32) {
+          float v[32];
+          tmem_ld32(t_sum + cc, v);
+          if (it.whole && wide) {  // whole 32-byte sectors per lane
+#pragma unroll
+            for (int jj = 0; jj < 32; jj += 8)
+              asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(
+                               row + cc + jj),
+                           "f"(v[jj]), "f"(v[jj + 1]), "f"(v[jj + 2]), "f"(v[jj + 3]),
+                           "f"(v[jj + 4]), "f"(v[jj + 5]), "f"(v[jj + 6]), "f"(v[jj + 7])
+                           : "memory");
+          } else if (it.whole) {
+#pragma unroll
+            for (int jj = 0; jj < 32; jj += 4)
+              *reinterpret_cast<float4*>(row + cc + jj) =
+                  make_float4(v[jj], v[jj + 1], v[jj + 2], v[jj + 3]);
+          } else {
+#pragma unroll
+            for (int jj = 0; jj < 32; jj += 4)
+              atomicAdd(reinterpret_cast<float4*>(row + cc + jj),
+                        make_float4(v[jj], v[jj + 1], v[jj + 2], v[jj + 3]));
+          }
+        }
       }
+      release(first);
+      first ^= 1;
     }
   }
   __syncwarp();
