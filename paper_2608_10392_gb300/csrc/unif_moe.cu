@@ -104,29 +104,59 @@ void free_all(unif_moe_layer* L) {
   if (L->copy_out) cudaStreamDestroy(L->copy_out);
 }
 
-// Takes a handle back to the unbundled down projection after an allocation for
-// the bundled one failed.
-void drop_bundles(unif_moe_layer* L) {
-  void** ptrs[] = {reinterpret_cast<void**>(&L->ws.bd_fill),
-                   reinterpret_cast<void**>(&L->ws.bd_rows),
-                   reinterpret_cast<void**>(&L->ws.bd_dst),
-                   reinterpret_cast<void**>(&L->ws.bd_n_tiles),
-                   reinterpret_cast<void**>(&L->ws.bd_tile_group),
-                   reinterpret_cast<void**>(&L->ws.bd_tile_row0),
-                   reinterpret_cast<void**>(&L->ws.bd_tile_rows),
-                   reinterpret_cast<void**>(&L->ws.bd_tile_unit)};
-  for (void** q : ptrs) {
+size_t elt_size(const unif_moe_layer* L) { return L->dtype == UNIF_MOE_BF16 ? 2 : 4; }
+
+// The bundled down projection's tables and h in its layout (more rows), in
+// place of the h of max_rows rows allocated before. Last of a handle's
+// allocations, and given up where one fails: the layer then keeps its unbundled
+// kernels, so that it needs no more memory than those. The rows' list is the
+// largest table, 8 bytes per group and token slot of a pass; with the larger h
+// the bundles of 12,608 tokens of d = 768, K = B = 16 take 0.2 GB, those of
+// 32,768 tokens of d = 1024, K = 32 0.8 GB (below 17 GB for any layer, by the
+// int32 indexes of bundles_fit).
+int alloc_bundles(unif_moe_layer* L) {
+  unif::Workspace& w = L->ws;
+  const size_t G2 = (size_t)unif::bundle_groups(L), nt = (size_t)unif::bundle_max_tiles(L);
+  const size_t h_row = elt_size(L) * (size_t)L->M;
+  bool ok = dalloc(&w.bd_fill, G2) == UNIF_MOE_OK &&
+            dalloc(&w.bd_rows, G2 * L->region_rows) == UNIF_MOE_OK &&
+            dalloc(&w.bd_dst, (size_t)L->pass_tokens * (L->K + 1) * (L->B / unif::kBundle)) ==
+                UNIF_MOE_OK &&
+            dalloc(&w.bd_n_tiles, 1) == UNIF_MOE_OK && dalloc(&w.bd_tile_group, nt) == UNIF_MOE_OK &&
+            dalloc(&w.bd_tile_row0, nt) == UNIF_MOE_OK &&
+            dalloc(&w.bd_tile_rows, nt) == UNIF_MOE_OK && dalloc(&w.bd_tile_unit, nt) == UNIF_MOE_OK;
+  char* h = nullptr;
+  if (ok) {
+    cudaFree(w.hbuf);
+    w.hbuf = nullptr;
+    L->h_rows = std::max(L->max_rows, unif::bundle_h_rows(L));
+    ok = dalloc(&h, h_row * (size_t)L->h_rows) == UNIF_MOE_OK;
+    w.hbuf = h;
+  }
+  if (ok) return UNIF_MOE_OK;
+  void** tables[] = {reinterpret_cast<void**>(&w.bd_fill),
+                     reinterpret_cast<void**>(&w.bd_rows),
+                     reinterpret_cast<void**>(&w.bd_dst),
+                     reinterpret_cast<void**>(&w.bd_n_tiles),
+                     reinterpret_cast<void**>(&w.bd_tile_group),
+                     reinterpret_cast<void**>(&w.bd_tile_row0),
+                     reinterpret_cast<void**>(&w.bd_tile_rows),
+                     reinterpret_cast<void**>(&w.bd_tile_unit)};
+  for (void** q : tables) {
     if (*q) cudaFree(*q);
     *q = nullptr;
   }
   L->bundles = false;
   L->h_rows = L->max_rows;
   cudaGetLastError();  // the failed allocation must not surface at a later launch
+  unif::g_err[0] = 0;
+  if (w.hbuf) return UNIF_MOE_OK;
+  const int rc = dalloc(&h, h_row * (size_t)L->h_rows);
+  w.hbuf = h;
+  return rc;
 }
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
-
-size_t elt_size(const unif_moe_layer* L) { return L->dtype == UNIF_MOE_BF16 ? 2 : 4; }
 
 }  // namespace
 
@@ -284,32 +314,9 @@ int unif_moe_create_ex(unif_moe_t* out, int d_model, int d_ff, int n_experts, in
   const size_t row_cap = L->fused_group ? (size_t)L->G * L->region_rows : (size_t)L->max_rows;
   ALLOC(w.row_tok, row_cap); ALLOC(w.row_w, row_cap);
   if (L->fused_group) ALLOC(w.grp_fill, (size_t)L->G);
-  // wide layers' passes of many tokens: the down projection's rows bundled
-  // over four blocks, h in their layout; without room for the tables (at most
-  // 1.4 GB) the layer keeps its unbundled kernels
-  L->bundles = true;
-  L->bundles = rc == UNIF_MOE_OK && dtype == UNIF_MOE_BF16 && unif::bundles_fit(L) &&
-               unif::bundles_apply(L, L->pass_tokens);
   L->h_rows = L->max_rows;
-  if (L->bundles) {
-    const size_t G2 = (size_t)unif::bundle_groups(L), nt = (size_t)unif::bundle_max_tiles(L);
-    L->h_rows = std::max(L->h_rows, unif::bundle_h_rows(L));
-    ALLOC(w.bd_fill, G2);
-    ALLOC(w.bd_rows, G2 * L->region_rows);
-    ALLOC(w.bd_dst, (size_t)L->pass_tokens * E * (n_blocks / unif::kBundle));
-    ALLOC(w.bd_n_tiles, 1); ALLOC(w.bd_tile_group, nt); ALLOC(w.bd_tile_row0, nt);
-    ALLOC(w.bd_tile_rows, nt); ALLOC(w.bd_tile_unit, nt);
-    if (rc != UNIF_MOE_OK) {
-      drop_bundles(L);
-      rc = UNIF_MOE_OK;
-    }
-  }
   void* hb = nullptr;
   if (rc == UNIF_MOE_OK) rc = dalloc(reinterpret_cast<char**>(&hb), es * (size_t)L->h_rows * M);
-  if (rc != UNIF_MOE_OK && L->bundles) {  // h in the unbundled layout is smaller
-    drop_bundles(L);
-    rc = dalloc(reinterpret_cast<char**>(&hb), es * (size_t)L->h_rows * M);
-  }
   w.hbuf = hb;
   ALLOC(w.y32, (size_t)L->pass_tokens * d_model);
   if (L->ffn_fused) ALLOC(w.y32_b, (size_t)L->pass_tokens * d_model);
@@ -362,6 +369,12 @@ int unif_moe_create_ex(unif_moe_t* out, int d_model, int d_ff, int n_experts, in
     ALLOC(w.diag_E, T * K * d_model); ALLOC(w.diag_ES, T * K * d_model);
   }
 #undef ALLOC
+  // wide layers' passes of many tokens: the down projection's rows bundled
+  // over four blocks, where memory for it is left
+  L->bundles = true;
+  L->bundles = rc == UNIF_MOE_OK && dtype == UNIF_MOE_BF16 && unif::bundles_fit(L) &&
+               unif::bundles_apply(L, L->pass_tokens);
+  if (L->bundles) rc = alloc_bundles(L);
   if (rc == UNIF_MOE_OK && (cudaMemset(w.status, 0, sizeof(int)) != cudaSuccess ||
                             cudaMemset(w.y32, 0, sizeof(float) * L->pass_tokens * d_model) !=
                                 cudaSuccess ||

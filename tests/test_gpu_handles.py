@@ -65,3 +65,44 @@ def test_a_later_handle_leaves_an_earlier_one_as_it_is(large, small, kernels):
     outputs(b, xb, dyb, train)
     for u, v in zip(before, after):
         assert (u - v).abs().max() <= 2.0 ** -7 * u.abs().max()
+
+
+def test_a_handle_without_room_for_the_bundles_is_made_unbundled():
+    """With too little memory left for the bundled down projection's tables, but
+    enough for everything else of a training handle, the handle is made and runs
+    the unbundled kernels."""
+    from paper_2608_10392_gb300 import FEATURE_BACKWARD, FEATURES_DEFAULT, Layer
+    T, shape = 16000, (640, 3072, 32, 16)
+
+    def layer():
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        free = torch.cuda.mem_get_info()[0]
+        made = Layer(*shape, max_tokens=T, features=FEATURES_DEFAULT | FEATURE_BACKWARD)
+        return made, free - torch.cuda.mem_get_info()[0]
+
+    src, x, dy = make(*shape, T)
+    weights = src._keep[:3]
+    del src
+    a, size = layer()
+    assert a.kernels_per_forward() == 6
+    a.load_weights(*weights)
+    y = a.forward(x).float()
+    grads = a.backward(x, dy)
+    a.close()
+    # the tables and the larger h take 0.4 GB: leave all but half of that
+    room = size - (200 << 20)
+    held = torch.empty(torch.cuda.mem_get_info()[0] - room, dtype=torch.uint8, device="cuda")
+    b, smaller = layer()
+    try:
+        assert b.kernels_per_forward() == 4 and smaller < room
+        b.load_weights(*weights)
+        out = b.forward(x)
+        b.backward(x, dy, out=grads)
+        torch.cuda.synchronize()
+        assert b.sync_status() == 0
+    finally:
+        b.close()
+        del held
+        torch.cuda.empty_cache()
+    assert (out.float() - y).abs().max() <= 2.0 ** -7 * y.abs().max()
