@@ -7,6 +7,7 @@
 //   down : y[tok(row)] += w(row) * h[row] V_e[H_b, :]       (Eqs. 16, 28-30)
 // where (e, b) is the tile's group and w(row) is alpha or p_i.
 #include "internal.cuh"
+#include "items.cuh"
 
 namespace unif {
 namespace {
@@ -62,9 +63,10 @@ simt_gemm_kernel(const float* __restrict__ A, const float* __restrict__ W, float
   const int n_chunks = (N + kTN - 1) / kTN;
   grid_dep_launch();
   grid_dep_wait();  // the tile list, the rows and (down) h are complete
-  const int n_items = a.n_tiles[0] * 4 * n_chunks;
-  for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
-    const int q = (item / n_chunks) & 3, tile = item / (4 * n_chunks), n0 = item % n_chunks * kTN;
+  const int n_tiles = a.n_tiles[0];
+  ItemWalk item(blockIdx.x, gridDim.x, 4 * n_chunks);
+  for (; item.tile < n_tiles; item.next()) {
+    const int tile = item.tile, q = item.part / n_chunks, n0 = item.part % n_chunks * kTN;
     const int rows = min(kTM, a.tile_rows[tile] - kTM * q);
     if (rows <= 0) continue;  // padding only
     const int g = a.tile_group[tile], row0 = a.tile_row0[tile] + kTM * q;

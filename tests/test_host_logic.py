@@ -4,6 +4,7 @@ multi-rank bookkeeping of bench.py, run as two gloo ranks."""
 import math
 import os
 import socket
+import subprocess
 
 import pytest
 import torch
@@ -125,3 +126,38 @@ def test_two_rank_weak_scaling_bookkeeping():
     for rank, t, n, v in res:
         assert t == 0.40 and n == 1900.0
         assert v == pytest.approx(1900 / 0.40e-3)
+
+
+# ------------------------------------------------------------ kernel items
+
+def test_work_items_beyond_32_bits(tmp_path):
+    """The fp32 projections' walk over their items, compiled for the host: the
+    items of every CTA against 64-bit arithmetic, for a layer whose items are
+    more than 2^31 (1.1e9 group rows, d = 4096), and for few tiles."""
+    csrc = os.path.join(os.path.dirname(bench.__file__), "paper_2608_10392_gb300", "csrc")
+    src = tmp_path / "walk.cpp"
+    src.write_text(r"""
+#define __host__
+#define __device__
+#define __forceinline__ inline
+#include "items.cuh"
+#include <cstdio>
+#include <cstdlib>
+int main(int argc, char** argv) {
+  const long long tiles = atoll(argv[1]), parts = atoll(argv[2]), ctas = atoll(argv[3]);
+  long long n = 0;
+  for (int cta = 0; cta < ctas; cta += 1 + (int)ctas / 20) {
+    unif::ItemWalk w(cta, (int)ctas, (int)parts);
+    long long item = cta;
+    for (; w.tile < tiles; w.next(), item += ctas, ++n)
+      if (w.tile != item / parts || w.part != item % parts) return 1;
+    if (item < tiles * parts || item - ctas >= tiles * parts) return 2;
+  }
+  printf("%lld", n);
+}
+""")
+    exe = tmp_path / "walk"
+    subprocess.run(["g++", "-O2", "-I", csrc, "-o", str(exe), str(src)], check=True)
+    for tiles, parts, ctas in ((8_500_000, 256, 608), (1, 4, 608), (3, 1000, 608), (700, 4, 608)):
+        r = subprocess.run([str(exe), str(tiles), str(parts), str(ctas)], capture_output=True)
+        assert r.returncode == 0, (tiles, parts, ctas, r.returncode)
