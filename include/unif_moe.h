@@ -212,7 +212,8 @@ UNIF_MOE_API int unif_moe_sublayer_forward(unif_moe_t h, const void* x_dev, void
  * address are written by the kernels directly, with no copy back. Large
  * batches of pinned buffers (layers with the expert-tile FFN) run in three
  * parts of tokens, whose copies overlap one another's kernels on the handle's
- * copy streams; results and records are those of one pass. The staging
+ * copy streams; results and records are those of one pass. The buffers may
+ * overlap (then all of x_host is read before any output is written). The staging
  * buffers are allocated at create time (UNIF_MOE_FEATURE_HOST_IO;
  * ERR_STATE on a handle created without it). */
 UNIF_MOE_API int unif_moe_forward_host(unif_moe_t h, const void* x_host, void* out_host, int T,

@@ -724,6 +724,12 @@ static bool pinned_host(const void* p) {
   return at.type == cudaMemoryTypeHost;
 }
 
+// Whether [p, p + pn) and [q, q + qn) have a byte in common.
+static bool overlap(const void* p, size_t pn, const void* q, size_t qn) {
+  const uintptr_t a = reinterpret_cast<uintptr_t>(p), b = reinterpret_cast<uintptr_t>(q);
+  return a < b + qn && b < a + pn;
+}
+
 // The host-buffer forward in three parts of tokens (a quarter, a half, a
 // quarter), each a pass of its own: the later parts' inputs and the first
 // two's outputs move under the kernels, which a single pass leaves waiting
@@ -732,7 +738,9 @@ static bool pinned_host(const void* p) {
 // layer, us, one pass against three parts: 8,000 tokens 168 and 191, 12,608
 // 235 and 231, 16,000 286 and 254, 40,000 641 and 502), so it is taken from
 // kHostPartTokens on. x_host and out_host are pinned, out_dev is out_host's
-// device address; T <= pass_tokens.
+// device address; T <= pass_tokens. A part's results are stored before the
+// inputs of later parts are read: x_host has no byte in common with out_host
+// (unless they are the same rows) or with the counts.
 constexpr int kHostPartTokens = 14336;
 static int forward_host_parts(unif_moe_t L, const void* x_host, void* out_host, char* out_dev, int T,
                               const uint8_t* mask_host, int32_t* b_dev, int32_t* k_dev,
@@ -812,7 +820,11 @@ int unif_moe_forward_host(unif_moe_t L, const void* x_host, void* out_host, int 
   // In parts from kHostPartTokens on, where pinned buffers let the copies run
   // beside the kernels, for layers whose group table follows from the routing
   // records (the expert-tile FFN).
-  if (L->ffn_fused && T >= kHostPartTokens && T <= L->pass_tokens && out_dev &&
+  const size_t cb = sizeof(int32_t) * (size_t)T;
+  const bool apart = (x_host == out_host || !overlap(x_host, xb, out_host, xb)) &&
+                     !(b_host && overlap(x_host, xb, b_host, cb)) &&
+                     !(k_host && overlap(x_host, xb, k_host, cb));
+  if (L->ffn_fused && T >= kHostPartTokens && T <= L->pass_tokens && out_dev && apart &&
       pinned_host(x_host) && (!b_host || b_dev) && (!k_host || k_dev)) {
     // a failure leaves no copy of the caller's buffers in flight
     const int rc = forward_host_parts(L, x_host, out_host, static_cast<char*>(out_dev), T,

@@ -157,6 +157,22 @@ def test_host_forward_in_parts(T, masked):
     assert torch.equal(again[3], w)
 
 
+@pytest.mark.parametrize("shift", [0, 15000, -10000, 3])
+def test_host_forward_of_overlapping_buffers(shift):
+    """x and out in one pinned buffer, out `shift` rows after x: as with buffers
+    of their own (x is read before any of it is overwritten)."""
+    T, d = 20000, 384
+    wl = workloads.make_workload(small(tokens=T, d_model=d, n_experts=2))
+    g = run_gpu(wl)
+    for _ in range(3):
+        buf = torch.zeros(T + abs(shift), d, dtype=torch.bfloat16).pin_memory()
+        x, out = buf[max(-shift, 0):][:T], buf[max(shift, 0):][:T]
+        x.copy_(wl.x)
+        g.layer.forward_host(x, out)
+        assert g.layer.sync_status() == 0
+        assert np.abs(out.float().numpy() - g.y).max() <= 2.0 ** -7 * np.abs(g.y).max()
+
+
 @pytest.mark.parametrize("kw", [
     dict(tokens=3000, n_experts=2),                   # groups of more than one chunk: added
     dict(tokens=900, n_experts=3, d_ff=768),          # single chunks: stored (M = 192)
