@@ -24,6 +24,10 @@
 // in units of 128 rows x M, |s| units per tile (one per block of s, in
 // order), and the up projection, whose own groups stay (expert, block),
 // writes each row to the place that dst names.
+#include <math.h>
+
+#include <algorithm>
+
 #include "decide.cuh"
 #include "internal.cuh"
 
@@ -247,17 +251,29 @@ int64_t bundle_max_tiles(const unif_moe_layer* L) {
 
 // A pass of T tokens bundles its rows where the groups hold at least M^2 / 500
 // tokens on average: T (1 + k) / (K + 1) tokens per expert over 15 patterns, k
-// the fixed count or else about K / 3. Narrow blocks gain most (an output
+// the fixed count or else about K / 3, or 2/3 beta K where a fixed mass (beta,
+// or 1 - alpha) makes it less. Narrow blocks gain most (an output
 // row per M channels of work), and small groups lose to padding. Measured, us
 // per forward without and with bundles: d = 768, K = 16, M = 192: 2,500
 // tokens (62 per group) 167 and 172, 4,000 228 and 203, 12,608 583 and 497;
-// with two experts per token 5,000 (59) 153 and 168, 12,608 288 and 250; K =
+// with two experts per token 5,000 (59) 153 and 168, 12,608 288 and 250; with
+// beta = 0.05 3,000 (24) 89 and 139, 6,000 135 and 162, 12,608 219 and 218; with
+// alpha = 0.9 3,000 102 and 118, 6,000 146 and 145, 12,608 220 and 199; K =
 // 10, M = 256: 4,000 (105) 163 and 149; K = 8, M = 384: 7,000 (190) 172 and
 // 177, 14,000 319 and 305; d = 1024, skewed, K = 32, M = 256: 6,000 (141) 412
 // and 415, 9,000 546 and 502; K = 12, M = 512: 20,000 (512) 414 and 420.
+// T counts padding too, which the host does not know: half-padded batches near
+// the line lose a little (3,000 slots of the first layer 132 and 154).
 bool bundles_apply(const unif_moe_layer* L, int T) {
   if (!L->bundles) return false;
-  const double k = L->th.topk_fixed > 0 ? L->th.topk_fixed : L->K / 3.0;
+  const unif_moe_thresholds& th = L->th;
+  double k = L->K / 3.0;
+  if (th.topk_fixed > 0) {
+    k = th.topk_fixed;
+  } else if (!isnan(th.beta_fixed) || !isnan(th.alpha_fixed)) {
+    const double beta = isnan(th.beta_fixed) ? 1.0 - th.alpha_fixed : th.beta_fixed;
+    k = std::min(k, std::max(1.0, 2.0 / 3.0 * beta * L->K));
+  }
   return (double)T * (1.0 + k) * 500.0 >= (double)L->M * L->M * kPatterns * (L->K + 1);
 }
 

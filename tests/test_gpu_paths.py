@@ -133,6 +133,19 @@ def test_bundled_down_projection(shape, kw):
     assert np.abs(again.y - g.y).max() <= 2e-2 * np.abs(g.y).max()
 
 
+@pytest.mark.parametrize("T,kw,kernels", [
+    (3000, dict(), 6), (3000, dict(beta_fixed=0.05), 4), (3000, dict(alpha_fixed=0.95), 4),
+    (6000, dict(beta_fixed=0.05), 6), (3000, dict(beta_fixed=0.9), 6),
+])
+def test_few_experts_per_token_bundle_later(T, kw, kernels):
+    """A fixed mass that one expert reaches leaves fewer rows per group: the
+    bundled down projection begins at more tokens."""
+    wl = workloads.make_workload(small(tokens=T, d_model=832, d_ff=768, n_experts=9, **kw))
+    g, rep = _run(wl)
+    assert g.layer.kernels_per_forward() == kernels
+    assert_parity(wl, g, rep)
+
+
 @pytest.mark.parametrize("T,masked", [(14335, False), (14336, True), (20011, False)])
 def test_host_forward_in_parts(T, masked):
     """From 14,336 tokens on, a forward of pinned buffers runs in three parts:
