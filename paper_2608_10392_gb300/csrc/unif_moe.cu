@@ -736,12 +736,15 @@ static bool overlap(const void* p, size_t pn, const void* q, size_t qn) {
 // for the whole input and then storing the whole output over the link. Each
 // part costs its own router, launches and copy latencies, though (ViT-S
 // layer, us, one pass against three parts: 8,000 tokens 168 and 191, 12,608
-// 235 and 231, 16,000 286 and 254, 40,000 641 and 502), so it is taken from
-// kHostPartTokens on. x_host and out_host are pinned, out_dev is out_host's
+// 235 and 231, 16,000 286 and 254, 40,000 641 and 502; d = 256, K = 2, 14,336
+// tokens 142 and 141; d = 128, K = 4, whose copies are short, 14,336 102 and
+// 120, 20,000 129 and 134, 24,000 139 and 138, 28,672 162 and 152), so it is
+// taken from kHostPartTokens tokens and kHostPartBytes of input on. x_host and out_host are pinned, out_dev is out_host's
 // device address; T <= pass_tokens. A part's results are stored before the
 // inputs of later parts are read: x_host has no byte in common with out_host
 // (unless they are the same rows) or with the counts.
 constexpr int kHostPartTokens = 14336;
+constexpr size_t kHostPartBytes = 7u << 20;  // 14,336 tokens of d = 256
 static int forward_host_parts(unif_moe_t L, const void* x_host, void* out_host, char* out_dev, int T,
                               const uint8_t* mask_host, int32_t* b_dev, int32_t* k_dev,
                               cudaStream_t s) {
@@ -817,15 +820,15 @@ int unif_moe_forward_host(unif_moe_t L, const void* x_host, void* out_host, int 
   void* out_dev = mapped_host(out_host);
   int32_t* b_dev = static_cast<int32_t*>(mapped_host(b_host));
   int32_t* k_dev = static_cast<int32_t*>(mapped_host(k_host));
-  // In parts from kHostPartTokens on, where pinned buffers let the copies run
-  // beside the kernels, for layers whose group table follows from the routing
-  // records (the expert-tile FFN).
+  // In parts from kHostPartTokens and kHostPartBytes on, where pinned buffers
+  // let the copies run beside the kernels, for layers whose group table follows
+  // from the routing records (the expert-tile FFN).
   const size_t cb = sizeof(int32_t) * (size_t)T;
   const bool apart = (x_host == out_host || !overlap(x_host, xb, out_host, xb)) &&
                      !(b_host && overlap(x_host, xb, b_host, cb)) &&
                      !(k_host && overlap(x_host, xb, k_host, cb));
-  if (L->ffn_fused && T >= kHostPartTokens && T <= L->pass_tokens && out_dev && apart &&
-      pinned_host(x_host) && (!b_host || b_dev) && (!k_host || k_dev)) {
+  if (L->ffn_fused && T >= kHostPartTokens && xb >= kHostPartBytes && T <= L->pass_tokens &&
+      out_dev && apart && pinned_host(x_host) && (!b_host || b_dev) && (!k_host || k_dev)) {
     // a failure leaves no copy of the caller's buffers in flight
     const int rc = forward_host_parts(L, x_host, out_host, static_cast<char*>(out_dev), T,
                                       mask_host, b_dev, k_dev, s);

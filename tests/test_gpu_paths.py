@@ -146,11 +146,14 @@ def test_few_experts_per_token_bundle_later(T, kw, kernels):
     assert_parity(wl, g, rep)
 
 
-@pytest.mark.parametrize("T,masked", [(14335, False), (14336, True), (20011, False)])
-def test_host_forward_in_parts(T, masked):
-    """From 14,336 tokens on, a forward of pinned buffers runs in three parts:
-    outputs, counts, records and the group table as of one pass."""
-    s = small(tokens=T, n_experts=2, d_ff=256, **(dict(seq_len=50, min_len=1) if masked else {}))
+@pytest.mark.parametrize("T,d,masked", [(14335, 256, False), (14336, 256, True),
+                                        (20011, 256, False), (28671, 128, True),
+                                        (28672, 128, False)])
+def test_host_forward_in_parts(T, d, masked):
+    """From 14,336 tokens and 7 MiB on, a forward of pinned buffers runs in three
+    parts: outputs, counts, records and the group table as of one pass."""
+    s = small(tokens=T, d_model=d, n_experts=2, d_ff=256,
+              **(dict(seq_len=50, min_len=1) if masked else {}))
     wl = workloads.make_workload(s)
     g = run_gpu(wl)
     counts, offsets, tok, w = g.layer.groups()
