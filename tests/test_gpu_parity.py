@@ -552,10 +552,11 @@ def test_repeated_forwards_match_streaming_kernels():
 
 
 def test_repeated_forwards_sliced_down_projection():
-    """A ViT-B-shaped layer (d = 768: the weight-stationary down projection
-    runs in three 256-column slices) agrees with the streaming kernels over
-    repeated forwards, and with the oracle on every token."""
-    s = workloads.spec("vit_b", tokens=3000)
+    """A ViT-B-shaped layer with two experts per token (d = 768: from 4,096 tokens
+    on the weight-stationary down projection runs in three 256-column slices,
+    until the rows are bundled from 6,267 on) agrees with the streaming kernels
+    over repeated forwards, and with the oracle on every token."""
+    s = workloads.spec("vit_b", tokens=4500, topk_fixed=2)
     wl = workloads.make_workload(s)
     dev = torch.device("cuda")
 
@@ -567,6 +568,7 @@ def test_repeated_forwards_sliced_down_projection():
     x = wl.x.to(dev)
     ref = layer("streaming").forward(x).float()
     L = layer("auto")
+    assert L.kernels_per_forward() == 4
     for _ in range(5):
         y = L.forward(x).float()
         torch.cuda.synchronize()
