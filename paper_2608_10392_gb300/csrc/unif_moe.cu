@@ -102,57 +102,114 @@ void free_all(unif_moe_layer* L) {
   }
   if (L->copy_in) cudaStreamDestroy(L->copy_in);
   if (L->copy_out) cudaStreamDestroy(L->copy_out);
+  L->wr = L->bias = nullptr;
+  L->wr_bf = nullptr;
+  L->w_up = L->w_down = nullptr;
+  L->ws = unif::Workspace();
+  for (int i = 0; i < 2; ++i) L->ev_in[i] = L->ev_comp[i] = L->ev_out[i] = nullptr;
+  L->copy_in = L->copy_out = nullptr;
 }
 
 size_t elt_size(const unif_moe_layer* L) { return L->dtype == UNIF_MOE_BF16 ? 2 : 4; }
 
-// The bundled down projection's tables and h in its layout (more rows), in
-// place of the h of max_rows rows allocated before. Last of a handle's
-// allocations, and given up where one fails: the layer then keeps its unbundled
-// kernels, so that it needs no more memory than those. The rows' list is the
-// largest table, 8 bytes per group and token slot of a pass; with the larger h
-// the bundles of 12,608 tokens of d = 768, K = B = 16 take 0.2 GB, those of
-// 32,768 tokens of d = 1024, K = 32 0.8 GB (below 17 GB for any layer, by the
-// int32 indexes of bundles_fit).
-int alloc_bundles(unif_moe_layer* L) {
+// All device buffers of a handle, its copy streams and events. With
+// L->bundles they include the bundled down projection's; where they do not fit,
+// a caller frees all and allocates again without, so that bundles never ask for
+// memory that the layer cannot do without. The rows' list is the largest of
+// their tables, 8 bytes per group and token slot of a pass; with the larger h they
+// take 0.2 GB for 12,608 tokens of d = 768, K = B = 16, 0.8 GB for 32,768 tokens
+// of d = 1024, K = 32 (below 17 GB for any layer, by the int32 indexes that
+// bundles_fit asks for).
+int alloc_buffers(unif_moe_layer* L) {
+  const bool bf16 = L->dtype == UNIF_MOE_BF16;
+  const size_t es = elt_size(L);
+  const size_t T = (size_t)L->max_tokens, K = (size_t)L->K, E = K + 1;
+  const size_t d = (size_t)L->d, H = (size_t)L->H;
   unif::Workspace& w = L->ws;
-  const size_t G2 = (size_t)unif::bundle_groups(L), nt = (size_t)unif::bundle_max_tiles(L);
-  const size_t h_row = elt_size(L) * (size_t)L->M;
-  bool ok = dalloc(&w.bd_fill, G2) == UNIF_MOE_OK &&
-            dalloc(&w.bd_rows, G2 * L->region_rows) == UNIF_MOE_OK &&
-            dalloc(&w.bd_dst, (size_t)L->pass_tokens * (L->K + 1) * (L->B / unif::kBundle)) ==
-                UNIF_MOE_OK &&
-            dalloc(&w.bd_n_tiles, 1) == UNIF_MOE_OK && dalloc(&w.bd_tile_group, nt) == UNIF_MOE_OK &&
-            dalloc(&w.bd_tile_row0, nt) == UNIF_MOE_OK &&
-            dalloc(&w.bd_tile_rows, nt) == UNIF_MOE_OK && dalloc(&w.bd_tile_unit, nt) == UNIF_MOE_OK;
-  char* h = nullptr;
-  if (ok) {
-    cudaFree(w.hbuf);
-    w.hbuf = nullptr;
-    L->h_rows = std::max(L->max_rows, unif::bundle_h_rows(L));
-    ok = dalloc(&h, h_row * (size_t)L->h_rows) == UNIF_MOE_OK;
-    w.hbuf = h;
-  }
-  if (ok) return UNIF_MOE_OK;
-  void** tables[] = {reinterpret_cast<void**>(&w.bd_fill),
-                     reinterpret_cast<void**>(&w.bd_rows),
-                     reinterpret_cast<void**>(&w.bd_dst),
-                     reinterpret_cast<void**>(&w.bd_n_tiles),
-                     reinterpret_cast<void**>(&w.bd_tile_group),
-                     reinterpret_cast<void**>(&w.bd_tile_row0),
-                     reinterpret_cast<void**>(&w.bd_tile_rows),
-                     reinterpret_cast<void**>(&w.bd_tile_unit)};
-  for (void** q : tables) {
-    if (*q) cudaFree(*q);
-    *q = nullptr;
-  }
-  L->bundles = false;
+  int rc = UNIF_MOE_OK;
+#define ALLOC(ptr, n)                          \
+  if (rc == UNIF_MOE_OK) rc = dalloc(&(ptr), (n));
+  ALLOC(L->wr, (size_t)L->router_cols_pad * d);
+  if (bf16) ALLOC(L->wr_bf, (size_t)L->router_cols_pad * d);
+  ALLOC(L->bias, E);
+  void* wup = nullptr;
+  void* wdn = nullptr;
+  if (rc == UNIF_MOE_OK) rc = dalloc(reinterpret_cast<char**>(&wup), es * E * H * d);
+  if (rc == UNIF_MOE_OK) rc = dalloc(reinterpret_cast<char**>(&wdn), es * E * H * d);
+  L->w_up = wup; L->w_down = wdn;
+  ALLOC(w.alpha, T); ALLOC(w.b, T); ALLOC(w.k, T); ALLOC(w.shr_mask, T); ALLOC(w.exp_mask, T);
+  ALLOC(w.s, T * K);
+  ALLOC(w.chunk_cnt, (size_t)L->G * L->max_chunks);
+  ALLOC(w.grp_cnt, (size_t)L->G); ALLOC(w.grp_off, (size_t)L->G + 1); ALLOC(w.n_tiles, 1);
+  ALLOC(w.tile_group, (size_t)L->max_tiles); ALLOC(w.tile_row0, (size_t)L->max_tiles);
+  ALLOC(w.tile_rows, (size_t)L->max_tiles);
+  const size_t row_cap = L->fused_group ? (size_t)L->G * L->region_rows : (size_t)L->max_rows;
+  ALLOC(w.row_tok, row_cap); ALLOC(w.row_w, row_cap);
+  if (L->fused_group) ALLOC(w.grp_fill, (size_t)L->G);
   L->h_rows = L->max_rows;
-  cudaGetLastError();  // the failed allocation must not surface at a later launch
-  unif::g_err[0] = 0;
-  if (w.hbuf) return UNIF_MOE_OK;
-  const int rc = dalloc(&h, h_row * (size_t)L->h_rows);
-  w.hbuf = h;
+  if (L->bundles) {  // their tables, and h in their layout (more rows)
+    const size_t G2 = (size_t)unif::bundle_groups(L), nt = (size_t)unif::bundle_max_tiles(L);
+    L->h_rows = std::max(L->h_rows, unif::bundle_h_rows(L));
+    ALLOC(w.bd_fill, G2);
+    ALLOC(w.bd_rows, G2 * L->region_rows);
+    ALLOC(w.bd_dst, (size_t)L->pass_tokens * E * (L->B / unif::kBundle));
+    ALLOC(w.bd_n_tiles, 1); ALLOC(w.bd_tile_group, nt); ALLOC(w.bd_tile_row0, nt);
+    ALLOC(w.bd_tile_rows, nt); ALLOC(w.bd_tile_unit, nt);
+  }
+  void* hb = nullptr;
+  if (rc == UNIF_MOE_OK) rc = dalloc(reinterpret_cast<char**>(&hb), es * (size_t)L->h_rows * L->M);
+  w.hbuf = hb;
+  ALLOC(w.y32, (size_t)L->pass_tokens * d);
+  if (L->ffn_fused) ALLOC(w.y32_b, (size_t)L->pass_tokens * d);
+  if (L->ffn_fused) {  // the expert weights as the expert-tile FFN's operand slabs
+    if (rc == UNIF_MOE_OK) rc = dalloc(reinterpret_cast<char**>(&w.wk_slabs), es * E * H * d);
+    if (rc == UNIF_MOE_OK) rc = dalloc(reinterpret_cast<char**>(&w.wv_slabs), es * E * H * d);
+  }
+  ALLOC(w.status, 1);
+  // optional features: every buffer a later call needs, so that no later
+  // call allocates
+  if (L->features & UNIF_MOE_FEATURE_NORM_FIRST) {
+    if (rc == UNIF_MOE_OK) rc = dalloc(reinterpret_cast<char**>(&w.xn), es * T * d);
+  }
+  if (L->features & UNIF_MOE_FEATURE_HOST_IO) {
+    for (int i = 0; i < 2; ++i) {
+      if (rc == UNIF_MOE_OK) rc = dalloc(reinterpret_cast<char**>(&w.x_stage[i]), es * T * d);
+      if (rc == UNIF_MOE_OK) rc = dalloc(reinterpret_cast<char**>(&w.out_stage[i]), es * T * d);
+      ALLOC(w.mask_stage[i], T); ALLOC(w.b_stage[i], T); ALLOC(w.k_stage[i], T);
+    }
+    // the pipelined forward's copy streams and slot events
+    bool ok = rc == UNIF_MOE_OK &&
+              cudaStreamCreateWithFlags(&L->copy_in, cudaStreamNonBlocking) == cudaSuccess &&
+              cudaStreamCreateWithFlags(&L->copy_out, cudaStreamNonBlocking) == cudaSuccess;
+    for (int i = 0; i < 2 && ok; ++i)
+      ok = cudaEventCreateWithFlags(&L->ev_in[i], cudaEventDisableTiming) == cudaSuccess &&
+           cudaEventCreateWithFlags(&L->ev_comp[i], cudaEventDisableTiming) == cudaSuccess &&
+           cudaEventCreateWithFlags(&L->ev_out[i], cudaEventDisableTiming) == cudaSuccess;
+    if (rc == UNIF_MOE_OK && !ok) {
+      set_error("creating the host-buffer copy streams or events failed");
+      rc = UNIF_MOE_ERR_CUDA;
+    }
+  }
+  if (L->features & UNIF_MOE_FEATURE_BACKWARD) {
+    if (rc == UNIF_MOE_OK && (!bf16 || !L->fused_group || d % 128 != 0)) {
+      set_error("the backward pass needs a bf16 layer with d %% 128 == 0 (d=%d)", L->d);
+      rc = UNIF_MOE_ERR_SHAPE;
+    }
+    const size_t wbytes = es * E * H * d;
+    if (rc == UNIF_MOE_OK) rc = dalloc(reinterpret_cast<char**>(&w.w_upT), wbytes);
+    if (rc == UNIF_MOE_OK) rc = dalloc(reinterpret_cast<char**>(&w.w_downT), wbytes);
+    if (rc == UNIF_MOE_OK) rc = dalloc(reinterpret_cast<char**>(&w.da), es * (size_t)L->max_rows * L->M);
+    if (rc == UNIF_MOE_OK) rc = dalloc(reinterpret_cast<char**>(&w.hw), es * (size_t)L->max_rows * L->M);
+    ALLOC(w.dwt, T * E); ALLOC(w.dz, T * E);
+    ALLOC(w.wrT, E * d); ALLOC(w.gram, E * E);
+  }
+  if (L->features & UNIF_MOE_FEATURE_DIAGNOSTICS) {
+    const size_t H32 = ((size_t)H + 31) / 32;
+    ALLOC(w.diag_sets, K * K * H32); ALLOC(w.diag_counts, K * K);
+    ALLOC(w.diag_pair, 2 * T); ALLOC(w.diag_wts, 2 * T); ALLOC(w.diag_q, T * K);
+    ALLOC(w.diag_E, T * K * d); ALLOC(w.diag_ES, T * K * d);
+  }
+#undef ALLOC
   return rc;
 }
 
@@ -280,26 +337,6 @@ int unif_moe_create_ex(unif_moe_t* out, int d_model, int d_ff, int n_experts, in
     delete L;
     return UNIF_MOE_ERR_CUDA;
   }
-  const size_t es = elt_size(L);
-  const size_t T = (size_t)max_tokens, K = (size_t)n_experts, E = K + 1;
-  unif::Workspace& w = L->ws;
-  int rc = UNIF_MOE_OK;
-#define ALLOC(ptr, n)                          \
-  if (rc == UNIF_MOE_OK) rc = dalloc(&(ptr), (n));
-  ALLOC(L->wr, (size_t)L->router_cols_pad * d_model);
-  if (dtype == UNIF_MOE_BF16) ALLOC(L->wr_bf, (size_t)L->router_cols_pad * d_model);
-  ALLOC(L->bias, E);
-  void* wup = nullptr;
-  void* wdn = nullptr;
-  if (rc == UNIF_MOE_OK) rc = dalloc(reinterpret_cast<char**>(&wup), es * E * d_ff * d_model);
-  if (rc == UNIF_MOE_OK) rc = dalloc(reinterpret_cast<char**>(&wdn), es * E * d_ff * d_model);
-  L->w_up = wup; L->w_down = wdn;
-  ALLOC(w.alpha, T); ALLOC(w.b, T); ALLOC(w.k, T); ALLOC(w.shr_mask, T); ALLOC(w.exp_mask, T);
-  ALLOC(w.s, T * K);
-  ALLOC(w.chunk_cnt, (size_t)L->G * L->max_chunks);
-  ALLOC(w.grp_cnt, (size_t)L->G); ALLOC(w.grp_off, (size_t)L->G + 1); ALLOC(w.n_tiles, 1);
-  ALLOC(w.tile_group, (size_t)L->max_tiles); ALLOC(w.tile_row0, (size_t)L->max_tiles);
-  ALLOC(w.tile_rows, (size_t)L->max_tiles);
   // bf16 layers group inside the router: each group owns a region of
   // max_tokens rows (rounded up to whole tiles) in the row arrays
   L->fused_group = dtype == UNIF_MOE_BF16 && L->router_cols_pad <= 160 &&
@@ -311,70 +348,20 @@ int unif_moe_create_ex(unif_moe_t* out, int d_model, int d_ff, int n_experts, in
                  (o.gemm_kernels == UNIF_MOE_GEMM_EXPERT_TILE ||
                   o.gemm_kernels == UNIF_MOE_GEMM_AUTO) &&
                  !(o.features & UNIF_MOE_FEATURE_BACKWARD) && unif::ffn_fused_fits(d_model, d_ff, M);
-  const size_t row_cap = L->fused_group ? (size_t)L->G * L->region_rows : (size_t)L->max_rows;
-  ALLOC(w.row_tok, row_cap); ALLOC(w.row_w, row_cap);
-  if (L->fused_group) ALLOC(w.grp_fill, (size_t)L->G);
-  L->h_rows = L->max_rows;
-  void* hb = nullptr;
-  if (rc == UNIF_MOE_OK) rc = dalloc(reinterpret_cast<char**>(&hb), es * (size_t)L->h_rows * M);
-  w.hbuf = hb;
-  ALLOC(w.y32, (size_t)L->pass_tokens * d_model);
-  if (L->ffn_fused) ALLOC(w.y32_b, (size_t)L->pass_tokens * d_model);
-  if (L->ffn_fused) {  // the expert weights as the expert-tile FFN's operand slabs
-    if (rc == UNIF_MOE_OK) rc = dalloc(reinterpret_cast<char**>(&w.wk_slabs), es * E * d_ff * d_model);
-    if (rc == UNIF_MOE_OK) rc = dalloc(reinterpret_cast<char**>(&w.wv_slabs), es * E * d_ff * d_model);
-  }
-  ALLOC(w.status, 1);
-  // optional features: every buffer a later call needs, so that no later
-  // call allocates
-  if (o.features & UNIF_MOE_FEATURE_NORM_FIRST) {
-    if (rc == UNIF_MOE_OK) rc = dalloc(reinterpret_cast<char**>(&w.xn), es * T * d_model);
-  }
-  if (o.features & UNIF_MOE_FEATURE_HOST_IO) {
-    for (int i = 0; i < 2; ++i) {
-      if (rc == UNIF_MOE_OK) rc = dalloc(reinterpret_cast<char**>(&w.x_stage[i]), es * T * d_model);
-      if (rc == UNIF_MOE_OK) rc = dalloc(reinterpret_cast<char**>(&w.out_stage[i]), es * T * d_model);
-      ALLOC(w.mask_stage[i], T); ALLOC(w.b_stage[i], T); ALLOC(w.k_stage[i], T);
-    }
-    // the pipelined forward's copy streams and slot events
-    bool ok = rc == UNIF_MOE_OK &&
-              cudaStreamCreateWithFlags(&L->copy_in, cudaStreamNonBlocking) == cudaSuccess &&
-              cudaStreamCreateWithFlags(&L->copy_out, cudaStreamNonBlocking) == cudaSuccess;
-    for (int i = 0; i < 2 && ok; ++i)
-      ok = cudaEventCreateWithFlags(&L->ev_in[i], cudaEventDisableTiming) == cudaSuccess &&
-           cudaEventCreateWithFlags(&L->ev_comp[i], cudaEventDisableTiming) == cudaSuccess &&
-           cudaEventCreateWithFlags(&L->ev_out[i], cudaEventDisableTiming) == cudaSuccess;
-    if (rc == UNIF_MOE_OK && !ok) {
-      set_error("creating the host-buffer copy streams or events failed");
-      rc = UNIF_MOE_ERR_CUDA;
-    }
-  }
-  if (o.features & UNIF_MOE_FEATURE_BACKWARD) {
-    if (rc == UNIF_MOE_OK && (dtype != UNIF_MOE_BF16 || !L->fused_group || d_model % 128 != 0)) {
-      set_error("the backward pass needs a bf16 layer with d %% 128 == 0 (d=%d)", d_model);
-      rc = UNIF_MOE_ERR_SHAPE;
-    }
-    const size_t wbytes = es * E * d_ff * d_model;
-    if (rc == UNIF_MOE_OK) rc = dalloc(reinterpret_cast<char**>(&w.w_upT), wbytes);
-    if (rc == UNIF_MOE_OK) rc = dalloc(reinterpret_cast<char**>(&w.w_downT), wbytes);
-    if (rc == UNIF_MOE_OK) rc = dalloc(reinterpret_cast<char**>(&w.da), es * (size_t)L->max_rows * M);
-    if (rc == UNIF_MOE_OK) rc = dalloc(reinterpret_cast<char**>(&w.hw), es * (size_t)L->max_rows * M);
-    ALLOC(w.dwt, T * E); ALLOC(w.dz, T * E);
-    ALLOC(w.wrT, E * d_model); ALLOC(w.gram, E * E);
-  }
-  if (o.features & UNIF_MOE_FEATURE_DIAGNOSTICS) {
-    const size_t H32 = ((size_t)d_ff + 31) / 32;
-    ALLOC(w.diag_sets, K * K * H32); ALLOC(w.diag_counts, K * K);
-    ALLOC(w.diag_pair, 2 * T); ALLOC(w.diag_wts, 2 * T); ALLOC(w.diag_q, T * K);
-    ALLOC(w.diag_E, T * K * d_model); ALLOC(w.diag_ES, T * K * d_model);
-  }
-#undef ALLOC
   // wide layers' passes of many tokens: the down projection's rows bundled
-  // over four blocks, where memory for it is left
+  // over four blocks, where there is memory for it
   L->bundles = true;
-  L->bundles = rc == UNIF_MOE_OK && dtype == UNIF_MOE_BF16 && unif::bundles_fit(L) &&
+  L->bundles = dtype == UNIF_MOE_BF16 && unif::bundles_fit(L) &&
                unif::bundles_apply(L, L->pass_tokens);
-  if (L->bundles) rc = alloc_bundles(L);
+  unif::Workspace& w = L->ws;
+  int rc = alloc_buffers(L);
+  if (rc == UNIF_MOE_ERR_CUDA && L->bundles) {
+    free_all(L);
+    cudaGetLastError();  // the failed allocation must not surface at a later launch
+    L->bundles = false;
+    rc = alloc_buffers(L);
+    if (rc == UNIF_MOE_OK) unif::g_err[0] = 0;
+  }
   if (rc == UNIF_MOE_OK && (cudaMemset(w.status, 0, sizeof(int)) != cudaSuccess ||
                             cudaMemset(w.y32, 0, sizeof(float) * L->pass_tokens * d_model) !=
                                 cudaSuccess ||
@@ -384,14 +371,15 @@ int unif_moe_create_ex(unif_moe_t* out, int d_model, int d_ff, int n_experts, in
                             (L->bundles &&
                              (cudaMemset(w.bd_fill, 0, sizeof(int32_t) * unif::bundle_groups(L)) !=
                                   cudaSuccess ||
-                              cudaMemset(w.bd_dst, 0, sizeof(int32_t) * L->pass_tokens * E *
+                              cudaMemset(w.bd_dst, 0, sizeof(int32_t) * L->pass_tokens * (L->K + 1) *
                                                           (n_blocks / unif::kBundle)) !=
                                   cudaSuccess)) ||
                             (L->fused_group &&
                              (cudaMemset(w.grp_fill, 0, sizeof(int32_t) * L->G) != cudaSuccess ||
                               // rows hold token indices from the start, also any row a
                               // forward that gave up a wait left unwritten
-                              cudaMemset(w.row_tok, 0, sizeof(int32_t) * row_cap) != cudaSuccess)))) {
+                              cudaMemset(w.row_tok, 0, sizeof(int32_t) * L->G * L->region_rows) !=
+                                  cudaSuccess)))) {
     set_error("cudaMemset failed");
     rc = UNIF_MOE_ERR_CUDA;
   }
