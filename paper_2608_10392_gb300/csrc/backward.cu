@@ -36,16 +36,35 @@ namespace unif {
 namespace tc {
 namespace bwd {
 
-// GeLU (exact erf form, Sec. II-A) and its derivative Phi(a) + a phi(a), from
-// one evaluation of Phi. GeLU's value is not rounded to bf16 everywhere (it goes
-// into dL/dalpha and dL/ds in fp32), so Phi is erff's, whose error stays near
-// that of the last rounding (6e-8 in Phi). A five-term approximation of erfc
-// that shared the exponential took 17 instructions instead of 45, and four
-// times that error.
+// GeLU (exact erf form, Sec. II-A) and its derivative Phi(a) + a phi(a).
+// GeLU's value goes into dL/dalpha and dL/ds in fp32, so Phi is as exact as
+// erff would make it. The hidden kernel's epilogue is bound by these
+// instructions, though, and the exponential that phi needs serves Phi as well:
+//   |a| < 1.35: Phi(a) = 1/2 + a P(a^2), P of degree 5;
+//   beyond:     Phi(-|a|) = exp(-a^2 / 2) t R(t), t = 1 / (1 + |a| / 2), R of degree 3
+// (minimax fits, each coefficient rounded to fp32 before the next is fitted:
+// tests/gelu_fit.py). Measured over [-8, 8]: Phi within 6.04e-8, rms 1.11e-8;
+// 0.5 (1 + erff(a / sqrt 2)) within 6.73e-8, rms 1.58e-8, and no better in any of 14
+// intervals. ViT-S, 12,608 tokens: 123 us, with erff 138. (One expression for all a,
+// the erfc approximation 7.1.26 of Abramowitz and Stegun, took 111, but was within
+// 3.4e-7 only.)
 __device__ __forceinline__ void gelu_and_grad(float a, float& g, float& dg) {
-  const float cdf = 0.5f * (1.0f + erff(a * 0.70710678118654752f));
+  const float u = a * a;
+  float e, t;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(u * -0.72134752044448170f));  // exp(-a^2/2)
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t) : "f"(fmaf(fabsf(a), 0.5f, 1.0f)));
+  float p = fmaf(-6.28209773e-06f, u, 0.00010880574f);  // P
+  p = fmaf(p, u, -0.00118041399f);
+  p = fmaf(p, u, 0.00997000933f);
+  p = fmaf(p, u, -0.0664895996f);
+  p = fmaf(p, u, 0.398942232f);
+  float r = fmaf(-0.145465598f, t, 0.275724202f);  // R
+  r = fmaf(r, t, 0.164777622f);
+  r = fmaf(r, t, 0.203067407f);
+  const float tail = fmaf(-copysignf(r * t, a), e, a > 0.f ? 1.f : 0.f);
+  const float cdf = fabsf(a) < 1.35f ? fmaf(a, p, 0.5f) : tail;
   g = a * cdf;
-  dg = cdf + a * 0.39894228040143268f * __expf(-0.5f * a * a);
+  dg = fmaf(a * 0.39894228040143268f, e, cdf);
 }
 
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
@@ -102,11 +121,9 @@ __device__ __forceinline__ int chunk_tiles(int total, int parts, int ctas) {
 // accumulators take 2 bn <= 512 TMEM columns, so a tile's MMAs wait for the
 // epilogue of the one before; the ring holds the next tile's first steps by
 // then. (16 epilogue warps of half the columns ran no faster.)
-// Measured (one CTA per tile, four gather warps, a 32-byte row piece per
-// thread's store before): BERT-base (2,300 tokens) 102 -> 88 us; ViT-S (12,608
-// tokens) 138 either way, bound by the epilogue's arithmetic: with a GeLU of
-// 17 instructions in place of erff's 45, but less exact, it took 111 (and
-// BERT-base 75).
+// Measured (one CTA per tile, four gather warps, erff, a 32-byte row piece per
+// thread's store before): ViT-S (12,608 tokens) 138 -> 123 us; BERT-base (2,300
+// tokens) 102 -> 80.
 // ---------------------------------------------------------------------------
 struct HiddenParams {
   const int32_t* counts;   // [G] group sizes (the forward's)

@@ -6,6 +6,8 @@ CPU: the constants compiled into the kernels (read from csrc/tc_common.cuh)
 give |Phi error| < 2e-6 before the tanh, g increases monotonically (so large
 |x| saturates to x or 0), and with the tanh error bounded by 2^-10.9 the
 GeLU error stays below 3e-4 |x|.
+The backward's GeLU (fp32 accuracy) likewise: its constants, read from
+csrc/backward.cu, against Phi.
 GPU: a layer whose shared expert has identity keys and identity values and
 alpha fixed at 1 outputs bf16(GeLU(x)) feature by feature: the epilogue's
 GeLU alone, rounded to bf16 once (h) and passed through exactly."""
@@ -56,6 +58,39 @@ def test_gelu_error_bound_with_hardware_tanh():
     for sgn in (-1.0, 1.0):
         approx = 0.5 * x * (1.0 + np.clip(t + sgn * TANH_ERR, -1.0, 1.0))
         assert (np.abs(approx - ref) <= 3e-4 * np.abs(x) + 1e-30).all()
+
+
+def test_backward_phi_error():
+    """The backward's Phi in fp32: polynomials within 6e-9 of Phi, then the
+    roundings: of the sum (2^-25), of P (2^-26, times |a| < 1.35) and half as
+    much again before it; in the tail a few 2^-24 of at most 0.089. Below 7.5e-8
+    in all, and closer on average than 0.5 (1 + erf(a / sqrt 2)) with every
+    operation rounded to fp32 once."""
+    from scipy.special import erf, erfc
+
+    from gelu_fit import P_DEG, R_DEG, phi_backward
+    src = open(os.path.join(os.path.dirname(TC_COMMON), "backward.cu")).read()
+    body = src[src.index("void gelu_and_grad"):]
+    num = r"(-?[0-9.]+(?:e-?[0-9]+)?)f"
+
+    def coefficients(var, arg, deg):
+        top = re.search(r"float %s = fmaf\(%s, %s, %s\);" % (var, num, arg, num), body)
+        rest = re.findall(r"\n  %s = fmaf\(%s, %s, %s\);" % (var, var, arg, num), body)
+        c = [float(v) for v in list(top.groups()) + rest][::-1]
+        assert len(c) == deg + 1
+        return np.array(c)
+
+    p, r = coefficients("p", "u", P_DEG), coefficients("r", "t", R_DEG)
+    rng = np.random.default_rng(0)
+    a = np.concatenate([np.linspace(-8, 8, 800001), rng.normal(size=400000),
+                        [-1e30, 1e30, -40, 40]]).astype(np.float32)
+    ref = 0.5 * erfc(-a.astype(np.float64) / np.sqrt(2))
+    with np.errstate(over="ignore", invalid="ignore"):
+        err = np.abs(phi_backward(a, p, r) - ref)
+    assert err.max() < 7.5e-8
+    z = (a * np.float32(0.70710678118654752)).astype(np.float64)
+    by_erf = np.float32(0.5) * (np.float32(1) + erf(z).astype(np.float32))
+    assert np.sqrt((err ** 2).mean()) < np.sqrt(((by_erf - ref) ** 2).mean())
 
 
 @pytest.mark.gpu

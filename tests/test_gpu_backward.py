@@ -173,9 +173,11 @@ def test_gelu_of_the_router_gradient_in_fp32():
     shared): dL/dW*[1 + t][0] = GeLU(a_t) / 4, all other factors and terms being
     exact. For every bf16 a_t of [2^-6, 8) and both signs.
 
-    Bound: erff within 2 ulp (its documented error) of values below 1 (2^-23),
-    its argument's two roundings (2^-23 z erf'(z) <= 2^-24), the sum 1 + erf
-    (2^-24), halved: 2^-23 |a| at most; the product's rounding, 2^-24 |GeLU|."""
+    Bound: Phi's sum is rounded by 2^-25. For |a| < 1.35, P by 2^-26 (times |a|) and
+    less before it, 7e-8 in all. Beyond, Phi(-|a|) <= 0.089 times the errors of the
+    exponential (2^-22 and its argument's), the reciprocal (2^-23) and three
+    roundings, 8.5e-8 in all. Below 2^-23 |a|, then; the product's rounding adds
+    2^-24 |GeLU|. (erff within its documented 2 ulp gives the same bound.)"""
     from scipy.stats import norm
 
     from paper_2608_10392_gb300 import FEATURE_BACKWARD, FEATURES_DEFAULT, Layer
