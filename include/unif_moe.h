@@ -99,9 +99,13 @@ enum {
  *   multiple of 64, a handle without UNIF_MOE_FEATURE_BACKWARD (otherwise
  *   as GROUPED).
  * - GROUPED: rows grouped by (expert, block) pair (Eq. 35's C_B pairs per
- *   token), an up and a down projection kernel with h in device memory;
- *   weight-stationary kernels where a group's weight slice fits in shared
- *   memory, else the streaming ones.
+ *   token), an up and a down projection kernel with h in device memory. Up:
+ *   weight-stationary where a group's weight slice fits in shared memory and
+ *   the pass has at least 4,096 tokens, else on CTA pairs (streaming where the
+ *   pair kernel's tables do not fit). Down: for layers whose up projection is
+ *   never weight-stationary and B % 4 == 0, over rows bundled by four blocks
+ *   where the groups are large enough for the block width; else
+ *   weight-stationary as above, whole or in column slices, or streaming.
  * - STREAMING: as GROUPED, always the streaming kernels.
  * - AUTO: EXPERT_TILE where it applies, else GROUPED. */
 enum {

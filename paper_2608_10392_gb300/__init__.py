@@ -133,7 +133,8 @@ class Layer:
     expert, FFN width H split into B blocks. dtype "bf16" (tensor cores) or
     "f32" (CUDA-core FMA). `features` (FEATURE_* bits) picks the optional
     workspaces allocated at create time; `gemm_kernels` "grouped" ((expert,
-    block) groups, weight-stationary kernels where they fit), "streaming"
+    block) groups; weight-stationary, CTA-pair, bundled or streaming kernels by
+    the layer's shape and the number of tokens), "streaming"
     ((expert, block) groups, streaming kernels), "expert_tile" (rows grouped
     by expert, both projections in one kernel, where it applies) or "auto"
     (expert_tile where it applies, else grouped)."""
