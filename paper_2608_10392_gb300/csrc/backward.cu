@@ -45,7 +45,7 @@ namespace bwd {
 // (minimax fits, each coefficient rounded to fp32 before the next is fitted:
 // tests/gelu_fit.py). Measured over [-8, 8]: Phi within 6.04e-8, rms 1.11e-8;
 // 0.5 (1 + erff(a / sqrt 2)) within 6.73e-8, rms 1.58e-8, and no better in any of 14
-// intervals. ViT-S, 12,608 tokens: 123 us, with erff 138. (One expression for all a,
+// intervals. ViT-S, 12,608 tokens: 118 us, with erff 138. (One expression for all a,
 // the erfc approximation 7.1.26 of Abramowitz and Stegun, took 111, but was within
 // 3.4e-7 only.)
 __device__ __forceinline__ void gelu_and_grad(float a, float& g, float& dg) {
@@ -122,8 +122,8 @@ __device__ __forceinline__ int chunk_tiles(int total, int parts, int ctas) {
 // epilogue of the one before; the ring holds the next tile's first steps by
 // then. (16 epilogue warps of half the columns ran no faster.)
 // Measured (one CTA per tile, four gather warps, erff, a 32-byte row piece per
-// thread's store before): ViT-S (12,608 tokens) 138 -> 123 us; BERT-base (2,300
-// tokens) 102 -> 80.
+// thread's store before): ViT-S (12,608 tokens) 138 -> 118 us; BERT-base (2,300
+// tokens) 102 -> 77.
 // ---------------------------------------------------------------------------
 struct HiddenParams {
   const int32_t* counts;   // [G] group sizes (the forward's)
@@ -424,10 +424,10 @@ bwd_hidden_kernel(const __grid_constant__ CUtensorMap tm_wk, const __grid_consta
         const int col0 = it.ns * p.bn + c_begin;
         float dot0 = 0.f, dot1 = 0.f;
         for (int c = 0; c < cols; c += 32) {
-          uint32_t od[16], oh[16];
 #pragma unroll
-          for (int hh = 0; hh < 2; ++hh) {
+          for (int hh = 0; hh < 2; ++hh) {  // (all 32 columns at once: registers spill)
             float a[16], gv[16];
+            uint32_t od[8], oh[8];
             tmem_ld16(t_row + c + 16 * hh, a);
             tmem_ld16(t_row + kAcc2 + c + 16 * hh, gv);
 #pragma unroll
@@ -440,19 +440,21 @@ bwd_hidden_kernel(const __grid_constant__ CUtensorMap tm_wk, const __grid_consta
               gelu_and_grad(a1, g1, dg1);
               dot0 = fmaf(g0, v0, dot0);
               dot1 = fmaf(g1, v1, dot1);
-              od[8 * hh + i] = pack_bf16(w * v0 * dg0, w * v1 * dg1);
-              oh[8 * hh + i] = pack_bf16(w * g0, w * g1);
+              od[i] = pack_bf16(w * v0 * dg0, w * v1 * dg1);
+              oh[i] = pack_bf16(w * g0, w * g1);
             }
-          }
-          if (lane == 0) bulk_wait_read();  // the last pieces have left the staging
-          __syncwarp();
+            if (hh == 0) {
+              if (lane == 0) bulk_wait_read();  // the last pieces have left the staging
+              __syncwarp();
+            }
 #pragma unroll
-          for (int jj = 0; jj < 4; ++jj) {
-            const uint32_t ch = ((uint32_t)jj ^ sx) << 4;
-            *reinterpret_cast<uint4*>(srow + ch) =
-                make_uint4(od[4 * jj], od[4 * jj + 1], od[4 * jj + 2], od[4 * jj + 3]);
-            *reinterpret_cast<uint4*>(srow + kHPiece + ch) =
-                make_uint4(oh[4 * jj], oh[4 * jj + 1], oh[4 * jj + 2], oh[4 * jj + 3]);
+            for (int jj = 0; jj < 2; ++jj) {
+              const uint32_t ch = ((uint32_t)(2 * hh + jj) ^ sx) << 4;
+              *reinterpret_cast<uint4*>(srow + ch) =
+                  make_uint4(od[4 * jj], od[4 * jj + 1], od[4 * jj + 2], od[4 * jj + 3]);
+              *reinterpret_cast<uint4*>(srow + kHPiece + ch) =
+                  make_uint4(oh[4 * jj], oh[4 * jj + 1], oh[4 * jj + 2], oh[4 * jj + 3]);
+            }
           }
           fence_proxy_async();
           __syncwarp();
